@@ -227,6 +227,7 @@ void fill_pr(PR<R>& o, const Params& P) {
   o.eos_a = (R)P.eos_a;
   o.eta_c0 = (R)P.eta.c0; o.eta_c1 = (R)P.eta.c1; o.eta_inv_c2 = (R)(1.0 / P.eta.c2); o.eta_ln_c0 = (R)P.eta.ln_c0;
   o.eta_inv_c1 = (R)(1.0 / P.eta.c1);
+  o.eta_inv_5c0 = (R)(1.0 / (5.0 * P.eta.c0));
   o.zeta_c0 = (R)P.zeta.c0; o.zeta_c1 = (R)P.zeta.c1; o.zeta_inv_c2 = (R)(1.0 / P.zeta.c2);
   o.zeta_ln_c0 = (R)P.zeta.ln_c0; o.zeta_inv_c1 = (R)(1.0 / P.zeta.c1);
 }

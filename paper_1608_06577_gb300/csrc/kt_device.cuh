@@ -93,7 +93,7 @@ struct PR {
   R tpp;               // tau_pipi/tau_pi
   R rho_max, xi0_rho_max;
   R eos_a;
-  R eta_c0, eta_c1, eta_inv_c2, eta_ln_c0, eta_inv_c1;
+  R eta_c0, eta_c1, eta_inv_c2, eta_ln_c0, eta_inv_c1, eta_inv_5c0;  // eta_inv_5c0 = 1/(5 c0)
   R zeta_c0, zeta_c1, zeta_inv_c2, zeta_ln_c0, zeta_inv_c1;
 };
 
@@ -258,6 +258,17 @@ __device__ __forceinline__ float nmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double nmax(double a, double b) {
   return (__double_as_longlong(a) < __double_as_longlong(b)) ? b : a;
 }
+
+// min(a, b) of non-negative a, b (FP64: compared as integers; a NaN loses, as in fmin)
+__device__ __forceinline__ float nmin(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ double nmin(double a, double b) {
+  return (__double_as_longlong(a) < __double_as_longlong(b)) ? a : b;
+}
+
+// a b rounded to nearest, never contracted with a following addition: a product that several sums
+// read gives the same bits in every kernel that inlines the expression
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 
 // a / b for b > 0 (face velocities: b is an extrapolated u^tau >= 1).  FP32: the fast hardware
 // division.  FP64, for b within [2^-125, 2^125): Newton-Raphson for 1/b from a single-precision

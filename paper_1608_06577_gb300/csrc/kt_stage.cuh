@@ -197,7 +197,7 @@ __device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, co
   F.wRp = (aR - vRp) * hinv;
 
 #pragma unroll
-  for (int m = 0; m < 4; ++m) du[D + 1][m] = (up1[m] - um1[m]) * hinv;
+  for (int m = 0; m < 4; ++m) du[D + 1][m] = rmul(up1[m] - um1[m], hinv);
   const R vpl = vdiv(up1[D + 1], up1[0]), vmi = vdiv(um1[D + 1], um1[0]);
   dv += (vpl - vmi) * hinv;
   F.vpl_h = vpl * hinv;
@@ -698,7 +698,7 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
   // ---- b) sources at the cell
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    du[0][m] = (uc[m] - ld<R>(io.u_prev + m * fs, c)) * pr<R>(P).inv_dtau;  // backward difference
+    du[0][m] = rmul(uc[m] - ld<R>(io.u_prev + m * fs, c), pr<R>(P).inv_dtau);  // backward difference
   }
   const R* q = io.qr_in;
   R pi[4][4];
@@ -725,48 +725,65 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
   }
 
   if (P.shear_on || P.bulk_on) {
-    const R glo[4] = {R(1), R(-1), R(-1), -gnn};
     const R gup[4] = {R(1), R(-1), R(-1), -inv_gnn};
-    // u^mu_{;alpha}, alpha = 0..3 (only Gamma^eta_{tau eta} = 1/tau, Gamma^tau_{eta eta} = tau)
-    R cov[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      cov[0][a] = du[a][0] + ((a == 3) ? tg * uc[3] : R(-0.0));
-      cov[1][a] = du[a][1];
-      cov[2][a] = du[a][2];
-      cov[3][a] = du[a][3] + ((a == 0) ? it * uc[3] : ((a == 3) ? it * uc[0] : R(-0.0)));
-    }
-    const R theta = cov[0][0] + cov[1][1] + cov[2][2] + cov[3][3];
-    const R theta3 = theta * R(1.0 / 3.0);
-    R Dup[4], Dlo[4];
+    // u^m_{;a} = d_a u^m + Gamma^m_{a b} u^b in place of du[a][m] (only Gamma^eta_{tau eta} = 1/tau and
+    // Gamma^tau_{eta eta} = tau)
+    du[3][0] = fma(tg, uc[3], du[3][0]);
+    du[0][3] = fma(it, uc[3], du[0][3]);
+    du[3][3] = fma(it, uc[0], du[3][3]);
+    const R theta = du[0][0] + du[1][1] + du[2][2] + du[3][3];
+    const R th3 = rmul(theta, R(1.0 / 3.0));
+    R D[4], hD[4], th3u[4];  // D u^m, half of it, theta u^m / 3
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      Dup[m] = uc[0] * cov[m][0] + uc[1] * cov[m][1] + uc[2] * cov[m][2] + uc[3] * cov[m][3];
-      Dlo[m] = glo[m] * Dup[m];
+      D[m] = fma(uc[0], du[0][m], fma(uc[1], du[1][m], fma(uc[2], du[2][m], uc[3] * du[3][m])));
+      hD[m] = R(0.5) * D[m];
+      th3u[m] = th3 * uc[m];
     }
-    // nabla^a u^m = Delta^{a b} u^m_{;b} = g^{aa} u^m_{;a} - u^a D u^m
-    R nab[4][4];
+    // The relaxation terms of pi^{ab} are contractions of pi with matrices built from u^m_{;a}:
+    //   I_1 = pi^{al} D u_l u^b + (a <-> b),  I_3 = pi^a_l omega^{bl} + (a <-> b),
+    //   I_4 = pi^a_l sigma^{bl} / 2 + (a <-> b) - Delta^{ab} pi:sigma / 3,
+    //   G_pi^{ab} = K^a_l pi^{lb} + (a <-> b), K^0_3 = tau u^eta, K^3_0 = u^eta/tau, K^3_3 = u^tau/tau
+    // so -(I_1 - I_3 + (tau_pipi/tau_pi) I_4) - G_pi is ONE product with Y^{bl} = -u^b D u^l +
+    // omega^{bl} - (tau_pipi/(2 tau_pi)) sigma^{bl}, and with G^{bl} = g^{bb} u^l_{;b} the u D terms of
+    // omega (= (G^{lb} - G^{bl} - u^l D^b + u^b D^l)/2) combine to
+    //   Y^{bl} = (G^{lb} - G^{bl})/2 - (u^b D^l + u^l D^b)/2 - (tau_pipi/(2 tau_pi)) sigma^{bl}.
+    // Terms proportional to pi^{ab} itself go on the diagonal of the matrix.  One 4x4 product in place
+    // of three (I_1, I_3, I_4), without nabla^a u^m and omega as arrays.  (Products that several sums
+    // read are formed by rmul, so that no kernel contracts them into a different multiply-add.)
+    // FP64 is bound by its pipe (one warp instruction per 19 cycles and SM), so every product saved
+    // counts: three 128^3 steps with set and get 44.4 -> 39.2 ms; FP32, bound by issue: six learned
+    // 128^3 steps 7.31 -> 7.18 ms, FP32 pi storage at 96x96x64 2.64 -> 2.52 ms.
+    R G[4][4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int l = 0; l < 4; ++l) {
+      G[0][l] = du[0][l];
+      G[1][l] = -du[1][l];
+      G[2][l] = -du[2][l];
+      G[3][l] = rmul(gup[3], du[3][l]);
+    }
+    const R hk = R(0.5) * pr<R>(P).tpp;
+    R sig[4][4], Y[4][4];  // sigma^{ab} (a <= b), Y^{bl}
 #pragma unroll
-      for (int m = 0; m < 4; ++m) nab[a][m] = gup[a] * cov[m][a] - uc[a] * Dup[m];
-    R sig[4][4], om[4][4];  // symmetric and antisymmetric: each pair is computed once
+    for (int a = 0; a < 4; ++a) {
+      const R uD = rmul(uc[a], D[a]);
+      const R sd = fma(th3u[a], uc[a], G[a][a] - uD);
+      sig[a][a] = (a == 0) ? sd - th3 : ((a == 3) ? fma(-gup[3], th3, sd) : sd + th3);
+      Y[a][a] = fma(-hk, sig[a][a], -uD);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = a; b < 4; ++b) {
-        R Dab = ((a == b) ? gup[a] : R(-0.0)) - uc[a] * uc[b];
-        sig[a][b] = R(0.5) * (nab[a][b] + nab[b][a]) - theta3 * Dab;
-        sig[b][a] = sig[a][b];
-        om[a][b] = (a == b) ? R(0) : R(0.5) * (nab[b][a] - nab[a][b]);  // App. A convention
-        om[b][a] = -om[a][b];
+      for (int b = a + 1; b < 4; ++b) {
+        const R hW = fma(uc[a], hD[b], uc[b] * hD[a]);
+        sig[a][b] = fma(th3u[a], uc[b], fma(R(0.5), G[a][b] + G[b][a], -hW));
+        const R s = fma(-hk, sig[a][b], -hW), A = G[b][a] - G[a][b];
+        Y[a][b] = fma(R(0.5), A, s);
+        Y[b][a] = fma(R(-0.5), A, s);
       }
-    R ps = R(-0.0);  // pi^{mu nu} sigma_{mu nu}
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) ps += pi[a][b] * sig[a][b] * glo[a] * glo[b];
-    const R ps3 = ps * R(1.0 / 3.0);
+    }
+    // pi^{mu nu} sigma_{mu nu}, by powers of g_{eta eta} = -gnn
+    const R psd = fma(pi[0][0], sig[0][0], fma(pi[1][1], sig[1][1], pi[2][2] * sig[2][2]));
+    const R pso = fma(pi[1][2], sig[1][2], -fma(pi[0][1], sig[0][1], pi[0][2] * sig[0][2]));
+    const R psn = fma(pi[1][3], sig[1][3], fma(pi[2][3], sig[2][3], -(pi[0][3] * sig[0][3])));
+    const R ps = fma(gnn, fma(gnn, pi[3][3] * sig[3][3], R(2) * psn), fma(R(2), pso, psd));
 
     // transport coefficients (Sec. 2.2) from T(e), ln(1/3 - c_s^2)(e)
     R T, lnd;
@@ -774,67 +791,85 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
     const R iu0 = sdiv(R(1), uc[0]);
 
     if (P.shear_on) {
-      R eta_tp = (ec + P0c) * R(0.2);
-      R es = eta_over_s<R>(P, T);
-      R rate_pi = (es > R(0)) ? sdiv(T, R(5) * es) : R(INFINITY);
-      rate_pi = fmin(rate_pi, pr<R>(P).rate_max);
-      const R tpp = pr<R>(P).tpp;
-      R xs = R(-0.0);  // sigma.sigma (diagnostics)
-      R av[4];  // pi^{mu lambda} D u_lambda
+      const R eta_tp = (ec + P0c) * R(0.2);
+      const R es = eta_over_s<R>(P, T);
+      R rate_pi = (es > R(0)) ? ((P.eta.kind == 0) ? T * pr<R>(P).eta_inv_5c0 : sdiv(T, R(5) * es)) : R(INFINITY);
+      rate_pi = nmin(rate_pi, pr<R>(P).rate_max);
+      const R tp3 = pr<R>(P).tpp * ps * R(1.0 / 3.0);
+      const R csig = fma(R(1.2), Pic, R(2) * eta_tp);
+      if constexpr (DIAG) {  // sums over the full tensor: off-diagonal pairs count twice
+        const R glo[4] = {R(1), R(-1), R(-1), -gnn};
+        R xs = R(0);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) av[m] = pi[m][0] * Dlo[0] + pi[m][1] * Dlo[1] + pi[m][2] * Dlo[2] + pi[m][3] * Dlo[3];
-      // B^{mu nu} = pi^{mu l} g_ll omega^{nu l};  C^{mu nu} = pi^{mu l} g_ll sigma^{nu l}
-      R B[4][4], Cm[4][4];
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+          for (int b = a; b < 4; ++b) {
+            R c = R(0);  // pi^a_l (omega^{bl} - (tau_pipi/(2 tau_pi)) sigma^{bl}) + (a <-> b)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          R sb = R(-0.0), sc = R(-0.0);
-#pragma unroll
-          for (int l = 0; l < 4; ++l) {
-            if (l != b) sb += pi[a][l] * glo[l] * om[b][l];  // omega^{bb} = 0
-            sc += pi[a][l] * glo[l] * sig[b][l];
-          }
-          B[a][b] = sb;
-          Cm[a][b] = sc;
-        }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = a; b < 4; ++b) {
-          R Dab = ((a == b) ? gup[a] : R(-0.0)) - uc[a] * uc[b];
-          R I1 = av[a] * uc[b] + av[b] * uc[a];
-          R I3 = B[a][b] + B[b][a];
-          R I4 = R(0.5) * (Cm[a][b] + Cm[b][a]) - Dab * ps3;
-          R Ipi = I1 + R(4.0 / 3.0) * theta * pi[a][b] - I3 + tpp * I4 - R(1.2) * Pic * sig[a][b];
-          R S = (R(2) * eta_tp * sig[a][b] - rate_pi * pi[a][b] - Ipi) * iu0 + pi[a][b] * dv;
-          if constexpr (DIAG) {  // sums over the full tensor: off-diagonal pairs count twice
+            for (int l = 0; l < 4; ++l)
+              c += glo[l] * (pi[a][l] * fma(uc[b], D[l], Y[b][l]) + pi[b][l] * fma(uc[a], D[l], Y[a][l]));
             const R w = glo[a] * glo[b] * ((a == b) ? R(1) : R(2));
-            const R X = Ipi - I1;  // -J^{ab}/tau_pi
+            const R Dab = ((a == b) ? gup[a] : R(-0.0)) - uc[a] * uc[b];
+            const R X = R(4.0 / 3.0) * theta * pi[a][b] - c - tp3 * Dab - R(1.2) * Pic * sig[a][b];  // -J^{ab}/tau_pi
             dg[2] += pi[a][b] * pi[a][b] * w;
             dg[4] += X * X * w;
             xs += sig[a][b] * sig[a][b] * w;
           }
-          // -G^{ab}/u^tau with G^{ab} = u^c Gamma^a_{cd} pi^{db} + (a <-> b)
-          R ha = (a == 0) ? tg * uc[3] * pi[3][b] : ((a == 3) ? it * (uc[0] * pi[3][b] + uc[3] * pi[0][b]) : R(-0.0));
-          R hb = (b == 0) ? tg * uc[3] * pi[3][a] : ((b == 3) ? it * (uc[0] * pi[3][a] + uc[3] * pi[0][a]) : R(-0.0));
-          const bool geo = (a == 0 || a == 3 || b == 0 || b == 3);  // (a, b) in {1, 2}^2: G^{ab} = 0
-          dq[pix(a, b)] += geo ? S - (ha + hb) * iu0 : S;
-        }
-      if constexpr (DIAG) {
         dg[0] = sdiv(R(5) * es, T) * theta;
         dg[4] = (xs > R(0)) ? sdiv(sqrt(dg[4]), R(2) * eta_tp * sqrt(xs)) : R(0);
-        (void)xs;
+      }
+      // M^b_l = g_{ll} Y^{bl} - K^b_l, and on its diagonal half of the coefficient of pi^{ab}:
+      // -1/tau_pi - 4 theta/3 (delta_pipi) + u^tau d_i v^i (S_pi's pi d_i v^i, taken inside the 1/u^tau)
+      const R hc = rmul(R(0.5), fma(uc[0], dv, fma(R(-4.0 / 3.0), theta, -rate_pi)));
+      R M[4][4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        M[b][0] = Y[b][0];
+        M[b][1] = -Y[b][1];
+        M[b][2] = -Y[b][2];
+        M[b][3] = rmul(-gnn, Y[b][3]);
+      }
+      M[0][3] = fma(-tg, uc[3], M[0][3]);
+      M[3][0] = fma(-it, uc[3], M[3][0]);
+      M[3][3] = fma(-it, uc[0], M[3][3] + hc);
+      M[0][0] += hc;
+      M[1][1] += hc;
+      M[2][2] += hc;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const R tpu = tp3 * uc[a];
+        // diagonal: twice pi^{al} M^a_l
+        R h = fma(pi[a][0], M[a][0], fma(pi[a][1], M[a][1], fma(pi[a][2], M[a][2], pi[a][3] * M[a][3])));
+        const R dg0 = (a == 0) ? tp3 : ((a == 3) ? gup[3] * tp3 : -tp3);
+        h = fma(R(2), h, fma(csig, sig[a][a], fma(-tpu, uc[a], dg0)));
+        dq[pix(a, a)] = fma(iu0, h, dq[pix(a, a)]);
+#pragma unroll
+        for (int b = a + 1; b < 4; ++b) {
+          R s = fma(csig, sig[a][b], -(tpu * uc[b]));
+#pragma unroll
+          for (int l = 0; l < 4; ++l) s = fma(pi[a][l], M[b][l], fma(pi[b][l], M[a][l], s));
+          dq[pix(a, b)] = fma(iu0, s, dq[pix(a, b)]);
+        }
       }
     }
     if (P.bulk_on) {
-      R lrate = R(2.70805020110221) + R(2) * lnd + slog(T) - ln_zeta_over_s<R>(P, T);  // ln 15 + ...
-      R rate_Pi = fmin(sexp(lrate), pr<R>(P).rate_max);
-      R d = sexp(lnd);
-      R zt = R(15) * d * d * (ec + P0c);
-      R IPi = R(2.0 / 3.0) * Pic * theta - R(1.6) * d * ps;
+      const R d = sexp(lnd);
+      const R d15 = R(15) * d * d;
+      // 1/tau_Pi = 15 (1/3 - c_s^2)^2 T / (zeta/s): both factors span hundreds of e-folds away from the
+      // transition, so their quotient is formed in the exponent (Eq. (zetas), bounded below, divides)
+      R rate_Pi;
+      if (P.zeta.kind == 2) {
+        const R z = pr<R>(P).zeta_c0 * zeta_over_s_paper<R>(T * pr<R>(P).zeta_inv_c1);
+        rate_Pi = (z > R(0)) ? sdiv(d15 * T, z) : R(INFINITY);
+      } else {
+        rate_Pi = R(15) * T * sexp(fma(R(2), lnd, -ln_zeta_over_s<R>(P, T)));
+      }
+      rate_Pi = nmin(rate_Pi, pr<R>(P).rate_max);
+      const R zt = d15 * (ec + P0c);
+      const R IPi = R(2.0 / 3.0) * Pic * theta - R(1.6) * d * ps;
       dq[14] += (-zt * theta - rate_Pi * Pic - IPi) * iu0 + Pic * dv;
       if constexpr (DIAG) {
+        const R lrate = R(2.70805020110221) + R(2) * lnd + slog(T) - ln_zeta_over_s<R>(P, T);  // ln 15 + ...
         dg[1] = sexp(-lrate) * theta;
         dg[5] = (theta != R(0)) ? sdiv(fabs(IPi), zt * fabs(theta)) : R(0);
       }
