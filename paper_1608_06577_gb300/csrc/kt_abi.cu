@@ -222,8 +222,8 @@ void fill_pr(PR<R>& o, const Params& P) {
   o.half_dtau = (R)(0.5 * P.dtau);
   o.rate_max = (R)P.rate_max;
   o.tpp = (R)P.tpp;
-  o.rho_max = (R)P.rho_max;
-  o.xi0_rho_max = (R)(P.xi0 * P.rho_max);
+  o.inv_rho_max = (R)(1.0 / P.rho_max);
+  o.inv_xi0_rho_max = (R)(1.0 / (P.xi0 * P.rho_max));
   o.eos_a = (R)P.eos_a;
   o.eta_c0 = (R)P.eta.c0; o.eta_c1 = (R)P.eta.c1; o.eta_inv_c2 = (R)(1.0 / P.eta.c2); o.eta_ln_c0 = (R)P.eta.ln_c0;
   o.eta_inv_c1 = (R)(1.0 / P.eta.c1);

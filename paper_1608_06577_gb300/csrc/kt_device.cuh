@@ -91,7 +91,7 @@ struct PR {
   R inv_dtau, dtau, half_dtau;
   R rate_max;          // 1/tau_relax_min (or +inf)
   R tpp;               // tau_pipi/tau_pi
-  R rho_max, xi0_rho_max;
+  R inv_rho_max, inv_xi0_rho_max;  // 1/rho_max, 1/(xi0 rho_max)
   R eos_a;
   R eta_c0, eta_c1, eta_inv_c2, eta_ln_c0, eta_inv_c1, eta_inv_5c0;  // eta_inv_5c0 = 1/(5 c0)
   R zeta_c0, zeta_c1, zeta_inv_c2, zeta_ln_c0, zeta_inv_c1;
@@ -205,6 +205,13 @@ __device__ __forceinline__ void eos_T_lnd(const Params& P, R e, R& T, R& lnd) {
   lnd = fma(t, s.dl, s.l0);
 }
 
+// x / 2 by its exponent; |x| < 2^-1021 gives 0
+__device__ __forceinline__ double half_bits(double x) {
+  const int hi = __double2hiint(x);
+  return ((hi & 0x7ff00000) > 0x00100000) ? __hiloint2double(hi - 0x00100000, __double2loint(x)) : 0.0;
+}
+__device__ __forceinline__ float half_bits(float x) { return 0.5f * x; }
+
 // Generalised minmod of (theta dl, (dl + dr)/2, theta dr), Sec. 3.1, with sgn(0) = 0, from the
 // one-sided differences dl = q_i - q_{i-1}, dr = q_{i+1} - q_i: the three arguments share a sign
 // exactly when dl and dr do, and then the result is that sign times the smallest magnitude.
@@ -213,6 +220,7 @@ __device__ __forceinline__ void eos_T_lnd(const Params& P, R e, R& T, R& lnd) {
 // their bit patterns), so only the theta branch does FP64 arithmetic.  FP32 with theta = 1: the
 // median of (dl, dr, 0) by four min/max instructions.  (FP32 theta != 1 tests the sign by the
 // product, which loses slopes whose one-sided differences multiply below ~1e-45.)
+// (half_bits halves the sum in its exponent, off the FP64 pipe.)
 // TH1: theta = 1, where (|dl| + |dr|)/2 >= min(|dl|, |dr|) never decides.
 template <typename R, bool TH1 = false>
 __device__ __forceinline__ R limited_slope_d(R dl, R dr, R theta) {
@@ -221,7 +229,7 @@ __device__ __forceinline__ R limited_slope_d(R dl, R dr, R theta) {
     const long long ml = bl & 0x7fffffffffffffffLL, mr = br & 0x7fffffffffffffffLL;
     R m = (ml < mr) ? dl : dr;  // the smaller magnitude (0 if either is 0), with the shared sign
     if constexpr (!TH1) {
-      const R m1 = theta * m, m2 = R(0.5) * (dl + dr);
+      const R m1 = theta * m, m2 = half_bits(dl + dr);
       m = ((__double_as_longlong(m1) & 0x7fffffffffffffffLL) < (__double_as_longlong(m2) & 0x7fffffffffffffffLL))
               ? m1 : m2;
     }
@@ -264,6 +272,25 @@ __device__ __forceinline__ float nmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double nmin(double a, double b) {
   return (__double_as_longlong(a) < __double_as_longlong(b)) ? a : b;
 }
+
+// Tests of values without the FP64 pipe (whose compares cost as much as its additions): x > 0,
+// x < y for y > 0 (a NaN compares false), x != y, x finite
+__device__ __forceinline__ bool pos(float x) { return x > 0.f; }
+__device__ __forceinline__ bool pos(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ULL;  // 0 < bits <= +inf's
+}
+__device__ __forceinline__ bool below(float x, float y) { return x < y; }
+__device__ __forceinline__ bool below(double x, double y) {
+  const long long b = __double_as_longlong(x);  // negative x has the sign bit set: below any y > 0
+  return b < __double_as_longlong(y) && (unsigned long long)b <= 0xfff0000000000000ULL;
+}
+__device__ __forceinline__ bool differs(float x, float y) { return x != y; }
+__device__ __forceinline__ bool differs(double x, double y) { return __double_as_longlong(x) != __double_as_longlong(y); }
+__device__ __forceinline__ bool finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+// 1/sqrt(x) for x > 0: the library's in FP64, the hardware approximation (2 ulp) in FP32
+__device__ __forceinline__ float rsqrt_pos(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_pos(double x) { return rsqrt(x); }
 
 // a b rounded to nearest, never contracted with a following addition: a product that several sums
 // read gives the same bits in every kernel that inlines the expression

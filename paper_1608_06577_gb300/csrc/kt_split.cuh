@@ -384,7 +384,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
         pm[a][b] = qr[pix(a, b)];
         pm[b][a] = pm[a][b];
       }
-    const float f = regulator_factor<float>(P, go, eR, P0R, uo, pm, qr[14]);
+    const float f = regulator_factor<float>(P, go, from_f64<float>(tau_out), eR, P0R, uo, pm, qr[14]);
     if (f < 0.999f) ++nreg;
     if (STAGE == 2 && io.reg_out) io.reg_out[c] = f;
     if (f != 1.f) {
