@@ -87,7 +87,7 @@ struct Ctx {
   // work decomposition
   int shape = 0;
   int ntiles = 0;
-  int grid_blocks = 0;    // fused stage kernel (FP64)
+  int grid_blocks = 0;    // the stage kernel's blocks (FP64), or grid_rhs
   int grid_rhs = 0;       // mixed precision: right-hand-side kernel
   int grid_upd = 0;       // mixed precision: update kernel
   bool tuned = false;
@@ -161,6 +161,23 @@ int tiles_for(const std::vector<Lattice>& lat, const Shape& s) {
   return (int)n;
 }
 
+// the FP64 stage's blocks: 32 consecutive cells of an event each
+long long strips_of(const Lattice& L) { return ((long long)L.nx * L.ny * L.nz + 31) / 32; }
+long long strips_for(const std::vector<Lattice>& lat) {
+  long long n = 0;
+  for (const auto& L : lat) n += strips_of(L);
+  return n;
+}
+
+// entries of the work table: the tiles of the shape with most of them (mixed precision), or the
+// strips of a batch (FP64; a single event needs no table)
+long long table_entries(const std::vector<Lattice>& lat, int mixed) {
+  if (!mixed) return lat.size() > 1 ? strips_for(lat) : 1;
+  int n = 0;
+  for (const auto& s : kShapes) n = std::max(n, tiles_for(lat, s));
+  return n;
+}
+
 void build_tiles(const std::vector<Lattice>& lat, const Shape& s, std::vector<Tile>& out) {
   out.clear();
   for (int e = 0; e < (int)lat.size(); ++e) {
@@ -175,8 +192,6 @@ void build_tiles(const std::vector<Lattice>& lat, const Shape& s, std::vector<Ti
 size_t state_bytes(const std::vector<Lattice>& lat, long long gs, size_t max_cells, int mixed, int eos_n) {
   const size_t fs = (size_t)gs;
   const size_t es = mixed ? 4 : 8;
-  int max_tiles = 0;
-  for (const auto& s : kShapes) max_tiles = std::max(max_tiles, tiles_for(lat, s));
   size_t b = 0;
   b += align_up(30 * fs * 8, 256);             // q, qs
   if (mixed) b += align_up(30 * fs * 4, 256);  // FP32 copies of q, qs
@@ -192,7 +207,7 @@ size_t state_bytes(const std::vector<Lattice>& lat, long long gs, size_t max_cel
   b += align_up(KT_MLP_NPARAM * 4, 256);       // MLP weights
   b += align_up(KT_MLP_PACKED_BYTES, 256);     // packed MLP weights
   b += align_up(lat.size() * sizeof(Lattice), 256);
-  b += align_up((size_t)max_tiles * sizeof(Tile), 256);
+  b += align_up((size_t)table_entries(lat, mixed) * sizeof(Tile), 256);
   if (mixed) b += align_up(2 * lat.size() * sizeof(CUtensorMap), 256);
   if (mixed) b += align_up(kUpdMaps * lat.size() * sizeof(CUtensorMap), 256);
   b += align_up(fs * 4, 256);                  // regulation factors
@@ -565,17 +580,14 @@ UpdIO make_uio(Ctx* c, int stage) {
 
 template <int STAGE>
 void launch_stage(Ctx* c, const StageIO<double>& io) {
-  const Shape& s = kShapes[c->shape];
-  const dim3 blk(s.x, s.y, s.z);
   const bool t1 = (c->P.theta == 1.0), inv = c->P.iface_invert;
-  if (t1 && !inv)
-    stage_kernel<double, STAGE, true, false><<<c->grid_blocks, blk, 0, c->stream>>>(c->P, io, c->d_lat, c->d_tiles, c->ntiles);
-  else if (!inv)
-    stage_kernel<double, STAGE, false, false><<<c->grid_blocks, blk, 0, c->stream>>>(c->P, io, c->d_lat, c->d_tiles, c->ntiles);
-  else if (t1)
-    stage_kernel<double, STAGE, true, true><<<c->grid_blocks, blk, 0, c->stream>>>(c->P, io, c->d_lat, c->d_tiles, c->ntiles);
-  else
-    stage_kernel<double, STAGE, false, true><<<c->grid_blocks, blk, 0, c->stream>>>(c->P, io, c->d_lat, c->d_tiles, c->ntiles);
+  auto go = [&](auto kernel) {
+    kernel<<<c->grid_blocks, 32, 0, c->stream>>>(c->P, io, c->lat[0], c->d_lat, c->d_tiles, c->nev);
+  };
+  if (t1 && !inv) go(stage_kernel<double, STAGE, true, false>);
+  else if (!inv) go(stage_kernel<double, STAGE, false, false>);
+  else if (t1) go(stage_kernel<double, STAGE, true, true>);
+  else go(stage_kernel<double, STAGE, false, true>);
 }
 
 // the right-hand-side kernel of a stage, with the minmod specialised when theta = 1
@@ -822,10 +834,27 @@ int encode_tensor_maps(Ctx* c) {
   return KT_OK;
 }
 
+// The FP64 mode has one layout (see stage_kernel): blocks of 32 consecutive cells, whatever candidate
+// is asked for.
+int select_strips(Ctx* c, int cand) {
+  c->grid_blocks = (int)strips_for(c->lat);
+  if (c->nev > 1 && c->ntiles == 0) {
+    std::vector<Tile> strips;
+    for (int e = 0; e < c->nev; ++e)
+      for (long long s = 0; s < strips_of(c->lat[e]); ++s) strips.push_back(Tile{e, (int)(32 * s), 0, 0});
+    CK(cudaMemcpyAsync(c->d_tiles, strips.data(), strips.size() * sizeof(Tile), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+  }
+  c->ntiles = c->grid_blocks;
+  c->cand = cand;
+  return KT_OK;
+}
+
 int select_shape(Ctx* c, int cand) {
+  if (!c->mixed) return select_strips(c, cand);
   const int base = cand % kNumBase, shape = base / 2, one_per_tile = base % 2, variant = cand / kNumBase;
-  const bool fusable = c->mixed && !c->pi32 && !c->P.iface_invert;
-  c->staged = (variant == 1) && c->mixed && !c->pi32;
+  const bool fusable = !c->pi32 && !c->P.iface_invert;
+  c->staged = (variant == 1) && !c->pi32;
   c->fused = (variant == 2) && fusable;
   c->upd_nbuf = one_per_tile ? 1 : 2;
   std::vector<Tile> tiles;
@@ -835,28 +864,22 @@ int select_shape(Ctx* c, int cand) {
   CK(cudaStreamSynchronize(c->stream));
   c->shape = shape;
   c->ntiles = (int)tiles.size();
-  if (c->mixed) {
-    int rc = encode_tensor_maps(c);
-    if (rc != KT_OK) return rc;
-  }
+  int rc = encode_tensor_maps(c);
+  if (rc != KT_OK) return rc;
   const Shape& sh = kShapes[shape];
   auto grid = [&](int cap) { return one_per_tile ? c->ntiles : std::max(1, std::min(cap, c->ntiles)); };
-  if (c->mixed) {
-    const size_t rsm = rhs_smem_bytes(sh.x, sh.y, sh.z);
-    c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<1, true, false, true>, sh, rsm)
-                                : occupancy_blocks(rhs_kernel<1, true, false>, sh, rsm));
-    if (c->staged) {
-      const size_t usm = upd_smem_bytes(sh.x, sh.y, sh.z, c->upd_nbuf);
-      c->grid_upd = grid(c->learned ? occupancy_blocks(update_staged_kernel<2, true>, sh, usm)
-                                    : occupancy_blocks(update_staged_kernel<2, false>, sh, usm));
-    } else {
-      c->grid_upd = grid(c->learned ? occupancy_blocks(update_kernel<1, true, false>, sh)
-                                    : occupancy_blocks(update_kernel<1, false, false>, sh));
-    }
-    c->grid_blocks = c->grid_rhs;
+  const size_t rsm = rhs_smem_bytes(sh.x, sh.y, sh.z);
+  c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<1, true, false, true>, sh, rsm)
+                              : occupancy_blocks(rhs_kernel<1, true, false>, sh, rsm));
+  if (c->staged) {
+    const size_t usm = upd_smem_bytes(sh.x, sh.y, sh.z, c->upd_nbuf);
+    c->grid_upd = grid(c->learned ? occupancy_blocks(update_staged_kernel<2, true>, sh, usm)
+                                  : occupancy_blocks(update_staged_kernel<2, false>, sh, usm));
   } else {
-    c->grid_blocks = grid(occupancy_blocks(stage_kernel<double, 1, true, false>, sh));  // same launch bounds
+    c->grid_upd = grid(c->learned ? occupancy_blocks(update_kernel<1, true, false>, sh)
+                                  : occupancy_blocks(update_kernel<1, false, false>, sh));
   }
+  c->grid_blocks = c->grid_rhs;
   c->cand = cand;
   for (int p = 0; p < 3; ++p)
     if (c->graph[p]) { cudaGraphExecDestroy(c->graph[p]); c->graph[p] = nullptr; }
@@ -866,18 +889,13 @@ int select_shape(Ctx* c, int cand) {
 // Autotuner: time first-stage launches for every candidate (tile shape, grid size, layout).  The
 // launches write only scratch buffers (q*, its FP32 copy, e*, p*, and u* redirected to the spare
 // buffer), so the state is untouched; the fastest candidate is kept.
-template <typename R>
 int time_first_stage(Ctx* c, float* ms) {
-  StageIO<R> io = make_io<R>(c, 1);
-  io.u_out = (R*)c->U[c->spare];
-  auto launch = [&]() {
-    if constexpr (sizeof(R) == 4) {  // writes k_1, q*'s FP32 copy, e*, P*, u* (spare buffer)
-      UpdIO u = make_uio(c, 1);
-      u.u_out = (float*)c->U[c->spare];
-      launch_split_stage<1>(c, io, u);
-    } else {
-      launch_stage<1>(c, io);
-    }
+  StageIO<float> io = make_io<float>(c, 1);
+  io.u_out = (float*)c->U[c->spare];
+  auto launch = [&]() {  // writes k_1, q*'s FP32 copy, e*, P*, u* (spare buffer)
+    UpdIO u = make_uio(c, 1);
+    u.u_out = (float*)c->U[c->spare];
+    launch_split_stage<1>(c, io, u);
   };
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
@@ -901,14 +919,13 @@ int autotune(Ctx* c) {
   Range range_("kt autotune");
   int best = 0;
   for (int s = 0; s < kNumCandidates; ++s) c->tune_ms[s] = 0.f;
-  const bool fusable = c->mixed && !c->pi32 && !c->P.iface_invert;
+  const bool fusable = !c->pi32 && !c->P.iface_invert;
   for (int s = 0; s < kNumCandidates; ++s) {
     if (!(s < kNumBase || (fusable && s >= kFusedFirst))) continue;
     int rc = select_shape(c, s);
     if (rc != KT_OK) return rc;
     float ms = 0.f;
-    if (c->mixed) rc = time_first_stage<float>(c, &ms);
-    else rc = time_first_stage<double>(c, &ms);
+    rc = time_first_stage(c, &ms);
     if (rc != KT_OK) return rc;
     c->tune_ms[s] = ms;
     if (ms < c->tune_ms[best]) best = s;
@@ -1114,7 +1131,7 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->d_mlp = (float*)carve(KT_MLP_NPARAM * 4);
   c->d_mlp_packed = (uint32_t*)carve(KT_MLP_PACKED_BYTES);
   c->d_lat = (Lattice*)carve(c->lat.size() * sizeof(Lattice));
-  for (const auto& s : kShapes) c->max_tiles = std::max(c->max_tiles, tiles_for(c->lat, s));
+  c->max_tiles = (int)table_entries(c->lat, c->mixed);
   c->d_tiles = (Tile*)carve((size_t)c->max_tiles * sizeof(Tile));
   if (c->mixed) c->d_tmaps = (CUtensorMap*)carve(2 * c->lat.size() * sizeof(CUtensorMap));
   if (c->mixed) c->d_umaps = (CUtensorMap*)carve(kUpdMaps * c->lat.size() * sizeof(CUtensorMap));
@@ -1236,7 +1253,7 @@ namespace {
 int begin_steps(Ctx* c, int n_steps) {
   for (int e = 0; e < c->nev; ++e)
     if (!c->ev_set[e]) return fail(c, KT_ERR_ARG, "kt_step: event %d has no state", e);
-  if (c->opt.autotune && !c->tuned && n_steps > 0) {
+  if (c->mixed && c->opt.autotune && !c->tuned && n_steps > 0) {
     int rc = autotune(c);
     if (rc != KT_OK) return rc;
   }
@@ -1522,9 +1539,10 @@ int kt_mlp_features(kt_ctx* c, long long n, const long long* cells, float* x, fl
 int kt_get_tuning(kt_ctx* c, int* block_xyz, int* grid_blocks, float* candidate_ms, int* n_candidates) {
   if (!c) return KT_ERR_ARG;
   if (block_xyz) {
-    block_xyz[0] = kShapes[c->shape].x;
-    block_xyz[1] = kShapes[c->shape].y;
-    block_xyz[2] = kShapes[c->shape].z;
+    const Shape s = c->mixed ? kShapes[c->shape] : Shape{32, 1, 1};
+    block_xyz[0] = s.x;
+    block_xyz[1] = s.y;
+    block_xyz[2] = s.z;
   }
   if (grid_blocks) *grid_blocks = c->grid_blocks;
   if (n_candidates) {

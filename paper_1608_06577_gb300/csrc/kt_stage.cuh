@@ -214,6 +214,18 @@ __device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, co
   dq[D + 1] -= ((D == 2) ? (Ppl - Pmi) * inv_gnn : (Ppl - Pmi)) * hinv;
 }
 
+// An axis of one cell: its neighbours are copies of the cell, so every difference along it vanishes; the
+// local speed is that of the cell itself.
+template <typename R, int D>
+__device__ __forceinline__ void face_none(const R (&uc)[4], R sfac, R (&du)[4][4], float& amax, Faces<R>& F) {
+  const R a = fabs(vdiv(uc[D + 1], uc[0]));
+  amax = fmaxf(amax, to_f32((D == 2) ? a * sfac : a));
+  F.c0 = F.wLm = F.wRp = F.hdW = F.vpl_h = F.vmi_h = R(0);
+  F.s = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) du[D + 1][m] = R(0);
+}
+
 // row nu of T^{tau nu} that component n feeds through -d_d(-v^d pi^{tau nu}) (first == true:
 // n = pi^{tau nu}) or -d_d(pi^{d nu}) (n = pi^{d nu}); -1 if none
 template <int D>
@@ -369,17 +381,70 @@ __device__ __forceinline__ void component_rhs_xy(const Params& P, int n, const f
   }
 }
 
-// All 15 components from global memory.  The component loop is not unrolled: one compact body
-// keeps the instruction stream of the whole kernel small.
+// All 15 components from global memory (FP64), all 32 lanes of the warp together.  An FP64 instruction
+// costs its warp 64 cycles however many lanes are active, so work that cannot contribute is skipped by
+// the whole warp: a component whose stencil is zero in every cell of the warp (pi and Pi of an ideal
+// fluid, Pi of a conformal one) adds zero, and so does an axis of one cell, whose neighbours are all
+// copies of it.  The next component's stencil is loaded while the current one computes: a grid with few
+// warps has nothing else to cover the load latency with.
+template <typename R>
+struct Stencil13 {
+  R a0, v[3][4];  // the cell and, per axis, i-2, i-1, i+1, i+2
+};
 template <typename R, bool TH1 = false>
 __device__ __forceinline__ void conserved_fluxes(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
                                                  const Faces<R>& Fx, const Faces<R>& Fy, const Faces<R>& Fz,
                                                  R (&dq)[NQ]) {
   const long long fs = L.fstride;
   const R th = pr<R>(P).theta;
-  const R* p = io.qr_in + c;
-#pragma unroll 1
-  for (int n = 0; n < NQ; ++n, p += fs) component_rhs<R, false, TH1>(P, n, p, Fx.s, Fy.s, Fz.s, th, Fx, Fy, Fz, dq);
+  const bool on[3] = {L.nx > 1, L.ny > 1, L.nz > 1};
+  const Faces<R>* const F[3] = {&Fx, &Fy, &Fz};
+  const R c0 = (on[0] ? Fx.c0 : R(0)) + (on[1] ? Fy.c0 : R(0)) + (on[2] ? Fz.c0 : R(0));
+  auto load = [&](int n) {
+    const R* p = io.qr_in + n * fs + c;
+    Stencil13<R> q;
+    q.a0 = ld<R>(p, 0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int s = F[d]->s;
+      q.v[d][0] = q.v[d][1] = q.v[d][2] = q.v[d][3] = R(0);
+      if (on[d]) {
+        q.v[d][0] = ld<R>(p, -2 * s); q.v[d][1] = ld<R>(p, -s); q.v[d][2] = ld<R>(p, s); q.v[d][3] = ld<R>(p, 2 * s);
+      }
+    }
+    return q;
+  };
+  Stencil13<R> q = load(0);
+#pragma unroll
+  for (int n = 0; n < NQ; ++n) {
+    Stencil13<R> next;
+    if (n + 1 < NQ) next = load(n + 1);
+    long long bits = __double_as_longlong(q.a0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) bits |= __double_as_longlong(q.v[d][k]);
+    if (__any_sync(0xffffffffu, (bits << 1) != 0)) {
+      R acc = c0 * q.a0, mix = R(-0.0);  // mix: sum of the v^d pi^{tau nu} differences
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (!on[d]) continue;
+        const R a1 = q.v[d][1], b1 = q.v[d][2];
+        const R d0 = a1 - q.v[d][0], d1 = q.a0 - a1, d2 = b1 - q.a0, d3 = q.v[d][3] - b1;
+        R sm, s0, sp;
+        three_slopes<R, TH1>(d0, d1, d2, d3, th, sm, s0, sp);
+        acc = fma(F[d]->wLm, fma(R(0.5), sm, a1), acc);
+        acc = fma(F[d]->wRp, fma(R(-0.5), sp, b1), acc);
+        acc = fma(F[d]->hdW, s0, acc);
+        if (n >= 4 && n <= 7) mix = fma(F[d]->vpl_h, b1, fma(-F[d]->vmi_h, a1, mix));
+        const int r = (d == 0) ? cross_row<0>(n, false) : ((d == 1) ? cross_row<1>(n, false) : cross_row<2>(n, false));
+        if (n >= 4 && n <= 13 && r >= 0) add_row(dq, r, (a1 - b1) * pr<R>(P).half_inv_d[d]);
+      }
+      dq[n] += acc;
+      if (n >= 4 && n <= 7) dq[n - 4] += mix;
+    }
+    q = next;
+  }
 }
 
 // ------------------------------------------------------------- d) the root-find (Sec. 2.4)
@@ -665,9 +730,18 @@ __device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, co
   for (int m = 0; m < 4; ++m) uc[m] = ua(m, 0);
   dv = R(-0.0);
   const R sfac = P.milne ? G.tau : R(1);  // sqrt(-g_{eta eta}): speeds along eta in units of c
-  face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fx);
-  face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fy);
-  face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fz);
+  if constexpr (sizeof(R) == 8 && !IFACE) {
+    if (L.nx > 1) face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fx);
+    else face_none<R, 0>(uc, R(1), du, amax, Fx);
+    if (L.ny > 1) face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fy);
+    else face_none<R, 1>(uc, R(1), du, amax, Fy);
+    if (L.nz > 1) face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fz);
+    else face_none<R, 2>(uc, sfac, du, amax, Fz);
+  } else {
+    face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fx);
+    face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fy);
+    face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fz);
+  }
 }
 
 template <typename R, bool DIAG = false>
@@ -917,24 +991,26 @@ __device__ __forceinline__ double learned_start(const InvIn& v, float z) {
   return f2d_bits(v.Ef * ecE * __expf(0.1f * y));
 }
 
-// ---------------------------------------------------------------- one cell of a tile (FP64)
-// The whole stage for one cell in one thread; cells past the edge of the event (valid = false)
-// compute nothing and store nothing.
+// ---------------------------------------------------------------- one cell (FP64)
+// The whole stage for cell o (x fastest, then y, then eta) of an event in one thread.  The 32 lanes of a
+// warp hold consecutive cells and stay together; lanes past the last cell repeat it and store nothing.
 template <typename R, int STAGE, bool TH1, bool IFACE>
-__device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, const StageIO<R>& io, int i, int j,
-                                           int k, unsigned& st, unsigned& nit, unsigned& nreg, float& amax) {
+__device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, const StageIO<R>& io, unsigned o,
+                                           unsigned& st, unsigned& nit, unsigned& nreg, float& amax) {
   static_assert(sizeof(R) == 8, "the fused stage is the FP64 path; mixed precision uses kt_split.cuh");
-  const bool valid = (i < L.nx) && (j < L.ny) && (k < L.nz);
+  const unsigned ncells = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
+  const bool valid = o < ncells;
+  o = min(o, ncells - 1u);
+  const unsigned row = o / (unsigned)L.nx;
+  const int i = (int)(o - row * (unsigned)L.nx), k = (int)(row / (unsigned)L.ny), j = (int)row - k * L.ny;
   const long long fs = L.fstride;
   const long long c = L.idx(i + 2, j + 2, k + 2);
   const double tau_n = io.d_tau[0];
   const double tau_src = (STAGE == 1) ? tau_n : tau_n + P.dtau;
   const double tau_out = tau_n + P.dtau;
-  double qn[NQ];  // the new conserved state (a harmless rest state on lanes past the edge)
-#pragma unroll
-  for (int n = 0; n < NQ; ++n) qn[n] = (n == 0) ? 1.0 : 0.0;
+  double qn[NQ];  // the new conserved state
 
-  if (valid) {
+  {
     R dq[NQ];
     cell_rhs<R, TH1, IFACE>(P, L, io, c, tau_src, dq, amax);
 
@@ -949,12 +1025,16 @@ __device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, co
     }
   }
 
-  if (valid) {
+  {
     // ---- d) inversion at tau^{n+1}
     double e, P0;
     R uo[4];
     const double guess = to_f64<R>(ld<R>(io.e_in, c));
-    st |= invert_fp64(P, tau_out, qn, guess, e, P0, uo, nit);
+    unsigned its = 0;
+    const unsigned sti = invert_fp64(P, tau_out, qn, guess, e, P0, uo, its);
+    if (!valid) return;
+    st |= sti;
+    nit += its;
 
     // the new state in the stencil precision (the copy the next stage's stencil reads)
     R qr[NQ];
@@ -1036,25 +1116,45 @@ __device__ __forceinline__ void block_stats(unsigned* status, unsigned* max_spee
   }
 }
 
-// ---------------------------------------------------------------- the stage kernel
-// Persistent: every block walks its run of the tile table; a tile is one block-shaped patch of one
-// event, so one launch per Runge-Kutta stage advances every event of the context.
+// ---------------------------------------------------------------- the stage kernel (FP64)
+// One warp per block and per 32 consecutive cells of an event.  The kernel is bound by the FP64 pipe:
+// measured, one warp instruction per 19 cycles and SM from four warps on (64 cycles for a lone warp),
+// the same with one active lane as with 32.  Hence cells in linear order (a 32-wide tile of a 37-cell
+// row would leave 27 of 64 lanes idle at full cost), and blocks of one warp, so that a grid with few
+// cells spreads over all SMs and no SM's last wave holds eight warps.  Against 256-thread tiles on a
+// grid of resident blocks: shock tube of 200 cells, 80 steps, 9.03 -> 3.83 ms (with the one-cell axes
+// and vanishing components skipped), Gubser grid 32 x 32 x 8, 20 steps, 4.13 -> 3.58 ms, three 128^3
+// steps 36.5 -> 35.9 ms.
+__device__ __forceinline__ void warp_stats(const StageIO<double>& io, unsigned st, float amax, unsigned nit,
+                                           unsigned nreg) {
+  const unsigned full = 0xffffffffu;
+  const unsigned w_st = __reduce_or_sync(full, st), w_max = __reduce_max_sync(full, __float_as_uint(amax));
+  const unsigned w_it = __reduce_add_sync(full, nit), w_reg = __reduce_add_sync(full, nreg);
+  if (threadIdx.x == 0) {
+    if (w_st) atomicOr(io.status, w_st);
+    atomicMax(io.max_speed_bits, w_max);
+    if (w_it) atomicAdd(io.counters + 0, (unsigned long long)w_it);
+    if (w_reg) atomicAdd(io.counters + 1, (unsigned long long)w_reg);
+  }
+}
+
+// strips: (event, first cell) of every block; with a single event (n_events = 1) the block index says it
 template <typename R, int STAGE, bool TH1, bool IFACE>
-__global__ void __launch_bounds__(256, 1)
-    stage_kernel(const Params P, const StageIO<R> io, const Lattice* __restrict__ lats, const Tile* __restrict__ tiles,
-                 int ntiles) {
+__global__ void __launch_bounds__(32, 8)
+    stage_kernel(const Params P, const StageIO<R> io, const Lattice L0, const Lattice* __restrict__ lats,
+                 const Tile* __restrict__ strips, int n_events) {
   unsigned st = 0, nit = 0, nreg = 0;
   float amax = 0.f;
-  int t0, t1;
-  tile_range(ntiles, t0, t1);
-  for (int t = t0; t < t1; ++t) {
-    const Tile tl = tiles[t];
-    const Lattice L = lats[tl.event];
-    stage_cell<R, STAGE, TH1, IFACE>(P, L, io, tl.i0 + (int)threadIdx.x, tl.j0 + (int)threadIdx.y, tl.k0 + (int)threadIdx.z, st,
-                         nit, nreg, amax);
+  Lattice L = L0;
+  unsigned first = 32u * blockIdx.x;
+  if (n_events > 1) {
+    const Tile s = strips[blockIdx.x];
+    L = lats[s.event];
+    first = (unsigned)s.i0;
   }
-
-  block_stats(io.status, io.max_speed_bits, io.counters, st, amax, nit, nreg, 0u);
+  stage_cell<R, STAGE, TH1, IFACE>(P, L, io, first + threadIdx.x, st, nit, nreg, amax);
+  __syncwarp();
+  warp_stats(io, st, amax, nit, nreg);
 }
 
 }  // namespace kt
