@@ -67,8 +67,8 @@ SLOT_BYTES = {
 FUSED_SLOT_BYTES = {"learned_start": 40, "stage1_rhs": 380, "stage2_rhs": 488}
 FUSED_FIRST_CANDIDATE = 24  # tuning candidates 24-35 are the fused launches (timed by the autotuner too)
 SLOT_KERNEL = {"learned_start": "mlp_start_kernel", "stage1_rhs": "rhs_kernel", "stage2_rhs": "rhs_kernel",
-               "stage1_update": "update_kernel", "stage2_update": "update_kernel", "tau_advance": "advance_tau_kernel"}
-LAUNCHES_PER_STEP = {"fp64": 3, "mixed": 5}  # + the tau advance (+ 1 for the network, learned start)
+               "stage1_update": "update_kernel", "stage2_update": "update_kernel"}
+LAUNCHES_PER_STEP = {"fp64": 2, "mixed": 4}  # (+ 1 for the network, learned start)
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the current kernels: one-
 # kernel ncu captures of the 96^3 learned workload, per cell times the 128^3 cells (average over
 # the two stages of each kernel; the update and fused kernels captured on 32x2x2 tiles, one block
@@ -402,7 +402,7 @@ def run_ours(args, world, rank, local):
     # per kernel: launches per step, average launch time, algorithmic bytes per launch, GB/s
     kernels = {}
     for slot, t in main["slots_ms"].items():
-        if t <= 0.0 or (fused and slot.endswith("update")):  # (fused: the update slots are empty)
+        if t <= 0.0 or slot == "tau_advance" or (fused and slot.endswith("update")):  # (empty intervals)
             continue
         name = SLOT_KERNEL[slot]
         if slot.endswith("rhs") and (args.mode == "fp64" or fused):
@@ -433,7 +433,7 @@ def run_ours(args, world, rank, local):
     dom = max(kernels, key=lambda n: kernels[n]["ms_per_step"])
     traffic_k = None if (args.large or args.eos != "workload") else MEASURED_TRAFFIC.get((args.mode, n))
     traffic = None
-    if traffic_k and all(k in traffic_k for k in kernels if k != "advance_tau_kernel"):
+    if traffic_k and all(k in traffic_k for k in kernels):
         # DRAM bytes per step: every kernel's recorded traffic per launch times its launches
         traffic = sum(traffic_k[k] * v["launches_per_step"] for k, v in kernels.items() if k in traffic_k)
     achieved = cells * alg / (ms_step * 1e-3) / 1e9
@@ -532,7 +532,7 @@ def run_ours(args, world, rank, local):
                 "fp64_pipe": fp64_pipe, "layout_variants": variants,
                 "learned_training": train_info,
                 "roofline": roofline, "kernels": kernels, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-                "gpu_launches": ((3 if (args.mode == "fp64" or fused) else 5)
+                "gpu_launches": (LAUNCHES_PER_STEP["fp64" if (args.mode == "fp64" or fused) else "mixed"]
                                  + (1 if MODES[args.mode][1] == 1 else 0)) * main["steps"]}
         print(json.dumps(line), flush=True)
 

@@ -279,7 +279,8 @@ int kt_set_tuning(kt_ctx* ctx, int candidate);
  * network launch (0 without KT_INV_LEARNED), the stage-1 right-hand-side launch (FP64, fused
  * layout: the fused stage-1 launch), the stage-1 update launch (FP64, fused layout: 0), the
  * stage-2 right-hand-side launch (FP64, fused layout: the fused stage-2 launch), the stage-2
- * update launch (FP64, fused layout: 0) and the tau advance.  *n_kernels must be >= 6 on entry
+ * update launch (FP64, fused layout: 0) and the tau advance (an empty interval: the second stage's
+ * last launch advances tau).  *n_kernels must be >= 6 on entry
  * and is set to 6.  The state, tau and statistics advance as with kt_step; errors are those of
  * kt_step.  The per-step event synchronisation makes these steps slower in total than kt_step's. */
 int kt_time_kernels(kt_ctx* ctx, int n_steps, float* ms, int* n_kernels);

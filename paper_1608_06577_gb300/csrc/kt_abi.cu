@@ -69,7 +69,7 @@ struct Ctx {
   EosSeg<float>* seg_f = nullptr;
   RootSeg* seg_r = nullptr;
   RootSegM* seg_m = nullptr;
-  double* d_tau = nullptr;
+  double* d_tau = nullptr;  // three slots, used in rotation with the u buffers: tau^n is in slot cur
   unsigned* d_stat = nullptr;
   float* d_mlp = nullptr;
   uint32_t* d_mlp_packed = nullptr;
@@ -407,8 +407,6 @@ __global__ void scatter_kernel(const Params P, const Lattice L, const double* __
   for_cell_and_ghosts(P, L, i + 2, j + 2, k + 2, [&](long long t) { f[t] = v; });
 }
 
-__global__ void advance_tau_kernel(double* tau, double dtau) { tau[0] += dtau; }
-
 // smallest and largest e and smallest regulation factor over one event's physical cells (all
 // positive, so their float bit patterns order like the values): out[0] min e, [1] max e, [2] min f
 template <typename R>
@@ -544,7 +542,8 @@ StageIO<R> make_io(Ctx* c, int stage) {
     io.qr_in = (const R*)io.q_in;
     io.qr_out = nullptr;
   }
-  io.d_tau = c->d_tau;
+  io.d_tau = c->d_tau + c->cur;
+  io.tau_next = (stage == 2) ? c->d_tau + c->spare : nullptr;  // the next step's u^n buffer and tau slot
   io.status = c->d_stat;
   io.max_speed_bits = c->d_stat + 1;
   io.counters = (unsigned long long*)(c->d_stat + 4);
@@ -570,7 +569,8 @@ UpdIO make_uio(Ctx* c, int stage) {
   u.e_out = io.e_out;
   u.p_out = io.p_out;
   u.e_guess = io.e_in;
-  u.d_tau = c->d_tau;
+  u.d_tau = io.d_tau;
+  u.tau_next = io.tau_next;
   u.status = c->d_stat;
   u.counters = (unsigned long long*)(c->d_stat + 4);
   u.reg_out = io.reg_out;
@@ -703,7 +703,8 @@ void launch_split_stage(Ctx* c, const StageIO<float>& io, const UpdIO& uio) {
 
 // ev (optional, kNumTimed + 1 events): recorded between the launches of one step, in the order
 // learned start (the network's inference), stage-1 rhs (or fused stage 1), stage-1 update,
-// stage-2 rhs (or fused stage 2), stage-2 update, tau advance; intervals of launches a context
+// stage-2 rhs (or fused stage 2), stage-2 update, tau advance (always empty: the second stage
+// writes tau^{n+1}); intervals of launches a context
 // does not make (the network without the learned start, the update launches of the FP64 path and
 // of the fused layout) are empty.
 constexpr int kNumTimed = 6;
@@ -713,7 +714,7 @@ void mark(Ctx* c, cudaEvent_t* ev, int i) {
 
 // the learned start's network on the state at the start of the step (its FP32 copy)
 void launch_mlp_start(Ctx* c) {
-  kt::mlp_start_kernel<<<c->grid_mlp, 256, 0, c->stream>>>(c->qf, c->gs, c->d_tau, c->P.milne,
+  kt::mlp_start_kernel<<<c->grid_mlp, 256, 0, c->stream>>>(c->qf, c->gs, c->d_tau + c->cur, c->P.milne,
                                                            c->d_mlp_packed, c->z_net);
 }
 
@@ -751,11 +752,10 @@ void launch_step_stages(Ctx* c, cudaEvent_t* ev) {
   }
 }
 
-// enqueue one full step (two stages + tau advance) for the current rotation phase, then rotate
+// enqueue one full step (two stages; the second advances tau) for the current rotation phase, then rotate
 int enqueue_step(Ctx* c, cudaEvent_t* ev = nullptr) {
   if (c->mixed) launch_step_stages<float>(c, ev);
   else launch_step_stages<double>(c, ev);
-  advance_tau_kernel<<<1, 1, 0, c->stream>>>(c->d_tau, c->P.dtau);
   mark(c, ev, 6);
   // u^{n-1} <- u^n, u^n <- u^{n+1}; the old u^{n-1} buffer (holding u^*) becomes the spare
   int ncur = c->spare, nprev = c->cur, nspare = c->prev;
@@ -1215,7 +1215,7 @@ int kt_set_state_event(kt_ctx* c, int event, double tau, const double* e, const 
   if (u_prev) CK(cudaMemcpyAsync(s + 15 * ncp, u_prev, 3 * ncp * 8, kind, c->stream));
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   double tau_h = tau;
-  CK(cudaMemcpyAsync(c->d_tau, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
+  CK(cudaMemcpyAsync(c->d_tau + c->cur, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
   int nb = (int)((ncp + 255) / 256);
   // the state goes into the buffers that hold u^n and u^{n-1} in the current rotation
   if (c->mixed)
@@ -1463,7 +1463,7 @@ int kt_set_checkpoint(kt_ctx* c, int event, double tau, const double* buf, int o
     CK(cudaGetLastError());
   }
   double tau_h = tau;
-  CK(cudaMemcpyAsync(c->d_tau, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
+  CK(cudaMemcpyAsync(c->d_tau + c->cur, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->tau = tau;

@@ -34,6 +34,7 @@ struct UpdIO {
   float* p_out;
   const float* e_guess;     // the cell's previous energy density: the plain root-find's start
   const double* d_tau;      // tau^n
+  double* tau_next;         // stage 2: where tau^{n+1} goes
   unsigned* status;
   unsigned long long* counters;
   float* reg_out;           // stage 2: the regulation factor applied at each cell, or null
@@ -457,6 +458,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
     const UpdInGlobal in{io, L.fstride, L.idx(i + 2, j + 2, k + 2)};
     update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau_out, st, nit, nreg, nfb);
   }
+  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && (threadIdx.x | threadIdx.y | threadIdx.z) == 0);
   block_stats(io.status, nullptr, io.counters, st, 0.f, nit, nreg, nfb);
 }
 
@@ -603,6 +605,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
     for (; done < issued; ++done)
       mbar_wait(&s_bar[(nbuf == 2) ? (done & 1u) : 0u], (nbuf == 2) ? ((done >> 1) & 1u) : (done & 1u), kWaitPolls);
   }
+  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && tid == 0);
   block_stats(io.status, nullptr, io.counters, st | (bad ? ST_TIMEOUT : 0u), 0.f, nit, nreg, nfb);
 }
 
@@ -732,6 +735,7 @@ __global__ void __maxnreg__(128)
   if (bad) {  // a copy did not complete in time: let the ones in flight land before the block exits
     for (; done < issued; ++done) mbar_wait(&s_bar[done & 1u], (done >> 1) & 1u, kWaitPolls);
   }
+  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && tid == 0);
   block_stats(io.status, io.max_speed_bits, io.counters, st | (bad ? ST_TIMEOUT : 0u), amax, nit, nreg, nfb);
 }
 

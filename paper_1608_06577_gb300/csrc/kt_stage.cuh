@@ -33,6 +33,7 @@ struct StageIO {
   R* e_out;
   R* p_out;
   const double* d_tau;   // tau^n
+  double* tau_next;      // stage 2: where tau^{n+1} goes (another slot than d_tau), else null
   unsigned* status;
   unsigned* max_speed_bits;
   unsigned long long* counters;  // [0] Newton iterations, [1] regulated cells, [2] fallbacks
@@ -1074,6 +1075,12 @@ __device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, co
   }
 }
 
+// tau^{n+1} for the next step, written by one thread of the second stage into another slot than the one
+// this step's kernels read (a launch of its own cost 2 us per step: 4% of a small grid's)
+__device__ __forceinline__ void advance_tau(const Params& P, const double* d_tau, double* tau_next, bool first) {
+  if (tau_next && first) *tau_next = d_tau[0] + P.dtau;
+}
+
 // The contiguous run [t0, t1) of the tile table that this block processes.  Tiles are ordered
 // eta-fastest, so a block of a persistent grid walks up a column of tiles and the eta-neighbour
 // planes read by its stencil are mostly still in its SM's L1.
@@ -1154,6 +1161,7 @@ __global__ void __launch_bounds__(32, 8)
   }
   stage_cell<R, STAGE, TH1, IFACE>(P, L, io, first + threadIdx.x, st, nit, nreg, amax);
   __syncwarp();
+  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
   warp_stats(io, st, amax, nit, nreg);
 }
 
