@@ -317,81 +317,143 @@ void build_mixed_root_segments(const std::vector<RootSeg>& sr, std::vector<RootS
 // ------------------------------------------------------------------ small kernels
 __device__ __forceinline__ double gnn_at(const Params& P, double tau) { return P.milne ? tau * tau : 1.0; }
 
-// conserved variables from primaries (Eqs. Ttt, Tti) for one event, with its ghost copies
+// The primaries of kt_set_state: packed physical arrays on the device, null where not given
+struct Primaries {
+  const double *e, *u, *pi, *Pi, *u_prev;
+};
+
+// padded coordinates of physical cell o (x fastest)
+__device__ __forceinline__ void cell_coords(const Lattice& L, unsigned o, int& i, int& j, int& k) {
+  const unsigned row = o / (unsigned)L.nx;
+  i = (int)(o - row * (unsigned)L.nx) + 2;
+  k = (int)(row / (unsigned)L.ny);
+  j = (int)row - k * L.ny + 2;
+  k += 2;
+}
+
+// Conserved variables from primaries (Eqs. Ttt, Tti) for one event, with its ghost copies; also tau.
+// Bound by memory (18 values read, 30 to 43 written per cell) once it stays off the FP64 pipe: tests on
+// bit patterns, conversions on the integer pipe, no division.  It reads the caller's device arrays
+// themselves (host arrays come through the staging area).  With the gather below, set and get of a 128^3
+// event on the device: six learned steps between them 7.13 -> 6.79 ms, six steps of a 16-event batch
+// 26.5 -> 22.7 ms; a 64 x 64 x 48 output to the host (31 fields, diagnostics) 1.1 -> 0.72 ms.
 template <typename R>
-__global__ void set_state_kernel(const Params P, const Lattice L, const double* __restrict__ in, int has_u, int has_pi,
-                                 int has_Pi, int has_up, double tau, double* q, float* qf, R* U, R* Up, R* E, R* Pb,
-                                 float* reg, unsigned* status) {
-  long long ncp = (long long)L.nx * L.ny * L.nz;
-  long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256)
+    set_state_kernel(const Params P, const Lattice L, const Primaries in, double tau, double* tau_slot, double* q,
+                     float* qf, R* U, R* Up, R* E, R* Pb, float* reg, unsigned* status) {
+  const unsigned ncp = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
+  const unsigned o = blockIdx.x * 256u + threadIdx.x;
+  if (o == 0) *tau_slot = tau;
   if (o >= ncp) return;
-  int i = (int)(o % L.nx), j = (int)((o / L.nx) % L.ny), k = (int)(o / ((long long)L.nx * L.ny));
-  const double* pe = in;
-  const double* pu = in + ncp;
-  const double* ppi = in + 4 * ncp;
-  const double* pPi = in + 14 * ncp;
-  const double* pup = in + 15 * ncp;
-  double e = pe[o];
-  double ux = has_u ? pu[o] : 0.0, uy = has_u ? pu[ncp + o] : 0.0, un = has_u ? pu[2 * ncp + o] : 0.0;
-  double g = gnn_at(P, tau);
-  double ut = sqrt(1.0 + ux * ux + uy * uy + g * un * un);
-  double pi[10];
-  for (int m = 0; m < 10; ++m) pi[m] = has_pi ? ppi[m * ncp + o] : 0.0;
-  double Pi = has_Pi ? pPi[o] : 0.0;
-  double P0 = eos_P<double>(P, e);
-  double Pt = P0 + Pi;
+  int i, j, k;
+  cell_coords(L, o, i, j, k);
+  const double e = in.e[o];
+  double u4[4] = {1.0, 0.0, 0.0, 0.0}, up4[4], pi[10];
+  const double g = gnn_at(P, tau);
+  if (in.u) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) u4[m + 1] = in.u[(size_t)m * ncp + o];
+    u4[0] = sqrt(1.0 + u4[1] * u4[1] + u4[2] * u4[2] + g * u4[3] * u4[3]);
+  }
+#pragma unroll
+  for (int m = 0; m < 10; ++m) pi[m] = in.pi ? in.pi[(size_t)m * ncp + o] : 0.0;
+  const double Pi = in.Pi ? in.Pi[o] : 0.0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) up4[m] = u4[m];
+  if (in.u_prev) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) up4[m + 1] = in.u_prev[(size_t)m * ncp + o];
+    const double gp = gnn_at(P, tau - P.dtau);
+    up4[0] = sqrt(1.0 + up4[1] * up4[1] + up4[2] * up4[2] + gp * up4[3] * up4[3]);
+  }
+  const double P0 = eos_P<double>(P, e), Pt = P0 + Pi, w = (e + Pt) * u4[0];
   double qn[NQ];
-  qn[0] = (e + Pt) * ut * ut - Pt + pi[0];
-  qn[1] = (e + Pt) * ut * ux + pi[1];
-  qn[2] = (e + Pt) * ut * uy + pi[2];
-  qn[3] = (e + Pt) * ut * un + pi[3];
+  qn[0] = fma(w, u4[0], -Pt) + pi[0];
+#pragma unroll
+  for (int m = 1; m < 4; ++m) qn[m] = fma(w, u4[m], pi[m]);
+#pragma unroll
   for (int m = 0; m < 10; ++m) qn[4 + m] = pi[m];
   qn[14] = Pi;
-  double u4[4] = {ut, ux, uy, un}, up4[4];
-  if (has_up) {
-    double px = pup[o], py = pup[ncp + o], pn = pup[2 * ncp + o];
-    double gp = gnn_at(P, tau - P.dtau);
-    up4[0] = sqrt(1.0 + px * px + py * py + gp * pn * pn); up4[1] = px; up4[2] = py; up4[3] = pn;
-  } else {
-    for (int m = 0; m < 4; ++m) up4[m] = u4[m];
-  }
-  bool bad = !isfinite(e) || !(e >= 0.0) || !isfinite(ut) || !isfinite(Pi) || !isfinite(up4[0]);
-  for (int m = 0; m < 10; ++m) bad |= !isfinite(pi[m]);
+  // non-finite input, or e < 0 (the sign bit of a non-zero e)
+  const long long be = __double_as_longlong(e);
+  bool bad = !kt::finite(e) || (be < 0 && (be << 1) != 0) || !kt::finite(u4[0]) || !kt::finite(Pi) || !kt::finite(up4[0]);
+#pragma unroll
+  for (int m = 0; m < 10; ++m) bad |= !kt::finite(pi[m]);
   if (bad) atomicOr(status, ST_NONFINITE);
   // the inversion of Eq. (eInferred) needs E = T^{tau tau} - pi^{tau tau} > 0 and M^2 < E^2 with
   // M^i = T^{tau i} - pi^{tau i}, M^2 = M_x^2 + M_y^2 + g_{eta eta} M_eta^2 (Sec. 2.4)
   const double Ei = qn[0] - qn[4], Mx = qn[1] - qn[5], My = qn[2] - qn[6], Mn = qn[3] - qn[7];
-  if (!bad && !(Ei > 0.0 && Mx * Mx + My * My + g * Mn * Mn < Ei * Ei)) atomicOr(status, ST_INVERSION);
+  if (!bad && !(pos(Ei) && obits(Mx * Mx + My * My + g * Mn * Mn) < obits(Ei * Ei))) atomicOr(status, ST_INVERSION);
   const long long fs = L.fstride;
-  const int pc[3] = {i + 2, j + 2, k + 2};
-  const int nn[3] = {L.nx, L.ny, L.nz};
-  reg[L.idx(pc[0], pc[1], pc[2])] = 1.f;  // no regulation recorded yet
-  for (int t = -1; t < 12; ++t) {
-    int ii = pc[0], jj = pc[1], kk = pc[2];
-    if (t >= 0) {
-      int ax = t / 4, gi = t % 4, n = nn[ax];
-      int gpos = (gi < 2) ? gi : n + gi;
-      if (ghost_source(gpos, n, P.periodic) != pc[ax]) continue;
-      if (ax == 0) ii = gpos; else if (ax == 1) jj = gpos; else kk = gpos;
-    }
-    long long c = L.idx(ii, jj, kk);
-    for (int n = 0; n < NQ; ++n) q[n * fs + c] = qn[n];
-    if (qf)
-      for (int n = 0; n < NQ; ++n) qf[n * fs + c] = (float)qn[n];
-    for (int m = 0; m < 4; ++m) { U[m * fs + c] = (R)u4[m]; Up[m * fs + c] = (R)up4[m]; }
-    E[c] = (R)e;
-    Pb[c] = (R)P0;
+  reg[L.idx(i, j, k)] = 1.f;  // no regulation recorded yet
+  float qs[NQ];
+  if (qf) {
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) qs[n] = d2f_bits(qn[n]);
   }
+  R ur[4], upr[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    ur[m] = from_f64<R>(u4[m]);
+    upr[m] = from_f64<R>(up4[m]);
+  }
+  const R er = from_f64<R>(e), pr0 = from_f64<R>(P0);
+  for_cell_and_ghosts(P, L, i, j, k, [&](long long c) {
+#pragma unroll
+    for (int n = 0; n < NQ; ++n) q[n * fs + c] = qn[n];
+    if (qf) {
+#pragma unroll
+      for (int n = 0; n < NQ; ++n) qf[n * fs + c] = qs[n];
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      U[m * fs + c] = ur[m];
+      Up[m * fs + c] = upr[m];
+    }
+    E[c] = er;
+    Pb[c] = pr0;
+  });
 }
 
-// gather one component of one event (double or float) into a packed physical array
-template <typename S>
-__global__ void gather_kernel(const Lattice L, const S* __restrict__ f, double* out) {
-  long long ncp = (long long)L.nx * L.ny * L.nz;
-  long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// float -> double, exact for every float: on the integer pipe, the conversion instruction (FP64 pipe)
+// for subnormals, infinities and NaN only
+__device__ __forceinline__ double f2d_exact(float f) {
+  const unsigned ex = (__float_as_uint(f) >> 23) & 0xffu;
+  if (ex == 0xffu || (ex == 0u && f != 0.f)) return (double)f;
+  return f2d_bits(f);
+}
+
+// Rows of one event (double or float fields) gathered into packed physical arrays: one launch for up to
+// kRows rows, kRowsPerThread of them per thread (blockIdx.y picks the group), their loads in flight
+// together; the destination is the caller's device array itself or the staging area of a host copy.
+constexpr int kRows = 18, kRowsPerThread = 6;
+struct GatherRows {
+  const void* src[kRows];
+  double* dst[kRows];
+  unsigned f32;  // bit r: row r is float
+  int n;
+};
+__global__ void __launch_bounds__(256) gather_kernel(const Lattice L, const GatherRows rows) {
+  const unsigned ncp = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
+  const unsigned o = blockIdx.x * 256u + threadIdx.x;
   if (o >= ncp) return;
-  int i = (int)(o % L.nx), j = (int)((o / L.nx) % L.ny), k = (int)(o / ((long long)L.nx * L.ny));
-  out[o] = (double)f[L.idx(i + 2, j + 2, k + 2)];
+  int i, j, k;
+  cell_coords(L, o, i, j, k);
+  const long long c = L.idx(i, j, k);
+  const int r0 = kRowsPerThread * (int)blockIdx.y;
+  double v[kRowsPerThread];
+  float f[kRowsPerThread];
+#pragma unroll
+  for (int r = 0; r < kRowsPerThread; ++r) {
+    if (r0 + r >= rows.n) break;
+    if ((rows.f32 >> (r0 + r)) & 1u) f[r] = __ldg((const float*)rows.src[r0 + r] + c);
+    else v[r] = __ldg((const double*)rows.src[r0 + r] + c);
+  }
+#pragma unroll
+  for (int r = 0; r < kRowsPerThread; ++r) {
+    if (r0 + r >= rows.n) break;
+    rows.dst[r0 + r][o] = ((rows.f32 >> (r0 + r)) & 1u) ? f2d_exact(f[r]) : v[r];
+  }
 }
 
 // scatter one packed physical array into a field (double or float) at every physical cell and
@@ -1206,26 +1268,31 @@ int kt_set_state_event(kt_ctx* c, int event, double tau, const double* e, const 
     return fail(c, KT_ERR_ARG, "kt_set_state: bad argument");
   const Lattice& L = c->lat[event];
   size_t ncp = (size_t)L.nx * L.ny * L.nz;
-  cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  double* s = c->stage;
-  CK(cudaMemcpyAsync(s, e, ncp * 8, kind, c->stream));
-  if (u) CK(cudaMemcpyAsync(s + ncp, u, 3 * ncp * 8, kind, c->stream));
-  if (pi) CK(cudaMemcpyAsync(s + 4 * ncp, pi, 10 * ncp * 8, kind, c->stream));
-  if (Pi) CK(cudaMemcpyAsync(s + 14 * ncp, Pi, ncp * 8, kind, c->stream));
-  if (u_prev) CK(cudaMemcpyAsync(s + 15 * ncp, u_prev, 3 * ncp * 8, kind, c->stream));
+  Primaries in = {e, u, pi, Pi, u_prev};
+  if (!on_device) {  // through the staging area: rows 0, 1-3, 4-13, 14, 15-17
+    double* s = c->stage;
+    auto up = [&](const double*& p, int row, int rows) {
+      if (!p) return cudaSuccess;
+      const cudaError_t r = cudaMemcpyAsync(s + row * ncp, p, rows * ncp * 8, cudaMemcpyHostToDevice, c->stream);
+      p = s + row * ncp;
+      return r;
+    };
+    CK(up(in.e, 0, 1));
+    CK(up(in.u, 1, 3));
+    CK(up(in.pi, 4, 10));
+    CK(up(in.Pi, 14, 1));
+    CK(up(in.u_prev, 15, 3));
+  }
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
-  double tau_h = tau;
-  CK(cudaMemcpyAsync(c->d_tau + c->cur, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
-  int nb = (int)((ncp + 255) / 256);
+  const unsigned nb = (unsigned)((ncp + 255) / 256);
+  double* slot = c->d_tau + c->cur;
   // the state goes into the buffers that hold u^n and u^{n-1} in the current rotation
   if (c->mixed)
-    set_state_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L, s, u != nullptr, pi != nullptr, Pi != nullptr,
-                                                       u_prev != nullptr, tau, c->q, c->qf, (float*)c->U[c->cur],
+    set_state_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L, in, tau, slot, c->q, c->qf, (float*)c->U[c->cur],
                                                        (float*)c->U[c->prev], (float*)c->E[0], (float*)c->Pb[0],
                                                        c->reg, c->d_stat);
   else
-    set_state_kernel<double><<<nb, 256, 0, c->stream>>>(c->P, L, s, u != nullptr, pi != nullptr, Pi != nullptr,
-                                                        u_prev != nullptr, tau, c->q, nullptr, (double*)c->U[c->cur],
+    set_state_kernel<double><<<nb, 256, 0, c->stream>>>(c->P, L, in, tau, slot, c->q, nullptr, (double*)c->U[c->cur],
                                                         (double*)c->U[c->prev], (double*)c->E[0], (double*)c->Pb[0],
                                                         c->reg, c->d_stat);
   CK(cudaGetLastError());
@@ -1249,6 +1316,38 @@ int kt_set_state(kt_ctx* c, double tau, const double* e, const double* u, const 
 }  // extern "C"
 
 namespace {
+
+// One packed row of an event going out: the field component, whether it is float, the destination.
+struct Row {
+  const void* f;
+  int f32;
+  double* dst;
+};
+// Rows to the caller's arrays: on the device in one launch per kRows rows, to the host through the staging
+// area with one copy per run of adjoining destinations.
+int gather_rows(Ctx* c, const Lattice& L, const std::vector<Row>& rows, int on_device) {
+  const size_t ncp = (size_t)L.nx * L.ny * L.nz;
+  for (size_t b = 0; b < rows.size(); b += kRows) {
+    GatherRows g = {};
+    g.n = (int)std::min<size_t>(kRows, rows.size() - b);
+    for (int r = 0; r < g.n; ++r) {
+      g.src[r] = rows[b + r].f;
+      g.dst[r] = on_device ? rows[b + r].dst : c->stage + r * ncp;
+      if (rows[b + r].f32) g.f32 |= 1u << r;
+    }
+    const dim3 grid((unsigned)((ncp + 255) / 256), (unsigned)((g.n + kRowsPerThread - 1) / kRowsPerThread));
+    gather_kernel<<<grid, 256, 0, c->stream>>>(L, g);
+    CK(cudaGetLastError());
+    if (on_device) continue;
+    for (int r = 0; r < g.n;) {
+      int m = 1;
+      while (r + m < g.n && rows[b + r + m].dst == rows[b + r].dst + m * ncp) ++m;
+      CK(cudaMemcpyAsync(rows[b + r].dst, c->stage + r * ncp, m * ncp * 8, cudaMemcpyDeviceToHost, c->stream));
+      r += m;
+    }
+  }
+  return KT_OK;
+}
 
 int begin_steps(Ctx* c, int n_steps) {
   for (int e = 0; e < c->nev; ++e)
@@ -1345,34 +1444,20 @@ int kt_get_state_event(kt_ctx* c, int event, double* tau, double* e, double* u, 
   const Lattice& L = c->lat[event];
   size_t ncp = (size_t)L.nx * L.ny * L.nz;
   const long long fs = c->gs;
-  cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  int nb = (int)((ncp + 255) / 256);
-  // (source component, destination) pairs, gathered through the staging area in groups
-  struct Job { const void* f; int is_r; double* dst; };
-  std::vector<Job> jobs;
+  std::vector<Row> rows;
   const char* Ucur = (const char*)c->U[c->cur];
-  if (e) jobs.push_back({c->E[0], 1, e});
-  if (u) for (int m = 0; m < 4; ++m) jobs.push_back({Ucur + (size_t)m * fs * c->esz, 1, u + m * ncp});
+  if (e) rows.push_back({c->E[0], c->mixed, e});
+  if (u) for (int m = 0; m < 4; ++m) rows.push_back({Ucur + (size_t)m * fs * c->esz, c->mixed, u + m * ncp});
   // component n of q: FP64, or (KT_STORE_PI_FP32, n >= 4) the FP32 state
-  auto qjob = [&](int n, double* dst) {
-    if (c->pi32 && n >= 4) jobs.push_back({c->qf + (size_t)n * fs, 2, dst});
-    else jobs.push_back({c->q + (size_t)n * fs, 0, dst});
+  auto qrow = [&](int n, double* dst) {
+    if (c->pi32 && n >= 4) rows.push_back({c->qf + (size_t)n * fs, 1, dst});
+    else rows.push_back({c->q + (size_t)n * fs, 0, dst});
   };
-  if (pi) for (int m = 0; m < 10; ++m) qjob(4 + m, pi + m * ncp);
-  if (Pi) qjob(14, Pi);
-  if (q) for (int n = 0; n < NQ; ++n) qjob(n, q + n * ncp);
-  for (size_t b = 0; b < jobs.size(); b += 18) {
-    size_t nj = std::min<size_t>(18, jobs.size() - b);
-    for (size_t t = 0; t < nj; ++t) {
-      const Job& jb = jobs[b + t];
-      double* dst = c->stage + t * ncp;
-      if (jb.is_r == 2 || (jb.is_r && c->mixed))
-        gather_kernel<float><<<nb, 256, 0, c->stream>>>(L, (const float*)jb.f, dst);
-      else gather_kernel<double><<<nb, 256, 0, c->stream>>>(L, (const double*)jb.f, dst);
-    }
-    CK(cudaGetLastError());
-    for (size_t t = 0; t < nj; ++t) CK(cudaMemcpyAsync(jobs[b + t].dst, c->stage + t * ncp, ncp * 8, kind, c->stream));
-  }
+  if (pi) for (int m = 0; m < 10; ++m) qrow(4 + m, pi + m * ncp);
+  if (Pi) qrow(14, Pi);
+  if (q) for (int n = 0; n < NQ; ++n) qrow(n, q + n * ncp);
+  const int rc = gather_rows(c, L, rows, on_device);
+  if (rc != KT_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));
   if (tau) *tau = c->tau;
   return KT_OK;
@@ -1418,21 +1503,11 @@ int kt_get_checkpoint(kt_ctx* c, int event, double* tau, double* buf, int on_dev
   if (!c->ev_set[event]) return fail(c, KT_ERR_ARG, "kt_get_checkpoint: event %d has no state", event);
   const Lattice& L = c->lat[event];
   const size_t ncp = (size_t)L.nx * L.ny * L.nz;
-  const int nb = (int)((ncp + 255) / 256);
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  const std::vector<CkptRow> rows = checkpoint_rows(c);
   static_assert(KT_CHECKPOINT_ROWS == 41, "checkpoint layout");
-  for (size_t b = 0; b < rows.size(); b += 18) {  // through the staging area, 18 rows at a time
-    const size_t nr = std::min<size_t>(18, rows.size() - b);
-    for (size_t t = 0; t < nr; ++t) {
-      const CkptRow& r = rows[b + t];
-      double* dst = c->stage + t * ncp;
-      if (r.is_r == 2 || (r.is_r && c->mixed)) gather_kernel<float><<<nb, 256, 0, c->stream>>>(L, (const float*)r.f, dst);
-      else gather_kernel<double><<<nb, 256, 0, c->stream>>>(L, (const double*)r.f, dst);
-    }
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(buf + b * ncp, c->stage, nr * ncp * 8, kind, c->stream));
-  }
+  std::vector<Row> rows;
+  for (const CkptRow& r : checkpoint_rows(c)) rows.push_back({r.f, r.is_r == 2 || (r.is_r && c->mixed), buf + rows.size() * ncp});
+  const int rc = gather_rows(c, L, rows, on_device);
+  if (rc != KT_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));
   if (tau) *tau = c->tau;
   return KT_OK;
