@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/kt.h"
@@ -75,6 +76,7 @@ struct Ctx {
   uint32_t* d_mlp_packed = nullptr;
   Lattice* d_lat = nullptr;
   Tile* d_tiles = nullptr;
+  CUtensorMap map0[2] = {};        // mixed precision: the first event's maps of qf and qsf (kernel parameters)
   CUtensorMap* d_tmaps = nullptr;  // mixed precision: per event, the 4-d maps of qf (first nev) and qsf
   CUtensorMap* d_umaps = nullptr;  // mixed precision: per event, the kUpdMaps maps of the staged update
   int staged = 0;                  // the update kernels read their inputs staged by TMA
@@ -652,23 +654,37 @@ void launch_stage(Ctx* c, const StageIO<double>& io) {
   else go(stage_kernel<double, STAGE, false, true>);
 }
 
+Work make_work(Ctx* c) {
+  const Shape& s = kShapes[c->shape];
+  Work w;
+  w.L0 = c->lat[0];
+  w.tk = (unsigned)((w.L0.nz + s.z - 1) / s.z);
+  w.ti = (unsigned)((w.L0.nx + s.x - 1) / s.x);
+  w.ntiles = c->ntiles;
+  w.lats = c->d_lat;
+  w.tiles = c->d_tiles;
+  return w;
+}
+
+// f(integral constants...) with every run-time flag as a template argument
+template <typename F>
+void with_flags(F&& f) { f(); }
+template <typename F, typename... B>
+void with_flags(F&& f, bool b, B... rest) {
+  if (b) with_flags([&](auto... r) { f(std::true_type{}, r...); }, rest...);
+  else with_flags([&](auto... r) { f(std::false_type{}, r...); }, rest...);
+}
+
 // the right-hand-side kernel of a stage, with the minmod specialised when theta = 1
 template <int STAGE>
 void launch_rhs(Ctx* c, const StageIO<float>& io) {
   const Shape& s = kShapes[c->shape];
-  const dim3 blk(s.x, s.y, s.z);
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  const size_t sm = rhs_smem_bytes(s.x, s.y, s.z);
-  float* k = k_buf(c, STAGE);
-  const bool t1 = (c->P.theta == 1.0), inv = c->P.iface_invert;
-  if (t1 && !inv)
-    rhs_kernel<STAGE, true, false><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, k, c->d_lat, c->d_tiles, c->ntiles, maps);
-  else if (!inv)
-    rhs_kernel<STAGE, false, false><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, k, c->d_lat, c->d_tiles, c->ntiles, maps);
-  else if (t1)
-    rhs_kernel<STAGE, true, true><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, k, c->d_lat, c->d_tiles, c->ntiles, maps);
-  else
-    rhs_kernel<STAGE, false, true><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, k, c->d_lat, c->d_tiles, c->ntiles, maps);
+  with_flags([&](auto single, auto t1, auto inv) {
+    rhs_kernel<single.value, t1.value, inv.value>
+        <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
+            c->P, io, STAGE, k_buf(c, STAGE), make_work(c), c->map0[STAGE - 1], maps);
+  }, c->nev == 1, c->P.theta == 1.0, c->P.iface_invert != 0);
 }
 
 // every rhs kernel may take the dynamic shared memory of the largest tile shape
@@ -679,22 +695,13 @@ int allow_rhs_smem(Ctx* c) {
   auto set = [&](const void* f) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  set((const void*)rhs_kernel<1, true, false>);
-  set((const void*)rhs_kernel<1, false, false>);
-  set((const void*)rhs_kernel<1, true, true>);
-  set((const void*)rhs_kernel<1, false, true>);
-  set((const void*)rhs_kernel<2, true, false>);
-  set((const void*)rhs_kernel<2, false, false>);
-  set((const void*)rhs_kernel<2, true, true>);
-  set((const void*)rhs_kernel<2, false, true>);
-  set((const void*)fused_kernel<1, true, false, true>);
-  set((const void*)fused_kernel<1, true, false, false>);
-  set((const void*)fused_kernel<1, false, false, true>);
-  set((const void*)fused_kernel<1, false, false, false>);
-  set((const void*)fused_kernel<2, true, false, true>);
-  set((const void*)fused_kernel<2, true, false, false>);
-  set((const void*)fused_kernel<2, false, false, true>);
-  set((const void*)fused_kernel<2, false, false, false>);
+  for (int f = 0; f < 8; ++f) {
+    with_flags([&](auto a, auto b, auto d) {
+      set((const void*)rhs_kernel<a.value, b.value, d.value>);
+      set((const void*)fused_kernel<a.value, 1, b.value, d.value>);
+      set((const void*)fused_kernel<a.value, 2, b.value, d.value>);
+    }, (f & 1) != 0, (f & 2) != 0, (f & 4) != 0);
+  }
   if (e != cudaSuccess) return fail(c, KT_ERR_CUDA, "rhs shared memory: %s", cudaGetErrorString(e));
   bytes = 0;
   for (const auto& sh : kShapes) bytes = std::max(bytes, upd_smem_bytes(sh.x, sh.y, sh.z, 2));
@@ -721,36 +728,21 @@ void launch_update(Ctx* c, const UpdIO& uio) {
                                                                               c->ntiles, c->d_umaps, c->upd_nbuf);
     return;
   }
-  if (c->learned && c->pi32)
-    update_kernel<STAGE, true, true><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles, c->ntiles);
-  else if (c->learned)
-    update_kernel<STAGE, true, false><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles, c->ntiles);
-  else if (c->pi32)
-    update_kernel<STAGE, false, true><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles, c->ntiles);
-  else
-    update_kernel<STAGE, false, false><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles, c->ntiles);
+  with_flags([&](auto single, auto learned, auto pi32) {
+    update_kernel<single.value, STAGE, learned.value, pi32.value><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, make_work(c));
+  }, c->nev == 1, c->learned != 0, c->pi32 != 0);
 }
 
 // the fused stage kernel (right-hand side and update in one launch)
 template <int STAGE>
 void launch_fused(Ctx* c, const StageIO<float>& io, const UpdIO& uio) {
   const Shape& s = kShapes[c->shape];
-  const dim3 blk(s.x, s.y, s.z);
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  const size_t sm = rhs_smem_bytes(s.x, s.y, s.z);
-  const bool t1 = (c->P.theta == 1.0);
-  if (t1 && c->learned)
-    fused_kernel<STAGE, true, false, true><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, uio, c->d_lat, c->d_tiles,
-                                                                               c->ntiles, maps);
-  else if (t1)
-    fused_kernel<STAGE, true, false, false><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, uio, c->d_lat, c->d_tiles,
-                                                                                c->ntiles, maps);
-  else if (c->learned)
-    fused_kernel<STAGE, false, false, true><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, uio, c->d_lat, c->d_tiles,
-                                                                                c->ntiles, maps);
-  else
-    fused_kernel<STAGE, false, false, false><<<c->grid_rhs, blk, sm, c->stream>>>(c->P, io, uio, c->d_lat, c->d_tiles,
-                                                                                 c->ntiles, maps);
+  with_flags([&](auto single, auto t1, auto learned) {
+    fused_kernel<single.value, STAGE, t1.value, learned.value>
+        <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
+            c->P, io, uio, make_work(c), c->map0[STAGE - 1], maps);
+  }, c->nev == 1, c->P.theta == 1.0, c->learned != 0);
 }
 
 template <int STAGE>
@@ -867,6 +859,8 @@ int encode_tensor_maps(Ctx* c) {
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return fail(c, KT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for event %d", (int)r, e);
     }
+  c->map0[0] = maps[0];
+  c->map0[1] = maps[c->nev];
   CK(cudaMemcpyAsync(c->d_tmaps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, c->stream));
   // the staged update's boxes: the tile's cells in y and eta, bx + 4 cells in x from the tile's
   // padded x, for q (FP64: 8 components, and 1), k_1, k_2 and the FP32 copy of q (15 components)
@@ -931,15 +925,15 @@ int select_shape(Ctx* c, int cand) {
   const Shape& sh = kShapes[shape];
   auto grid = [&](int cap) { return one_per_tile ? c->ntiles : std::max(1, std::min(cap, c->ntiles)); };
   const size_t rsm = rhs_smem_bytes(sh.x, sh.y, sh.z);
-  c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<1, true, false, true>, sh, rsm)
-                              : occupancy_blocks(rhs_kernel<1, true, false>, sh, rsm));
+  c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<true, 1, true, true>, sh, rsm)
+                              : occupancy_blocks(rhs_kernel<true, true, false>, sh, rsm));
   if (c->staged) {
     const size_t usm = upd_smem_bytes(sh.x, sh.y, sh.z, c->upd_nbuf);
     c->grid_upd = grid(c->learned ? occupancy_blocks(update_staged_kernel<2, true>, sh, usm)
                                   : occupancy_blocks(update_staged_kernel<2, false>, sh, usm));
   } else {
-    c->grid_upd = grid(c->learned ? occupancy_blocks(update_kernel<1, true, false>, sh)
-                                  : occupancy_blocks(update_kernel<1, false, false>, sh));
+    c->grid_upd = grid(c->learned ? occupancy_blocks(update_kernel<true, 1, true, false>, sh)
+                                  : occupancy_blocks(update_kernel<true, 1, false, false>, sh));
   }
   c->grid_blocks = c->grid_rhs;
   c->cand = cand;

@@ -41,6 +41,26 @@ struct UpdIO {
   const float* z_net;       // learned start: the network's output z per cell for the step (mlp_start_kernel)
 };
 
+// The work of a launch.  A batch walks a table of (event, tile) entries, and reads the entry, then its
+// lattice, then the data: two dependent loads before a block's first useful one.  A single event
+// (SINGLE) needs neither: its lattice is a kernel parameter, so strides and bounds come from the constant
+// bank instead of registers, and tile t follows from t by two divisions (tiles run along eta, then x, y).
+// 128^3 step, learned start: split launches 1.018 -> 0.938 ms, fused 1.047 -> 0.931 ms; FP32 pi storage,
+// 96 x 96 x 64: 0.328 -> 0.302 ms.
+struct Work {
+  Lattice L0;             // the single event's lattice
+  unsigned tk, ti;        // its tiles along eta and x
+  int ntiles;
+  const Lattice* lats;    // batches
+  const Tile* tiles;
+};
+template <bool SINGLE>
+__device__ __forceinline__ Tile tile_at(const Work& W, int t) {
+  if constexpr (!SINGLE) return W.tiles[t];
+  const unsigned a = (unsigned)t / W.tk, k = (unsigned)t - a * W.tk, j = a / W.ti, i = a - j * W.ti;
+  return Tile{0, (int)(i * blockDim.x), (int)(j * blockDim.y), (int)(k * blockDim.z)};
+}
+
 // inversion inputs of q: T^{tau mu} (0-3), pi^{tau mu} (4-7), Pi (14)
 __device__ __forceinline__ constexpr bool inversion_component(int n) { return n < 8 || n == 14; }
 
@@ -65,10 +85,11 @@ __host__ __device__ constexpr int rhs_smem_bytes(int tx, int ty, int tz) {  // t
 // warps; 96 for the stage-2 update, which holds all 15 FP64 components.  Each measured faster than
 // the compiler's unconstrained choice; for the update kernels, caps of 64-80 (stage 1) and 72-96
 // (stage 2) all measure within 0.5% of each other (latency-bound: more warps, more spills).
-template <int STAGE, bool TH1, bool IFACE>
+// map0: the single event's tensor map, as a kernel parameter (no fence, no fetch through L2); tmaps: a batch's
+template <bool SINGLE, bool TH1, bool IFACE>
 __global__ void __maxnreg__(96)
-    rhs_kernel(const Params P, const StageIO<float> io, float* __restrict__ k_out, const Lattice* __restrict__ lats,
-               const Tile* __restrict__ tiles, int ntiles, const CUtensorMap* __restrict__ tmaps) {
+    rhs_kernel(const Params P, const StageIO<float> io, int stage, float* __restrict__ k_out, const Work W,
+               const __grid_constant__ CUtensorMap map0, const CUtensorMap* __restrict__ tmaps) {
   extern __shared__ __align__(128) float s_raw[];
   __shared__ alignas(8) uint64_t s_bar[2];
   float* const s_q = s_raw + ((32u - ((smem_u32(s_raw) >> 2) & 31u)) & 31u);  // TMA wants 128-byte buffers
@@ -82,13 +103,12 @@ __global__ void __maxnreg__(96)
     mbar_init(&s_bar[1], 1);
     fence_barrier_init();
   }
-  __syncthreads();
 
   float amax = 0.f;
   bool bad = false;
   unsigned issued = 0, done = 0;  // TMA copies issued and waited for (the same in every thread)
   const double tau_n = io.d_tau[0];
-  const CellGeom<float> G = cell_geom<float>(P, (STAGE == 1) ? tau_n : tau_n + P.dtau);
+  const CellGeom<float> G = cell_geom<float>(P, (stage == 1) ? tau_n : tau_n + P.dtau);
   const float th = pr<float>(P).theta;
   const int sy = bx, sz = bx * by;
   const int own = ((int)threadIdx.z + 2) * sz + ((int)threadIdx.y + 2) * sy + (int)threadIdx.x + 2;
@@ -100,16 +120,17 @@ __global__ void __maxnreg__(96)
   };
 
   int t0, t1;
-  tile_range(ntiles, t0, t1);
+  tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tiles[t];
-    const Lattice L = lats[tl.event];
-    const CUtensorMap* map = tmaps + tl.event;
-    if (__syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
+    const Tile tl = tile_at<SINGLE>(W, t);
+    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
+    const CUtensorMap* map = SINGLE ? &map0 : tmaps + tl.event;
+    if (t > t0 && __syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
     if (tid == 0) {
-      fence_tensormap_acquire(map);
+      if (!SINGLE) fence_tensormap_acquire(map);
       stage_group(map, tl, 0);
     }
+    if (t == t0) __syncthreads();  // the barriers are initialised
     ++issued;
 
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
@@ -443,17 +464,15 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
   });
 }
 
-template <int STAGE, bool LEARNED, bool PI32>
-__global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
-    update_kernel(const Params P, const UpdIO io, const Lattice* __restrict__ lats, const Tile* __restrict__ tiles,
-                  int ntiles) {
+template <bool SINGLE, int STAGE, bool LEARNED, bool PI32>
+__global__ void __maxnreg__(STAGE == 1 ? 72 : 96) update_kernel(const Params P, const UpdIO io, const Work W) {
   unsigned st = 0, nit = 0, nreg = 0, nfb = 0;
   const double tau_out = io.d_tau[0] + P.dtau;
   int t0, t1;
-  tile_range(ntiles, t0, t1);
+  tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tiles[t];
-    const Lattice L = lats[tl.event];
+    const Tile tl = tile_at<SINGLE>(W, t);
+    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
     const UpdInGlobal in{io, L.fstride, L.idx(i + 2, j + 2, k + 2)};
     update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau_out, st, nit, nreg, nfb);
@@ -634,10 +653,11 @@ struct UpdInFused {
 
 // 128 registers (16 warps of 128-thread tiles per SM): with the rhs kernel's 96 the two phases
 // spilled 500 bytes per thread and the launch ran 10% slower.
-template <int STAGE, bool TH1, bool IFACE, bool LEARNED>
+template <bool SINGLE, int STAGE, bool TH1, bool LEARNED>
 __global__ void __maxnreg__(128)
-    fused_kernel(const Params P, const StageIO<float> io, const UpdIO uio, const Lattice* __restrict__ lats,
-                 const Tile* __restrict__ tiles, int ntiles, const CUtensorMap* __restrict__ tmaps) {
+    fused_kernel(const Params P, const StageIO<float> io, const UpdIO uio, const Work W,
+                 const __grid_constant__ CUtensorMap map0, const CUtensorMap* __restrict__ tmaps) {
+  constexpr bool IFACE = false;  // (root-finds of face states run in the split layout)
   extern __shared__ __align__(128) float s_raw[];
   __shared__ alignas(8) uint64_t s_bar[2];
   float* const s_q = s_raw + ((32u - ((smem_u32(s_raw) >> 2) & 31u)) & 31u);  // TMA wants 128-byte buffers
@@ -652,7 +672,6 @@ __global__ void __maxnreg__(128)
     mbar_init(&s_bar[1], 1);
     fence_barrier_init();
   }
-  __syncthreads();
 
   float amax = 0.f;
   bool bad = false;
@@ -672,16 +691,17 @@ __global__ void __maxnreg__(128)
   };
 
   int t0, t1;
-  tile_range(ntiles, t0, t1);
+  tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tiles[t];
-    const Lattice L = lats[tl.event];
-    const CUtensorMap* map = tmaps + tl.event;
-    if (__syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
+    const Tile tl = tile_at<SINGLE>(W, t);
+    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
+    const CUtensorMap* map = SINGLE ? &map0 : tmaps + tl.event;
+    if (t > t0 && __syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
     if (tid == 0) {
-      fence_tensormap_acquire(map);
+      if (!SINGLE) fence_tensormap_acquire(map);
       stage_group(map, tl, 0);
     }
+    if (t == t0) __syncthreads();  // the barriers are initialised
     ++issued;
 
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
