@@ -70,6 +70,7 @@ struct Ctx {
   EosSeg<float>* seg_f = nullptr;
   RootSeg* seg_r = nullptr;
   RootSegM* seg_m = nullptr;
+  FaceSeg* seg_face = nullptr;
   double* d_tau = nullptr;  // three slots, used in rotation with the u buffers: tau^n is in slot cur
   unsigned* d_stat = nullptr;
   float* d_mlp = nullptr;
@@ -204,6 +205,7 @@ size_t state_bytes(const std::vector<Lattice>& lat, long long gs, size_t max_cel
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(EosSeg<float>), 256);
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(RootSeg), 256);
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(RootSegM), 256);
+  b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(FaceSeg), 256);
   b += 256;                                    // tau
   b += 256;                                    // stats
   b += align_up(KT_MLP_NPARAM * 4, 256);       // MLP weights
@@ -544,8 +546,11 @@ __global__ void diag_kernel(const Params P, const Lattice L, const StageIO<R> io
   R uc[4];
   cell_faces<R, false, false>(P, L, io, c, u_global(L, io, c), G, dq, uc, du, dv, amax, Fx, Fy, Fz);
   cell_sources<R, true>(P, L, io, c, G, uc, du, dv, dq, dg);
-  for (int m = 0; m < 6; ++m) out[m * ncp + o] = to_f64<R>(dg[m]);
-  out[6 * ncp + o] = f2d_bits(reg[c]);
+  for (int m = 0; m < 6; ++m) {
+    if constexpr (sizeof(R) == 4) out[m * ncp + o] = f2d_exact(dg[m]);  // a quotient may be infinite
+    else out[m * ncp + o] = dg[m];
+  }
+  out[6 * ncp + o] = f2d_bits(reg[c]);  // (finite)
 }
 
 // training samples of the learned start: features as the stage kernel forms them, the exact
@@ -1182,6 +1187,7 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->seg_f = (EosSeg<float>*)carve(nseg * sizeof(EosSeg<float>));
   c->seg_r = (RootSeg*)carve(nseg * sizeof(RootSeg));
   c->seg_m = (RootSegM*)carve(nseg * sizeof(RootSegM));
+  c->seg_face = (FaceSeg*)carve(nseg * sizeof(FaceSeg));
   c->d_tau = (double*)carve(256);
   c->d_stat = (unsigned*)carve(256);
   c->d_mlp = (float*)carve(KT_MLP_NPARAM * 4);
@@ -1205,6 +1211,7 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   P.seg_f = c->seg_f;
   P.seg_r = c->seg_r;
   P.seg_m = c->seg_m;
+  P.seg_face = c->seg_face;
 
   CK(cudaMemsetAsync(qq, 0, 30 * fs * 8, c->stream));
   CK(cudaMemsetAsync(ep, 0, 4 * fs * c->esz, c->stream));
@@ -1233,6 +1240,11 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
     CK(cudaMemcpyAsync(c->seg_f, sf.data(), sf.size() * sizeof(sf[0]), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->seg_r, sr.data(), sr.size() * sizeof(sr[0]), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->seg_m, sm.data(), sm.size() * sizeof(sm[0]), cudaMemcpyHostToDevice, c->stream));
+    std::vector<FaceSeg> sface(sr.size());
+    for (size_t i = 0; i < sr.size(); ++i)
+      sface[i] = FaceSeg{(float)sr[i].e0, (float)sr[i].e1, (float)sr[i].P0, (float)sr[i].a1,
+                         (float)sr[i].a2, (float)sr[i].a3, 0.f,             0.f};
+    CK(cudaMemcpyAsync(c->seg_face, sface.data(), sface.size() * sizeof(FaceSeg), cudaMemcpyHostToDevice, c->stream));
   }
   if (o.mlp_weights) {
     CK(cudaMemcpyAsync(c->d_mlp, o.mlp_weights, KT_MLP_NPARAM * 4, cudaMemcpyHostToDevice, c->stream));

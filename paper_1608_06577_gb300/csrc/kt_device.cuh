@@ -75,6 +75,11 @@ struct alignas(64) RootSegM {
   float b3, unused0, unused1, unused2;
 };
 
+// The single-precision record of the same interval for the face root-finds: P0 in d = e - e0
+struct alignas(32) FaceSeg {
+  float e0, e1, P0, a1, a2, a3, unused0, unused1;
+};
+
 struct Coef {
   int kind;       // 0 const, 1 gauss
   double c0, c1, c2;
@@ -109,6 +114,7 @@ struct Params {
   const EosSeg<double>* seg_d;
   const EosSeg<float>* seg_f;
   const RootSeg* seg_r;
+  const FaceSeg* seg_face;  // the same intervals for the face root-finds (KT_IFACE_INVERT, FP32)
   const RootSegM* seg_m;  // the same intervals for the mixed-precision root-find
   Coef eta, zeta;
   int shear_on, bulk_on;
@@ -357,18 +363,15 @@ __device__ __forceinline__ R ln_zeta_over_s(const Params& P, R T) {
 
 // Conversions between float and double on the integer pipe.  On GB300 the F2F conversion
 // instructions issue on the FP64 pipe, which has 1/64 of the FP32 rate; these bit-level
-// versions leave it free.  float -> double is exact (subnormal floats flush to zero);
+// versions leave it free.  float -> double is exact (subnormal floats flush to zero; infinities and NaN
+// become finite values beyond 2^127, which no FP32 state survives: they round back to infinity);
 // double -> float rounds to nearest even (results below the smallest normal float flush to
 // zero; overflow, infinity and NaN give infinity, so a non-finite input stays non-finite).
 __device__ __forceinline__ double f2d_bits(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned ex = (b >> 23) & 0xffu;
-  const unsigned s = b & 0x80000000u;
-  const unsigned m = b & 0x7fffffu;
-  const unsigned ed = (ex == 0xffu) ? 0x7ffu : ex + 896u;
-  const unsigned hi = (ex == 0u) ? s : (s | (ed << 20) | (m >> 3));
-  const unsigned lo = (ex == 0u) ? 0u : (m << 29);
-  return __hiloint2double((int)hi, (int)lo);
+  const int b = __float_as_int(f);
+  const int hi = ((b >> 3) & (int)0x8fffffff) + 0x38000000;  // sign, exponent rebiased by 896, mantissa's top
+  const bool normal = (b & 0x7f800000) != 0;
+  return __hiloint2double(normal ? hi : (b & (int)0x80000000), normal ? (int)((unsigned)b << 29) : 0);
 }
 
 __device__ __forceinline__ float d2f_bits(double d) {

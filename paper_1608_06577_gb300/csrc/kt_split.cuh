@@ -81,10 +81,10 @@ __host__ __device__ constexpr int rhs_smem_bytes(int tx, int ty, int tz) {  // t
   return 4 * (2 * rhs_buffer_floats(tx, ty, tz) + 32);
 }
 
-// Register caps: 96 (rhs) lets 20 warps of 128-thread tiles share an SM; 72 (stage-1 update) 28
-// warps; 96 for the stage-2 update, which holds all 15 FP64 components.  Each measured faster than
-// the compiler's unconstrained choice; for the update kernels, caps of 64-80 (stage 1) and 72-96
-// (stage 2) all measure within 0.5% of each other (latency-bound: more warps, more spills).
+// Register caps: 96 (rhs) lets 20 warps of 128-thread tiles share an SM; 64 (stage-1 update) 32 warps;
+// 80 (stage-2 update, which holds all 15 FP64 components) 24.  Each measured faster than the compiler's
+// unconstrained choice; 128^3 step in the split layout: update caps 64/80 0.954 ms, 72/96 0.961 ms, 80/104
+// with rhs 80 1.023 ms.
 // map0: the single event's tensor map, as a kernel parameter (no fence, no fetch through L2); tmaps: a batch's
 template <bool SINGLE, bool TH1, bool IFACE>
 __global__ void __maxnreg__(96)
@@ -465,7 +465,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
 }
 
 template <bool SINGLE, int STAGE, bool LEARNED, bool PI32>
-__global__ void __maxnreg__(STAGE == 1 ? 72 : 96) update_kernel(const Params P, const UpdIO io, const Work W) {
+__global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, const UpdIO io, const Work W) {
   unsigned st = 0, nit = 0, nreg = 0, nfb = 0;
   const double tau_out = io.d_tau[0] + P.dtau;
   int t0, t1;
