@@ -647,12 +647,26 @@ UpdIO make_uio(Ctx* c, int stage) {
   return u;
 }
 
+// Two blocks of stage_team_kernel are resident per SM: beyond 304 strips a second wave doubles its time.
+// 12 viscous steps (us), one warp / four warps per strip: 64 strips 1672 / 1081, 480 strips 1692 / 2292;
+// the Gubser grid (256 strips, 20 steps) 3390 / 2255, the shock tube (7 strips, 80 steps) 3503 / 2955.
+constexpr int kTeamStrips = 2 * 152;
+
 template <int STAGE>
 void launch_stage(Ctx* c, const StageIO<double>& io) {
   const bool t1 = (c->P.theta == 1.0), inv = c->P.iface_invert;
   auto go = [&](auto kernel) {
     kernel<<<c->grid_blocks, 32, 0, c->stream>>>(c->P, io, c->lat[0], c->d_lat, c->d_tiles, c->nev);
   };
+  // up to kTeamStrips strips the four-warp kernel is the faster one: see there
+  if (!inv && c->grid_blocks <= kTeamStrips) {
+    auto team = [&](auto kernel) {
+      kernel<<<c->grid_blocks, 128, 0, c->stream>>>(c->P, io, c->lat[0], c->d_lat, c->d_tiles, c->nev);
+    };
+    if (t1) team(stage_team_kernel<double, STAGE, true>);
+    else team(stage_team_kernel<double, STAGE, false>);
+    return;
+  }
   if (t1 && !inv) go(stage_kernel<double, STAGE, true, false>);
   else if (!inv) go(stage_kernel<double, STAGE, false, false>);
   else if (t1) go(stage_kernel<double, STAGE, true, true>);

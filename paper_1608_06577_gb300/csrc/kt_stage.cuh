@@ -182,12 +182,12 @@ __device__ __forceinline__ UGlobal<R> u_global(const Lattice& L, const StageIO<R
 
 // Velocity part of direction D: limited face states of u^tau and u^d and their ratio v^d
 // (Sec. 3.1), the local speeds a = max(|v^p|, |v^m|) (Eq. ax), the central differences
-// d_d u^mu and d_d v^d, and the pressure part of S_c (App. B):
+// d_d u^mu and v^d_{i+1} - v^d_{i-1}, and the pressure part of S_c (App. B):
 // -d_d (v^d P delta^nu_tau - g^{d nu} P), P = P0 + Pi.
 template <typename R, int D, bool TH1, bool IFACE, typename UA>
 __device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
                                            const UA& ua, const R (&uc)[4], R inv_gnn, R sfac, R (&dq)[NQ],
-                                           R (&du)[4][4], R& dv, float& amax, Faces<R>& F) {
+                                           R (&du)[4][4], R& dvd, float& amax, Faces<R>& F) {
   const long long fs = L.fstride;
   const int s = (D == 0) ? 1 : ((D == 1) ? L.pitch : (int)L.plane);  // in the field arrays
   const int us = (D == 0) ? 1 : ((D == 1) ? ua.sy : ua.sz);           // where u is read
@@ -231,16 +231,16 @@ __device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, co
 #pragma unroll
   for (int m = 0; m < 4; ++m) du[D + 1][m] = rmul(up1[m] - um1[m], hinv);
   const R vpl = vdiv(up1[D + 1], up1[0]), vmi = vdiv(um1[D + 1], um1[0]);
-  dv += (vpl - vmi) * hinv;
-  F.vpl_h = vpl * hinv;
-  F.vmi_h = vmi * hinv;
+  dvd = vpl - vmi;
+  F.vpl_h = rmul(vpl, hinv);
+  F.vmi_h = rmul(vmi, hinv);
   F.s = s;
 
   const R* q = io.qr_in;
   const R Ppl = ld<R>(io.p_in, c + s) + ld<R>(q + 14 * fs, c + s);
   const R Pmi = ld<R>(io.p_in, c - s) + ld<R>(q + 14 * fs, c - s);
-  dq[0] -= Ppl * F.vpl_h - Pmi * F.vmi_h;
-  dq[D + 1] -= ((D == 2) ? (Ppl - Pmi) * inv_gnn : (Ppl - Pmi)) * hinv;
+  dq[0] -= fma(Ppl, F.vpl_h, -(Pmi * F.vmi_h));
+  dq[D + 1] -= rmul((D == 2) ? (Ppl - Pmi) * inv_gnn : (Ppl - Pmi), hinv);
 }
 
 // An axis of one cell: its neighbours are copies of the cell, so every difference along it vanishes; the
@@ -420,54 +420,73 @@ template <typename R>
 struct Stencil13 {
   R a0, v[3][4];  // the cell and, per axis, i-2, i-1, i+1, i+2
 };
+template <typename R>
+__device__ __forceinline__ Stencil13<R> load_stencil(const R* p, const bool (&on)[3], const int (&s)[3]) {
+  Stencil13<R> q;
+  q.a0 = ld<R>(p, 0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    q.v[d][0] = q.v[d][1] = q.v[d][2] = q.v[d][3] = R(0);
+    if (on[d]) {
+      q.v[d][0] = ld<R>(p, -2 * s[d]); q.v[d][1] = ld<R>(p, -s[d]); q.v[d][2] = ld<R>(p, s[d]); q.v[d][3] = ld<R>(p, 2 * s[d]);
+    }
+  }
+  return q;
+}
+template <typename R>
+__device__ __forceinline__ bool stencil_nonzero(const Stencil13<R>& q) {  // in any cell of the warp
+  long long bits = __double_as_longlong(q.a0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bits |= __double_as_longlong(q.v[d][k]);
+  return __any_sync(0xffffffffu, (bits << 1) != 0);
+}
+// -div H of one component, and for pi^{tau nu} the sum of the v^d pi^{tau nu} differences (mix)
+template <typename R, bool TH1>
+__device__ __forceinline__ void stencil_flux(const Stencil13<R>& q, R c0, const bool (&on)[3], const Faces<R> (&F)[3],
+                                             R th, bool with_mix, R& acc, R& mix) {
+  acc = rmul(c0, q.a0);
+  mix = R(-0.0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (!on[d]) continue;
+    const R a1 = q.v[d][1], b1 = q.v[d][2];
+    const R d0 = a1 - q.v[d][0], d1 = q.a0 - a1, d2 = b1 - q.a0, d3 = q.v[d][3] - b1;
+    R sm, s0, sp;
+    three_slopes<R, TH1>(d0, d1, d2, d3, th, sm, s0, sp);
+    acc = fma(F[d].wLm, fma(R(0.5), sm, a1), acc);
+    acc = fma(F[d].wRp, fma(R(-0.5), sp, b1), acc);
+    acc = fma(F[d].hdW, s0, acc);
+    if (with_mix) mix = fma(F[d].vpl_h, b1, fma(-F[d].vmi_h, a1, mix));
+  }
+}
+template <typename R>
+__device__ __forceinline__ R sum_c0(const Faces<R> (&F)[3], const bool (&on)[3]) {
+  return (on[0] ? F[0].c0 : R(0)) + (on[1] ? F[1].c0 : R(0)) + (on[2] ? F[2].c0 : R(0));
+}
+
 template <typename R, bool TH1 = false>
 __device__ __forceinline__ void conserved_fluxes(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
-                                                 const Faces<R>& Fx, const Faces<R>& Fy, const Faces<R>& Fz,
-                                                 R (&dq)[NQ]) {
+                                                 const Faces<R> (&F)[3], R (&dq)[NQ]) {
   const long long fs = L.fstride;
   const R th = pr<R>(P).theta;
   const bool on[3] = {L.nx > 1, L.ny > 1, L.nz > 1};
-  const Faces<R>* const F[3] = {&Fx, &Fy, &Fz};
-  const R c0 = (on[0] ? Fx.c0 : R(0)) + (on[1] ? Fy.c0 : R(0)) + (on[2] ? Fz.c0 : R(0));
-  auto load = [&](int n) {
-    const R* p = io.qr_in + n * fs + c;
-    Stencil13<R> q;
-    q.a0 = ld<R>(p, 0);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int s = F[d]->s;
-      q.v[d][0] = q.v[d][1] = q.v[d][2] = q.v[d][3] = R(0);
-      if (on[d]) {
-        q.v[d][0] = ld<R>(p, -2 * s); q.v[d][1] = ld<R>(p, -s); q.v[d][2] = ld<R>(p, s); q.v[d][3] = ld<R>(p, 2 * s);
-      }
-    }
-    return q;
-  };
-  Stencil13<R> q = load(0);
+  const int s[3] = {F[0].s, F[1].s, F[2].s};
+  const R c0 = sum_c0<R>(F, on);
+  const R* p = io.qr_in + c;
+  Stencil13<R> q = load_stencil<R>(p, on, s);
 #pragma unroll
   for (int n = 0; n < NQ; ++n) {
     Stencil13<R> next;
-    if (n + 1 < NQ) next = load(n + 1);
-    long long bits = __double_as_longlong(q.a0);
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) bits |= __double_as_longlong(q.v[d][k]);
-    if (__any_sync(0xffffffffu, (bits << 1) != 0)) {
-      R acc = c0 * q.a0, mix = R(-0.0);  // mix: sum of the v^d pi^{tau nu} differences
+    if (n + 1 < NQ) next = load_stencil<R>(p + (n + 1) * fs, on, s);
+    if (stencil_nonzero<R>(q)) {
+      R acc, mix;
+      stencil_flux<R, TH1>(q, c0, on, F, th, n >= 4 && n <= 7, acc, mix);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        if (!on[d]) continue;
-        const R a1 = q.v[d][1], b1 = q.v[d][2];
-        const R d0 = a1 - q.v[d][0], d1 = q.a0 - a1, d2 = b1 - q.a0, d3 = q.v[d][3] - b1;
-        R sm, s0, sp;
-        three_slopes<R, TH1>(d0, d1, d2, d3, th, sm, s0, sp);
-        acc = fma(F[d]->wLm, fma(R(0.5), sm, a1), acc);
-        acc = fma(F[d]->wRp, fma(R(-0.5), sp, b1), acc);
-        acc = fma(F[d]->hdW, s0, acc);
-        if (n >= 4 && n <= 7) mix = fma(F[d]->vpl_h, b1, fma(-F[d]->vmi_h, a1, mix));
         const int r = (d == 0) ? cross_row<0>(n, false) : ((d == 1) ? cross_row<1>(n, false) : cross_row<2>(n, false));
-        if (n >= 4 && n <= 13 && r >= 0) add_row(dq, r, (a1 - b1) * pr<R>(P).half_inv_d[d]);
+        if (on[d] && n >= 4 && n <= 13 && r >= 0) dq[r] = fma(q.v[d][1] - q.v[d][2], pr<R>(P).half_inv_d[d], dq[r]);
       }
       dq[n] += acc;
       if (n >= 4 && n <= 7) dq[n - 4] += mix;
@@ -757,6 +776,13 @@ __device__ __forceinline__ CellGeom<R> cell_geom(const Params& P, double tau_src
   return g;
 }
 
+// d_i v^i from the differences v^d_{i+1} - v^d_{i-1}
+template <typename R>
+__device__ __forceinline__ R divergence(const Params& P, const R (&d)[3]) {
+  const R* h = pr<R>(P).half_inv_d;
+  return fma(d[2], h[2], fma(d[1], h[1], rmul(d[0], h[0])));
+}
+
 // the three directions' face setups; uc returns u^mu at the cell
 template <typename R, bool TH1, bool IFACE, typename UA>
 __device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
@@ -767,20 +793,21 @@ __device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, co
   for (int n = 0; n < NQ; ++n) dq[n] = R(-0.0);  // exact additive identity
 #pragma unroll
   for (int m = 0; m < 4; ++m) uc[m] = ua(m, 0);
-  dv = R(-0.0);
   const R sfac = P.milne ? G.tau : R(1);  // sqrt(-g_{eta eta}): speeds along eta in units of c
+  R d[3] = {R(0), R(0), R(0)};
   if constexpr (sizeof(R) == 8 && !IFACE) {
-    if (L.nx > 1) face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fx);
+    if (L.nx > 1) face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[0], amax, Fx);
     else face_none<R, 0>(uc, R(1), du, amax, Fx);
-    if (L.ny > 1) face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fy);
+    if (L.ny > 1) face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[1], amax, Fy);
     else face_none<R, 1>(uc, R(1), du, amax, Fy);
-    if (L.nz > 1) face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fz);
+    if (L.nz > 1) face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[2], amax, Fz);
     else face_none<R, 2>(uc, sfac, du, amax, Fz);
   } else {
-    face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fx);
-    face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fy);
-    face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dv, amax, Fz);
+    face_setup<R, 0, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[0], amax, Fx);
+    face_setup<R, 1, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[1], amax, Fy);
+    face_setup<R, 2, TH1, IFACE>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, d[2], amax, Fz);
   }
+  dv = divergence<R>(P, d);
 }
 
 template <typename R, bool DIAG = false>
@@ -794,9 +821,9 @@ __device__ __forceinline__ void cell_rhs(const Params& P, const Lattice& L, cons
   const CellGeom<R> G = cell_geom<R>(P, tau_src);
   R uc[4], du[4][4];
   R dv;
-  Faces<R> Fx, Fy, Fz;
-  cell_faces<R, TH1, IFACE>(P, L, io, c, u_global(L, io, c), G, dq, uc, du, dv, amax, Fx, Fy, Fz);
-  conserved_fluxes<R, TH1>(P, L, io, c, Fx, Fy, Fz, dq);
+  Faces<R> F[3];
+  cell_faces<R, TH1, IFACE>(P, L, io, c, u_global(L, io, c), G, dq, uc, du, dv, amax, F[0], F[1], F[2]);
+  conserved_fluxes<R, TH1>(P, L, io, c, F, dq);
   cell_sources<R>(P, L, io, c, G, uc, du, dv, dq);
 }
 
@@ -1031,37 +1058,42 @@ __device__ __forceinline__ double learned_start(const InvIn& v, float z) {
 }
 
 // ---------------------------------------------------------------- one cell (FP64)
-// The whole stage for cell o (x fastest, then y, then eta) of an event in one thread.  The 32 lanes of a
-// warp hold consecutive cells and stay together; lanes past the last cell repeat it and store nothing.
-template <typename R, int STAGE, bool TH1, bool IFACE>
-__device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, const StageIO<R>& io, unsigned o,
-                                           unsigned& st, unsigned& nit, unsigned& nreg, float& amax) {
-  static_assert(sizeof(R) == 8, "the fused stage is the FP64 path; mixed precision uses kt_split.cuh");
+// Cell o of an event (x fastest, then y, then eta).  The 32 lanes of a warp hold consecutive cells and
+// stay together; lanes past the last cell repeat it and store nothing.
+struct CellAt {
+  long long c;
+  int i, j, k;
+  bool valid;
+};
+__device__ __forceinline__ CellAt cell_at(const Lattice& L, unsigned o) {
   const unsigned ncells = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
-  const bool valid = o < ncells;
+  CellAt a;
+  a.valid = o < ncells;
   o = min(o, ncells - 1u);
   const unsigned row = o / (unsigned)L.nx;
-  const int i = (int)(o - row * (unsigned)L.nx), k = (int)(row / (unsigned)L.ny), j = (int)row - k * L.ny;
-  const long long fs = L.fstride;
-  const long long c = L.idx(i + 2, j + 2, k + 2);
-  const double tau_n = io.d_tau[0];
-  const double tau_src = (STAGE == 1) ? tau_n : tau_n + P.dtau;
-  const double tau_out = tau_n + P.dtau;
+  a.i = (int)(o - row * (unsigned)L.nx);
+  a.k = (int)(row / (unsigned)L.ny);
+  a.j = (int)row - a.k * L.ny;
+  a.c = L.idx(a.i + 2, a.j + 2, a.k + 2);
+  return a;
+}
+
+// Everything after dq = C[q]: c) the Heun update, d) the inversion, e) the regulator, f) the stores
+template <typename R, int STAGE>
+__device__ __forceinline__ void stage_finish(const Params& P, const Lattice& L, const StageIO<R>& io, const CellAt& at,
+                                             double tau_out, const R (&dq)[NQ], unsigned& st, unsigned& nit,
+                                             unsigned& nreg) {
+  static_assert(sizeof(R) == 8, "the fused stage is the FP64 path; mixed precision uses kt_split.cuh");
+  const long long fs = L.fstride, c = at.c;
   double qn[NQ];  // the new conserved state
-
-  {
-    R dq[NQ];
-    cell_rhs<R, TH1, IFACE>(P, L, io, c, tau_src, dq, amax);
-
-    // ---- c) Heun update in FP64 (Eqs. step1-finalStep)
+  // ---- c) Heun update in FP64 (Eqs. step1-finalStep)
 #pragma unroll
-    for (int n = 0; n < NQ; ++n) {
-      const double qi = __ldg(io.q_in + n * fs + c);
-      if (STAGE == 1)
-        qn[n] = qi + to_f64<R>(dq[n] * pr<R>(P).dtau);  // q* = q^n + dtau C[q^n]
-      else  // q^{n+1} = (q^n + q* + dtau C[q*]) / 2
-        qn[n] = fma(0.5, io.q_base[n * fs + c] + qi, to_f64<R>(dq[n] * pr<R>(P).half_dtau));
-    }
+  for (int n = 0; n < NQ; ++n) {
+    const double qi = __ldg(io.q_in + n * fs + c);
+    if (STAGE == 1)
+      qn[n] = fma(dq[n], pr<R>(P).dtau, qi);  // q* = q^n + dtau C[q^n]
+    else  // q^{n+1} = (q^n + q* + dtau C[q*]) / 2
+      qn[n] = fma(0.5, io.q_base[n * fs + c] + qi, dq[n] * pr<R>(P).half_dtau);
   }
 
   {
@@ -1071,7 +1103,7 @@ __device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, co
     const double guess = to_f64<R>(ld<R>(io.e_in, c));
     unsigned its = 0;
     const unsigned sti = invert_fp64(P, tau_out, qn, guess, e, P0, uo, its);
-    if (!valid) return;
+    if (!at.valid) return;
     st |= sti;
     nit += its;
 
@@ -1109,7 +1141,7 @@ __device__ __forceinline__ void stage_cell(const Params& P, const Lattice& L, co
       if (!finite(qr[n])) st |= ST_NONFINITE;
 
     // ---- f) stores
-    store_with_ghosts<R>(P, L, io, i + 2, j + 2, k + 2, qn, qr, uo, eR, P0R);
+    store_with_ghosts<R>(P, L, io, at.i + 2, at.j + 2, at.k + 2, qn, qr, uo, eR, P0R);
   }
 }
 
@@ -1175,7 +1207,7 @@ __device__ __forceinline__ void warp_stats(const StageIO<double>& io, unsigned s
   const unsigned full = 0xffffffffu;
   const unsigned w_st = __reduce_or_sync(full, st), w_max = __reduce_max_sync(full, __float_as_uint(amax));
   const unsigned w_it = __reduce_add_sync(full, nit), w_reg = __reduce_add_sync(full, nreg);
-  if (threadIdx.x == 0) {
+  if ((threadIdx.x & 31) == 0) {
     if (w_st) atomicOr(io.status, w_st);
     atomicMax(io.max_speed_bits, w_max);
     if (w_it) atomicAdd(io.counters + 0, (unsigned long long)w_it);
@@ -1197,7 +1229,131 @@ __global__ void __launch_bounds__(32, 8)
     L = lats[s.event];
     first = (unsigned)s.i0;
   }
-  stage_cell<R, STAGE, TH1, IFACE>(P, L, io, first + threadIdx.x, st, nit, nreg, amax);
+  const CellAt at = cell_at(L, first + threadIdx.x);
+  const double tau_n = io.d_tau[0], tau_out = tau_n + P.dtau;
+  R dq[NQ];
+  cell_rhs<R, TH1, IFACE>(P, L, io, at.c, (STAGE == 1) ? tau_n : tau_out, dq, amax);
+  stage_finish<R, STAGE>(P, L, io, at, tau_out, dq, st, nit, nreg);
+  __syncwarp();
+  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
+  warp_stats(io, st, amax, nit, nreg);
+}
+
+// ---------------------------------------------------------------- the same for grids with few cells (FP64)
+// With fewer strips than the chip has FP64 issue slots (four warps per SM) the kernel above is a serial
+// chain of ~1,500 FP64 instructions at 64 cycles each while most units idle.  Here four warps share a
+// strip: one axis each for the face setup (warps 0-2), every fourth component each for the fluxes, then
+// warp 0 adds up and runs the sources and the update.  Values pass through shared memory and are added in
+// the order of the one-warp kernel, so both give the same bits.
+enum : int { TM_FACE = 0, TM_DU = 18, TM_DV = 30, TM_PR = 33, TM_ACC = 39, TM_MIX = 54, TM_DIFF = 58, TM_VALUES = 70 };
+
+template <typename R, int D, bool TH1>
+__device__ __forceinline__ void team_faces(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+                                           const CellGeom<R>& G, R (*sm)[32], float& amax) {
+  const int lane = threadIdx.x & 31;
+  const UGlobal<R> ua = u_global(L, io, c);
+  const R sfac = P.milne ? G.tau : R(1);
+  R uc[4], du[4][4], dq[NQ], dvd = R(0);
+  Faces<R> F;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) uc[m] = ua(m, 0);
+  dq[0] = dq[D + 1] = R(-0.0);
+  const int n = (D == 0) ? L.nx : ((D == 1) ? L.ny : L.nz);
+  if (n > 1) face_setup<R, D, TH1, false>(P, L, io, c, ua, uc, G.inv_gnn, sfac, dq, du, dvd, amax, F);
+  else face_none<R, D>(uc, (D == 2) ? sfac : R(1), du, amax, F);
+  const R f[6] = {F.c0, F.wLm, F.wRp, F.hdW, F.vpl_h, F.vmi_h};
+#pragma unroll
+  for (int m = 0; m < 6; ++m) sm[TM_FACE + 6 * D + m][lane] = f[m];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) sm[TM_DU + 4 * D + m][lane] = du[D + 1][m];
+  sm[TM_DV + D][lane] = dvd;
+  sm[TM_PR + 2 * D][lane] = dq[0];
+  sm[TM_PR + 2 * D + 1][lane] = dq[D + 1];
+}
+
+template <typename R, int STAGE, bool TH1>
+__global__ void __launch_bounds__(128, 2)
+    stage_team_kernel(const Params P, const StageIO<R> io, const Lattice L0, const Lattice* __restrict__ lats,
+                      const Tile* __restrict__ strips, int n_events) {
+  __shared__ R sm[TM_VALUES][32];
+  unsigned st = 0, nit = 0, nreg = 0;
+  float amax = 0.f;
+  Lattice L = L0;
+  unsigned first = 32u * blockIdx.x;
+  if (n_events > 1) {
+    const Tile s = strips[blockIdx.x];
+    L = lats[s.event];
+    first = (unsigned)s.i0;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const CellAt at = cell_at(L, first + lane);
+  const double tau_n = io.d_tau[0], tau_out = tau_n + P.dtau;
+  const CellGeom<R> G = cell_geom<R>(P, (STAGE == 1) ? tau_n : tau_out);
+  const long long fs = L.fstride, c = at.c;
+  const bool on[3] = {L.nx > 1, L.ny > 1, L.nz > 1};
+  const int s[3] = {1, L.pitch, (int)L.plane};
+  const R* p = io.qr_in + c;
+  Stencil13<R> q = load_stencil<R>(p + warp * fs, on, s);  // in flight during the face setup
+  if (warp == 0) team_faces<R, 0, TH1>(P, L, io, c, G, sm, amax);
+  else if (warp == 1) team_faces<R, 1, TH1>(P, L, io, c, G, sm, amax);
+  else if (warp == 2) team_faces<R, 2, TH1>(P, L, io, c, G, sm, amax);
+  __syncthreads();
+  {
+    Faces<R> F[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      F[d] = Faces<R>{sm[TM_FACE + 6 * d][lane], sm[TM_FACE + 6 * d + 1][lane], sm[TM_FACE + 6 * d + 2][lane],
+                      sm[TM_FACE + 6 * d + 3][lane], sm[TM_FACE + 6 * d + 4][lane], sm[TM_FACE + 6 * d + 5][lane], s[d]};
+    const R c0 = sum_c0<R>(F, on), th = pr<R>(P).theta;
+#pragma unroll 1
+    for (int n = warp; n < NQ; n += 4) {
+      const Stencil13<R> next = load_stencil<R>(p + min(n + 4, NQ - 1) * fs, on, s);
+      R acc = R(-0.0), mix = R(-0.0);  // (adding -0 changes nothing)
+      const bool any = stencil_nonzero<R>(q);
+      if (any) stencil_flux<R, TH1>(q, c0, on, F, th, n >= 4 && n <= 7, acc, mix);
+      sm[TM_ACC + n][lane] = acc;
+      if (n >= 4 && n <= 7) sm[TM_MIX + n - 4][lane] = mix;
+      if (n >= 4 && n <= 13) {
+        const int r[3] = {cross_row<0>(n, false), cross_row<1>(n, false), cross_row<2>(n, false)};
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+          if (r[d] >= 0) sm[TM_DIFF + 4 * d + r[d]][lane] = (any && on[d]) ? q.v[d][1] - q.v[d][2] : R(-0.0);
+      }
+      q = next;
+    }
+  }
+  __syncthreads();
+  if (warp > 0) {
+    warp_stats(io, 0u, amax, 0u, 0u);
+    return;
+  }
+  R dq[NQ], uc[4], du[4][4];
+#pragma unroll
+  for (int n = 0; n < NQ; ++n) dq[n] = R(-0.0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    dq[0] += sm[TM_PR + 2 * d][lane];
+    dq[d + 1] += sm[TM_PR + 2 * d + 1][lane];
+  }
+#pragma unroll
+  for (int n = 0; n < NQ; ++n) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int r = (d == 0) ? cross_row<0>(n, false) : ((d == 1) ? cross_row<1>(n, false) : cross_row<2>(n, false));
+      if (n >= 4 && n <= 13 && r >= 0) dq[r] = fma(sm[TM_DIFF + 4 * d + r][lane], pr<R>(P).half_inv_d[d], dq[r]);
+    }
+    dq[n] += sm[TM_ACC + n][lane];
+    if (n >= 4 && n <= 7) dq[n - 4] += sm[TM_MIX + n - 4][lane];
+  }
+  const R d[3] = {sm[TM_DV][lane], sm[TM_DV + 1][lane], sm[TM_DV + 2][lane]};
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    uc[m] = ld<R>(io.u_in + m * fs, c);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) du[a + 1][m] = sm[TM_DU + 4 * a + m][lane];
+  }
+  cell_sources<R>(P, L, io, c, G, uc, du, divergence<R>(P, d), dq);
+  stage_finish<R, STAGE>(P, L, io, at, tau_out, dq, st, nit, nreg);
   __syncwarp();
   if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
   warp_stats(io, st, amax, nit, nreg);

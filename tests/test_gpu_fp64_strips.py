@@ -68,3 +68,29 @@ def test_batch_of_strips_matches_oracle(baseline_eos):
         a, b = k.get_state(event=ev), single.get_state()
         for f in FIELDS:
             assert np.array_equal(a[f], b[f]), (ev, f)
+
+
+@pytest.mark.parametrize("theta", [1.0, 1.6])
+@pytest.mark.parametrize("ideal", [False, True])
+def test_four_warp_and_one_warp_kernels_agree_bitwise(theta, ideal, baseline_eos):
+    """A grid of few strips runs four warps per strip, a larger one (here: the batch) one; the values are
+    added in the same order, so an event gives the same bits in both."""
+    from dataclasses import replace
+    from paper_1608_06577_gb300 import KT
+    probs = [_viscous(*s, baseline_eos, theta=theta)
+             for s in ((33, 1, 1), (1, 37, 1), (1, 1, 34), (9, 7, 1), (1, 1, 1), (6, 9, 5), (64, 52, 4))]
+    if ideal:
+        probs = [replace(p, eta_over_s=("const", 0.0, 0.0, 1.0), zeta_over_s=("const", 0.0, 0.0, 1.0),
+                         pi=np.zeros_like(p.pi), Pi=np.zeros_like(p.Pi)) for p in probs]
+    k = KT(probs)
+    k.set_problem_state()
+    k.step(5)
+    assert k.tuning()["grid_blocks"] > 304  # one warp per strip
+    for ev, p in enumerate(probs[:-1]):
+        single = KT(p)
+        single.set_problem_state()
+        single.step(5)
+        assert single.tuning()["grid_blocks"] <= 304
+        a, b = k.get_state(event=ev), single.get_state()
+        for f in FIELDS:
+            assert np.array_equal(a[f], b[f]), (ev, f)
