@@ -428,44 +428,94 @@ __global__ void batch_kernel(const float* __restrict__ x, const float* __restric
 }  // namespace
 
 namespace kt {
-// FP32 parameters -> packed BF16 fragments + FP32 biases (see kt_mlp.cuh)
+constexpr long long kPredictBlocks = 2 * 152;  // resident at ~100 registers and 256 threads
+
+// word i of the packed BF16 fragments + FP32 biases (see kt_mlp.cuh) of FP32 parameters
+__device__ __forceinline__ uint32_t packed_word(const float* __restrict__ params, int i) {
+  if (i < PK_W2) {  // W1 rows of 4 words
+    const int n = i / 4, w = i % 4, k = 2 * w;
+    const float lo = (k < MLP_IN) ? params[OFF_W1 + n * MLP_IN + k] : 0.f;
+    const float hi = (k + 1 < MLP_IN) ? params[OFF_W1 + n * MLP_IN + k + 1] : 0.f;
+    return pack_bf16x2(lo, hi);
+  }
+  if (i < PK_W3) {  // W2 rows of 20 words (16 used)
+    const int n = (i - PK_W2) / PK_W2_STRIDE, w = (i - PK_W2) % PK_W2_STRIDE;
+    return (w < 16) ? pack_bf16x2(params[OFF_W2 + n * MLP_H + 2 * w], params[OFF_W2 + n * MLP_H + 2 * w + 1]) : 0u;
+  }
+  if (i < PK_B1) return pack_bf16x2(params[OFF_W3 + 2 * (i - PK_W3)], params[OFF_W3 + 2 * (i - PK_W3) + 1]);
+  if (i < PK_B2) return __float_as_uint(params[OFF_B1 + (i - PK_B1)]);
+  if (i < PK_B3) return __float_as_uint(params[OFF_B2 + (i - PK_B2)]);
+  return __float_as_uint(params[OFF_B3]);
+}
+
 __global__ void mlp_pack_kernel(const float* __restrict__ params, uint32_t* packed) {
+  for (int i = threadIdx.x; i < PK_WORDS; i += blockDim.x) packed[i] = packed_word(params, i);
+}
+
+// Tensor-core inference over an array of feature rows, one launch: every block packs the weights into
+// shared memory (block 0 also into the caller's scratch), every warp keeps its fragments in registers
+// and walks groups of 32 rows.  A lane reads the two features its fragment holds straight from the row
+// (VEC: one 8-byte load; X 8-byte aligned), a warp's load covering whole sectors, and the lanes that hold
+// an output store it: no shuffles.  Bound by memory (28 B per row) and, below ~1e5 rows, by the launch.
+// (A packing launch and blocks of 256 rows reading six scalars per lane took 24.6 us per call of 1e6 rows.)
+template <bool VEC>
+__global__ void __launch_bounds__(256) mlp_predict_kernel(const float* __restrict__ params, uint32_t* scratch,
+                                                          const float* __restrict__ X, long long n, float* Y) {
+  __shared__ alignas(16) uint32_t sw[PK_WORDS];
   for (int i = threadIdx.x; i < PK_WORDS; i += blockDim.x) {
-    uint32_t v = 0u;
-    if (i < PK_W2) {  // W1 rows of 4 words
-      const int n = i / 4, w = i % 4, k = 2 * w;
-      const float lo = (k < MLP_IN) ? params[OFF_W1 + n * MLP_IN + k] : 0.f;
-      const float hi = (k + 1 < MLP_IN) ? params[OFF_W1 + n * MLP_IN + k + 1] : 0.f;
-      v = pack_bf16x2(lo, hi);
-    } else if (i < PK_W3) {  // W2 rows of 20 words (16 used)
-      const int n = (i - PK_W2) / PK_W2_STRIDE, w = (i - PK_W2) % PK_W2_STRIDE;
-      if (w < 16) v = pack_bf16x2(params[OFF_W2 + n * MLP_H + 2 * w], params[OFF_W2 + n * MLP_H + 2 * w + 1]);
-    } else if (i < PK_B1) {
-      const int w = i - PK_W3;
-      v = pack_bf16x2(params[OFF_W3 + 2 * w], params[OFF_W3 + 2 * w + 1]);
-    } else if (i < PK_B2) {
-      v = __float_as_uint(params[OFF_B1 + (i - PK_B1)]);
-    } else if (i < PK_B3) {
-      v = __float_as_uint(params[OFF_B2 + (i - PK_B2)]);
-    } else {
-      v = __float_as_uint(params[OFF_B3]);
-    }
-    packed[i] = v;
+    const uint32_t v = packed_word(params, i);
+    sw[i] = v;
+    if (blockIdx.x == 0) scratch[i] = v;
+  }
+  __syncthreads();
+  const MlpFrags f = mlp_frags(sw);
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const long long groups = (n + 31) / 32, warps = (long long)gridDim.x * (blockDim.x >> 5);
+  auto load = [&](long long grp, float2 (&v)[2][2]) {
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long r = 32 * grp + 16 * mt + 8 * h + g;
+        v[mt][h] = make_float2(0.f, 0.f);
+        if (t < 3 && r < n) {
+          const float* p = X + r * MLP_IN + 2 * t;
+          v[mt][h] = VEC ? __ldg(reinterpret_cast<const float2*>(p)) : make_float2(__ldg(p), __ldg(p + 1));
+        }
+      }
+  };
+  long long grp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  float2 v[2][2];
+  load(grp, v);
+  for (; grp < groups; grp += warps) {
+    float2 next[2][2];
+    load(grp + warps, next);
+    uint32_t a[2][2];
+    float o[2][2];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) a[mt][h] = pack_bf16x2(v[mt][h].x, v[mt][h].y);
+    mlp_infer(f, a, o);
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long r = 32 * grp + 16 * mt + 8 * h + g;
+        if (t == 0 && r < n) Y[r] = o[mt][h];
+        v[mt][h] = next[mt][h];
+      }
   }
 }
 
-// tensor-core inference over an array of feature rows
-__global__ void __launch_bounds__(256) mlp_predict_kernel(const uint32_t* __restrict__ packed,
-                                                          const float* __restrict__ X, long long n, float* Y) {
-  __shared__ alignas(16) uint32_t sw[PK_WORDS];
-  mlp_load_shared(sw, packed);
-  __syncthreads();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  float x[MLP_IN];
-#pragma unroll
-  for (int k = 0; k < MLP_IN; ++k) x[k] = (i < n) ? X[i * MLP_IN + k] : 0.f;
-  const float y = mlp_warp_infer(sw, x);  // every lane of the warp takes part
-  if (i < n) Y[i] = y;
+// the grid: as many blocks as are resident at once, or one warp per 32 rows
+int launch_predict(const float* params, uint32_t* scratch, const float* x, long long n, float* y, cudaStream_t s) {
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 7u) == 0;
+  const long long want = ((n + 31) / 32 + 7) / 8;
+  const unsigned grid = (unsigned)(want < kPredictBlocks ? want : kPredictBlocks);
+  if (vec) mlp_predict_kernel<true><<<grid, 256, 0, s>>>(params, scratch, x, n, y);
+  else mlp_predict_kernel<false><<<grid, 256, 0, s>>>(params, scratch, x, n, y);
+  return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ERR_CUDA;
 }
 }  // namespace kt
 
@@ -475,10 +525,7 @@ int kt_mlp_predict(const float* params, const float* x, long long n, float* y, v
                    void* stream) {
   if (!params || !x || !y || n < 0 || !scratch || scratch_bytes < (size_t)KT_MLP_PACKED_BYTES) return KT_ERR_ARG;
   if (n == 0) return KT_OK;
-  cudaStream_t s = (cudaStream_t)stream;
-  kt::mlp_pack_kernel<<<1, 256, 0, s>>>(params, (uint32_t*)scratch);
-  kt::mlp_predict_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const uint32_t*)scratch, x, n, y);
-  return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ERR_CUDA;
+  return kt::launch_predict(params, (uint32_t*)scratch, x, n, y, (cudaStream_t)stream);
 }
 
 int kt_mlp_predict_static(const float* params, const float* x, long long n, float* y, void* stream) {
@@ -495,11 +542,7 @@ int kt_mlp_predict_static(const float* params, const float* x, long long n, floa
   uint32_t* scratch = nullptr;
   const int rc = static_scratch_address(&scratch);
   if (rc != KT_OK) return rc;
-  cudaStream_t s = (cudaStream_t)stream;
-  // the pack kernel overwrites every word of the scratch, so nothing needs clearing first
-  kt::mlp_pack_kernel<<<1, 256, 0, s>>>(params, scratch);
-  kt::mlp_predict_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(scratch, x, n, y);
-  return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ERR_CUDA;
+  return kt::launch_predict(params, scratch, x, n, y, (cudaStream_t)stream);
 }
 
 int kt_mlp_grad(const float* params, const float* x, const float* y_target, long long n, int bf16_forward,

@@ -2,9 +2,9 @@
 //
 // A 6 -> 32 -> 32 -> 1 ReLU network predicts z, the correction y = 10 ln(e / e_conf) = r^2 z of
 // the conformal closed-form root e_conf = sqrt(4E^2 - 3M^2) - E of Sec. 2.4 (r^2 = M^2/E^2), for
-// cells with r^2 > kMlpGateR2 (below it y = 0).  Inference runs inside the first stage's update
-// kernel with warp-level BF16 tensor-core MMAs (FP32 accumulation); the second stage applies the
-// same z to its own features.  The Newton steps that follow and the residual test are FP64.
+// cells with r^2 > kMlpGateR2 (below it y = 0).  Inference runs once per step in a launch of its own
+// with warp-level BF16 tensor-core MMAs (FP32 accumulation); both stages apply its z to their own
+// features.  The Newton steps that follow and the residual test are FP64.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -66,76 +66,121 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Inference for the 32 cells of a warp (lane = cell); all 32 lanes must call it together.
-// w: packed weights (shared memory, 16-byte aligned).  Fragment layouts are those of mma.m16n8k16: lane =
-// 4 g + t holds rows g, g+8 and columns 2t, 2t+1 (+8) of A and C, and B rows 2t, 2t+1 (+8),
-// column g.  The C fragments of one layer are the A fragments of the next.
-__device__ __forceinline__ float mlp_warp_infer(const uint32_t* __restrict__ w, const float (&x)[MLP_IN]) {
+// The network's weights as one lane's B fragments of mma.m16n8k16 (lane = 4 g + t holds rows 2t, 2t+1
+// (+8) of column g) and the biases of the columns 2t, 2t+1 it accumulates: 41 registers, loaded once per
+// warp, where reading them from shared memory for every 32 rows took 37 loads of about 250 instructions.
+struct MlpFrags {
+  uint32_t w1_[4], w2_[4][2][2], w3_[2][2];
+  float2 b1_[4], b2_[4];
+  float b3_;
+  __device__ __forceinline__ uint32_t w1(int nt) const { return w1_[nt]; }
+  __device__ __forceinline__ uint32_t w2(int nt, int ks, int h) const { return w2_[nt][ks][h]; }
+  __device__ __forceinline__ uint32_t w3(int ks, int h) const { return w3_[ks][h]; }
+  __device__ __forceinline__ float2 b1(int nt) const { return b1_[nt]; }
+  __device__ __forceinline__ float2 b2(int nt) const { return b2_[nt]; }
+  __device__ __forceinline__ float b3() const { return b3_; }
+};
+// The same read from the packed weights (shared memory, 16-byte aligned) where registers are better spent
+// on more warps (mlp_start_kernel: 41 registers fewer and twice the warps run it twice as fast).
+struct MlpShared {
+  const uint32_t* w;
+  int g, t;
+  __device__ __forceinline__ explicit MlpShared(const uint32_t* p)
+      : w(p), g((int)(threadIdx.x & 31) >> 2), t((int)threadIdx.x & 3) {}
+  __device__ __forceinline__ uint32_t w1(int nt) const { return w[PK_W1 + (nt * 8 + g) * 4 + t]; }
+  __device__ __forceinline__ uint32_t w2(int nt, int ks, int h) const {
+    return w[PK_W2 + (nt * 8 + g) * PK_W2_STRIDE + ks * 8 + 4 * h + t];
+  }
+  __device__ __forceinline__ uint32_t w3(int ks, int h) const { return (g == 0) ? w[PK_W3 + ks * 8 + 4 * h + t] : 0u; }
+  __device__ __forceinline__ float2 b1(int nt) const { return bias_pair(w, PK_B1 + nt * 8 + 2 * t); }
+  __device__ __forceinline__ float2 b2(int nt) const { return bias_pair(w, PK_B2 + nt * 8 + 2 * t); }
+  __device__ __forceinline__ float b3() const { return __uint_as_float(w[PK_B3]); }
+};
+__device__ __forceinline__ MlpFrags mlp_frags(const uint32_t* __restrict__ w) {
+  const MlpShared m(w);
+  MlpFrags f;
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    f.w1_[nt] = m.w1(nt);
+    f.b1_[nt] = m.b1(nt);
+    f.b2_[nt] = m.b2(nt);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f.w2_[nt][k >> 1][k & 1] = m.w2(nt, k >> 1, k & 1);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) f.w3_[k >> 1][k & 1] = m.w3(k >> 1, k & 1);
+  f.b3_ = m.b3();
+  return f;
+}
+
+// Inference for 32 rows of features, all 32 lanes together.  a: layer-1 A fragments, [m-tile][row half]:
+// features 2t, 2t+1 (t < 3; k >= 6 is zero) of row 16 mt + g + 8 h as BF16.  The C fragments of one layer
+// are the A fragments of the next.  The output of row 16 mt + g is out[mt][0], of row 16 mt + g + 8
+// out[mt][1], in the lanes with t = 0.
+template <typename Weights>
+__device__ __forceinline__ void mlp_infer(const Weights& f, const uint32_t (&a)[2][2], float (&out)[2][2]) {
+  uint32_t a2f[2][2][4];  // layer-2 A: [m-tile][k-step][4]
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt)  // layer 1: [32 x 8(k)] x [8 x 32] + b1, ReLU
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      float c[4] = {f.b1(nt).x, f.b1(nt).y, f.b1(nt).x, f.b1(nt).y};
+      mma_bf16_16816(c, a[mt][0], a[mt][1], 0u, 0u, f.w1(nt), 0u);
+      a2f[mt][nt >> 1][(nt & 1) * 2 + 0] = pack_relu_bf16x2(c[0], c[1]);
+      a2f[mt][nt >> 1][(nt & 1) * 2 + 1] = pack_relu_bf16x2(c[2], c[3]);
+    }
+  uint32_t a3f[2][2][4];
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {  // layer 2: [32 x 32] x [32 x 32] + b2, ReLU
+    const float2 b = f.b2(nt);
+    float c[2][4] = {{b.x, b.y, b.x, b.y}, {b.x, b.y, b.x, b.y}};
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+        mma_bf16_16816(c[mt], a2f[mt][ks][0], a2f[mt][ks][1], a2f[mt][ks][2], a2f[mt][ks][3], f.w2(nt, ks, 0),
+                       f.w2(nt, ks, 1));
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      a3f[mt][nt >> 1][(nt & 1) * 2 + 0] = pack_relu_bf16x2(c[mt][0], c[mt][1]);
+      a3f[mt][nt >> 1][(nt & 1) * 2 + 1] = pack_relu_bf16x2(c[mt][2], c[mt][3]);
+    }
+  }
+  // layer 3: [32 x 32] x [32 x 8 (column 0 used)] + b3
+  const float b3 = f.b3();
+  float c3[2][4] = {{b3, b3, b3, b3}, {b3, b3, b3, b3}};
+#pragma unroll
+  for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+      mma_bf16_16816(c3[mt], a3f[mt][ks][0], a3f[mt][ks][1], a3f[mt][ks][2], a3f[mt][ks][3], f.w3(ks, 0), f.w3(ks, 1));
+#pragma unroll
+  for (int mt = 0; mt < 2; ++mt) {
+    out[mt][0] = c3[mt][0];
+    out[mt][1] = c3[mt][2];
+  }
+}
+
+// The same with lane = row: every lane passes its row's features and gets its row's output.
+template <typename Weights>
+__device__ __forceinline__ float mlp_warp_infer(const Weights& f, const float (&x)[MLP_IN]) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const uint32_t p0 = pack_bf16x2(x[0], x[1]), p1 = pack_bf16x2(x[2], x[3]), p2 = pack_bf16x2(x[4], x[5]);
-  uint32_t a1f[2][2];  // layer-1 A: [m-tile][row half], columns 2t, 2t+1 (k >= 8 is zero)
+  uint32_t a[2][2];
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int src = mt * 16 + g + 8 * h;
-      uint32_t w0 = __shfl_sync(full, p0, src), w1 = __shfl_sync(full, p1, src), w2 = __shfl_sync(full, p2, src);
-      a1f[mt][h] = (t == 0) ? w0 : ((t == 1) ? w1 : ((t == 2) ? w2 : 0u));
+      const uint32_t w0 = __shfl_sync(full, p0, src), w1 = __shfl_sync(full, p1, src), w2 = __shfl_sync(full, p2, src);
+      a[mt][h] = (t == 0) ? w0 : ((t == 1) ? w1 : ((t == 2) ? w2 : 0u));
     }
-  // layer 1: [32 x 8(k)] x [8 x 32] + b1, ReLU
-  uint32_t a2f[2][2][4];  // layer-2 A: [m-tile][k-step][4]
-#pragma unroll
-  for (int nt = 0; nt < 4; ++nt) {
-    const uint32_t b0 = w[PK_W1 + (nt * 8 + g) * 4 + t];
-    const float2 bi = bias_pair(w, PK_B1 + nt * 8 + 2 * t);
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      float c[4] = {bi.x, bi.y, bi.x, bi.y};
-      mma_bf16_16816(c, a1f[mt][0], a1f[mt][1], 0u, 0u, b0, 0u);
-      const uint32_t lo = pack_relu_bf16x2(c[0], c[1]);
-      const uint32_t hi = pack_relu_bf16x2(c[2], c[3]);
-      const int ks = nt >> 1, half = nt & 1;
-      a2f[mt][ks][half * 2 + 0] = lo;
-      a2f[mt][ks][half * 2 + 1] = hi;
-    }
-  }
-  // layer 2: [32 x 32] x [32 x 32] + b2, ReLU
-  uint32_t a3f[2][2][4];
-#pragma unroll
-  for (int nt = 0; nt < 4; ++nt) {
-    const float2 bi = bias_pair(w, PK_B2 + nt * 8 + 2 * t);
-    float c[2][4] = {{bi.x, bi.y, bi.x, bi.y}, {bi.x, bi.y, bi.x, bi.y}};
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const uint32_t b0 = w[PK_W2 + (nt * 8 + g) * PK_W2_STRIDE + ks * 8 + t];
-      const uint32_t b1 = w[PK_W2 + (nt * 8 + g) * PK_W2_STRIDE + ks * 8 + 4 + t];
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-        mma_bf16_16816(c[mt], a2f[mt][ks][0], a2f[mt][ks][1], a2f[mt][ks][2], a2f[mt][ks][3], b0, b1);
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      const int ks = nt >> 1, half = nt & 1;
-      a3f[mt][ks][half * 2 + 0] = pack_relu_bf16x2(c[mt][0], c[mt][1]);
-      a3f[mt][ks][half * 2 + 1] = pack_relu_bf16x2(c[mt][2], c[mt][3]);
-    }
-  }
-  // layer 3: [32 x 32] x [32 x 8 (column 0 used)] + b3
-  const float b3 = __uint_as_float(w[PK_B3]);
-  float c3[2][4] = {{b3, b3, b3, b3}, {b3, b3, b3, b3}};
-#pragma unroll
-  for (int ks = 0; ks < 2; ++ks) {
-    const uint32_t b0 = (g == 0) ? w[PK_W3 + ks * 8 + t] : 0u;
-    const uint32_t b1 = (g == 0) ? w[PK_W3 + ks * 8 + 4 + t] : 0u;
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-      mma_bf16_16816(c3[mt], a3f[mt][ks][0], a3f[mt][ks][1], a3f[mt][ks][2], a3f[mt][ks][3], b0, b1);
-  }
-  // column 0 of row r of m-tile mt sits in lane 4 (r mod 8), register 0 (r < 8) or 2
+  float o[2][2];
+  mlp_infer(f, a, o);
   const int mt = lane >> 4, r = lane & 15, src = 4 * (r & 7);
-  const float v00 = __shfl_sync(full, c3[0][0], src), v02 = __shfl_sync(full, c3[0][2], src);
-  const float v10 = __shfl_sync(full, c3[1][0], src), v12 = __shfl_sync(full, c3[1][2], src);
+  const float v00 = __shfl_sync(full, o[0][0], src), v02 = __shfl_sync(full, o[0][1], src);
+  const float v10 = __shfl_sync(full, o[1][0], src), v12 = __shfl_sync(full, o[1][1], src);
   return (mt == 0) ? ((r < 8) ? v00 : v02) : ((r < 8) ? v10 : v12);
 }
 

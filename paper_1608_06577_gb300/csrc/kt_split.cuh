@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(256) mlp_start_kernel(const float* __restrict_
     }
     float x[MLP_IN], ecE;
     mlp_features(fmaxf(E, 1e-30f), fmaf(Mx, Mx, fmaf(My, My, gnn * Mn * Mn)), Pi, x, ecE);
-    const float z = __any_sync(0xffffffffu, x[1] > kMlpGateR2) ? mlp_warp_infer(sw, x) : 0.f;  // all lanes
+    const float z = __any_sync(0xffffffffu, x[1] > kMlpGateR2) ? mlp_warp_infer(MlpShared(sw), x) : 0.f;  // all lanes
     if (in) z_net[t] = z;
   }
 }
