@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256)
     upr[m] = from_f64<R>(up4[m]);
   }
   const R er = from_f64<R>(e), pr0 = from_f64<R>(P0);
-  for_cell_and_ghosts(P, L, i, j, k, [&](long long c) {
+  for_cell_and_ghosts(P, L, L.idx(i, j, k), i, j, k, [&](long long c) {
 #pragma unroll
     for (int n = 0; n < NQ; ++n) q[n * fs + c] = qn[n];
     if (qf) {
@@ -470,7 +470,7 @@ __global__ void scatter_kernel(const Params P, const Lattice L, const double* __
   if (o >= ncp) return;
   int i = (int)(o % L.nx), j = (int)((o / L.nx) % L.ny), k = (int)(o / ((long long)L.nx * L.ny));
   const S v = (S)in[o];
-  for_cell_and_ghosts(P, L, i + 2, j + 2, k + 2, [&](long long t) { f[t] = v; });
+  for_cell_and_ghosts(P, L, L.idx(i + 2, j + 2, k + 2), i + 2, j + 2, k + 2, [&](long long t) { f[t] = v; });
 }
 
 // smallest and largest e and smallest regulation factor over one event's physical cells (all
@@ -538,7 +538,7 @@ __global__ void diag_kernel(const Params P, const Lattice L, const StageIO<R> io
   const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= ncp) return;
   const int i = (int)(o % L.nx), j = (int)((o / L.nx) % L.ny), k = (int)(o / ((long long)L.nx * L.ny));
-  const long long c = L.idx(i + 2, j + 2, k + 2);
+  const Idx<R> c = cell_idx<R>(L, i + 2, j + 2, k + 2);
   const CellGeom<R> G = cell_geom<R>(P, tau);
   R dq[NQ], du[4][4], dv, dg[6];
   float amax = 0.f;
@@ -699,11 +699,12 @@ template <int STAGE>
 void launch_rhs(Ctx* c, const StageIO<float>& io) {
   const Shape& s = kShapes[c->shape];
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  with_flags([&](auto single, auto t1, auto inv) {
-    rhs_kernel<single.value, t1.value, inv.value>
+  with_flags([&](auto single, auto t1, auto inv, auto fixed) {
+    constexpr int f = fixed.value ? 2 : 0;
+    rhs_kernel<single.value, t1.value, inv.value, f, f>
         <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
             c->P, io, STAGE, k_buf(c, STAGE), make_work(c), c->map0[STAGE - 1], maps);
-  }, c->nev == 1, c->P.theta == 1.0, c->P.iface_invert != 0);
+  }, c->nev == 1, c->P.theta == 1.0, c->P.iface_invert != 0, s.y == 2 && s.z == 2);
 }
 
 // every rhs kernel may take the dynamic shared memory of the largest tile shape
@@ -714,12 +715,13 @@ int allow_rhs_smem(Ctx* c) {
   auto set = [&](const void* f) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  for (int f = 0; f < 8; ++f) {
-    with_flags([&](auto a, auto b, auto d) {
-      set((const void*)rhs_kernel<a.value, b.value, d.value>);
-      set((const void*)fused_kernel<a.value, 1, b.value, d.value>);
-      set((const void*)fused_kernel<a.value, 2, b.value, d.value>);
-    }, (f & 1) != 0, (f & 2) != 0, (f & 4) != 0);
+  for (int f = 0; f < 16; ++f) {
+    with_flags([&](auto a, auto b, auto d, auto fixed) {
+      constexpr int x = fixed.value ? 2 : 0;
+      set((const void*)rhs_kernel<a.value, b.value, d.value, x, x>);
+      set((const void*)fused_kernel<a.value, 1, b.value, d.value, x, x>);
+      set((const void*)fused_kernel<a.value, 2, b.value, d.value, x, x>);
+    }, (f & 1) != 0, (f & 2) != 0, (f & 4) != 0, (f & 8) != 0);
   }
   if (e != cudaSuccess) return fail(c, KT_ERR_CUDA, "rhs shared memory: %s", cudaGetErrorString(e));
   bytes = 0;
@@ -757,11 +759,12 @@ template <int STAGE>
 void launch_fused(Ctx* c, const StageIO<float>& io, const UpdIO& uio) {
   const Shape& s = kShapes[c->shape];
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  with_flags([&](auto single, auto t1, auto learned) {
-    fused_kernel<single.value, STAGE, t1.value, learned.value>
+  with_flags([&](auto single, auto t1, auto learned, auto fixed) {
+    constexpr int f = fixed.value ? 2 : 0;
+    fused_kernel<single.value, STAGE, t1.value, learned.value, f, f>
         <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
             c->P, io, uio, make_work(c), c->map0[STAGE - 1], maps);
-  }, c->nev == 1, c->P.theta == 1.0, c->learned != 0);
+  }, c->nev == 1, c->P.theta == 1.0, c->learned != 0, s.y == 2 && s.z == 2);
 }
 
 template <int STAGE>
@@ -944,8 +947,8 @@ int select_shape(Ctx* c, int cand) {
   const Shape& sh = kShapes[shape];
   auto grid = [&](int cap) { return one_per_tile ? c->ntiles : std::max(1, std::min(cap, c->ntiles)); };
   const size_t rsm = rhs_smem_bytes(sh.x, sh.y, sh.z);
-  c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<true, 1, true, true>, sh, rsm)
-                              : occupancy_blocks(rhs_kernel<true, true, false>, sh, rsm));
+  c->grid_rhs = grid(c->fused ? occupancy_blocks(fused_kernel<true, 1, true, true, 0, 0>, sh, rsm)
+                              : occupancy_blocks(rhs_kernel<true, true, false, 0, 0>, sh, rsm));
   if (c->staged) {
     const size_t usm = upd_smem_bytes(sh.x, sh.y, sh.z, c->upd_nbuf);
     c->grid_upd = grid(c->learned ? occupancy_blocks(update_staged_kernel<2, true>, sh, usm)

@@ -36,7 +36,22 @@ struct Lattice {
   __host__ __device__ long long idx(int i, int j, int k) const {
     return base + (long long)i + (long long)pitch * ((long long)j + (long long)NY * (long long)k);
   }
+  __device__ unsigned idx32(int i, int j, int k) const {
+    return (unsigned)base + (unsigned)(i + pitch * j) + (unsigned)plane * (unsigned)k;
+  }
 };
+
+// The index of a cell within a component: 32 bits on the mixed-precision path, whose byte offsets c * 8 fit
+// (a component of 2^29 elements would need more memory than the device has), so that an access is a
+// uniform component base plus one 32-bit offset shared by all components; 64 bits on the FP64 path.
+template <typename R> struct IdxOf { using type = long long; };
+template <> struct IdxOf<float> { using type = unsigned; };
+template <typename R> using Idx = typename IdxOf<R>::type;
+template <typename R>
+__device__ __forceinline__ Idx<R> cell_idx(const Lattice& L, int i, int j, int k) {
+  if constexpr (sizeof(R) == 4) return L.idx32(i, j, k);
+  else return L.idx(i, j, k);
+}
 
 // a block-shaped tile of one event: the persistent stage kernel walks a table of these
 struct Tile {
@@ -408,10 +423,25 @@ template <typename R> __device__ __forceinline__ R from_f64(double x);
 template <> __device__ __forceinline__ double from_f64<double>(double x) { return x; }
 template <> __device__ __forceinline__ float from_f64<float>(double x) { return d2f_bits(x); }
 
+// element i of a component (read through the read-only cache) with a 64-bit or a 32-bit index, and the
+// store of one with a 32-bit index
+template <typename S>
+__device__ __forceinline__ S at(const S* __restrict__ p, long long i) { return __ldg(p + i); }
+template <typename S>
+__device__ __forceinline__ S at(const S* __restrict__ p, unsigned i) {
+  return __ldg(reinterpret_cast<const S*>(reinterpret_cast<const char*>(p) + (i * (unsigned)sizeof(S))));
+}
+template <typename S>
+__device__ __forceinline__ void put(S* p, unsigned i, S v) {
+  *reinterpret_cast<S*>(reinterpret_cast<char*>(p) + (i * (unsigned)sizeof(S))) = v;
+}
+template <typename S>
+__device__ __forceinline__ void put(S* p, long long i, S v) { p[i] = v; }
+
 // per-cell read of an R-typed field from a buffer that may hold double or float
-template <typename R, typename S>
-__device__ __forceinline__ R ld(const S* __restrict__ p, long long i) {
-  return (R)__ldg(p + i);
+template <typename R, typename S, typename I>
+__device__ __forceinline__ R ld(const S* __restrict__ p, I i) {
+  return (R)at(p, i);
 }
 
 }  // namespace kt

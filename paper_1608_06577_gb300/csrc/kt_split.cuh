@@ -47,6 +47,11 @@ struct UpdIO {
 // bank instead of registers, and tile t follows from t by two divisions (tiles run along eta, then x, y).
 // 128^3 step, learned start: split launches 1.018 -> 0.938 ms, fused 1.047 -> 0.931 ms; FP32 pi storage,
 // 96 x 96 x 64: 0.328 -> 0.302 ms.
+constexpr int kTileX = 32;  // every tile is 32 cells wide: a warp is one x-row of a tile
+// TY, TZ of the stencil kernels: the tile's extents in y and eta where they are compile-time constants
+// (32 x 2 x 2, the shape that wins at most sizes: its shared-memory strides become immediates), 0 for the
+// other shapes.  With 32-bit cell indices, 128^3 step in the split layout on 32 x 2 x 2 tiles: right-hand
+// side 232 -> 217 us, updates 216 / 287 -> 205 / 277 us, step 0.951 -> 0.906 ms.
 struct Work {
   Lattice L0;             // the single event's lattice
   unsigned tk, ti;        // its tiles along eta and x
@@ -55,10 +60,18 @@ struct Work {
   const Tile* tiles;
 };
 template <bool SINGLE>
-__device__ __forceinline__ Tile tile_at(const Work& W, int t) {
+__device__ __forceinline__ Tile tile_at(const Work& W, int t, int ty, int tz) {
   if constexpr (!SINGLE) return W.tiles[t];
   const unsigned a = (unsigned)t / W.tk, k = (unsigned)t - a * W.tk, j = a / W.ti, i = a - j * W.ti;
-  return Tile{0, (int)(i * blockDim.x), (int)(j * blockDim.y), (int)(k * blockDim.z)};
+  return Tile{0, (int)i * kTileX, (int)j * ty, (int)k * tz};
+}
+// (the component stride is the same for all events: a kernel parameter for batches too)
+template <bool SINGLE>
+__device__ __forceinline__ Lattice lattice_at(const Work& W, int event) {
+  if constexpr (SINGLE) return W.L0;
+  Lattice L = W.lats[event];
+  L.fstride = W.L0.fstride;
+  return L;
 }
 
 // inversion inputs of q: T^{tau mu} (0-3), pi^{tau mu} (4-7), Pi (14)
@@ -86,18 +99,20 @@ __host__ __device__ constexpr int rhs_smem_bytes(int tx, int ty, int tz) {  // t
 // unconstrained choice; 128^3 step in the split layout: update caps 64/80 0.954 ms, 72/96 0.961 ms, 80/104
 // with rhs 80 1.023 ms.
 // map0: the single event's tensor map, as a kernel parameter (no fence, no fetch through L2); tmaps: a batch's
-template <bool SINGLE, bool TH1, bool IFACE>
+template <bool SINGLE, bool TH1, bool IFACE, int TY, int TZ>
 __global__ void __maxnreg__(96)
     rhs_kernel(const Params P, const StageIO<float> io, int stage, float* __restrict__ k_out, const Work W,
                const __grid_constant__ CUtensorMap map0, const CUtensorMap* __restrict__ tmaps) {
   extern __shared__ __align__(128) float s_raw[];
   __shared__ alignas(8) uint64_t s_bar[2];
   float* const s_q = s_raw + ((32u - ((smem_u32(s_raw) >> 2) & 31u)) & 31u);  // TMA wants 128-byte buffers
-  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int bx = blockDim.x + 4, by = blockDim.y + 4, bz = blockDim.z + 4;
+  const int ty = TY ? TY : (int)blockDim.y, tz = TZ ? TZ : (int)blockDim.z;
+  const int tid = threadIdx.x + kTileX * (threadIdx.y + ty * threadIdx.z);
+  constexpr int bx = kTileX + 4;
+  const int by = ty + 4, bz = tz + 4;
   const int vol = bx * by * bz;                  // floats per component in a buffer
   const unsigned box_bytes = 4u * kCompPerBox * vol;
-  const int bfl = rhs_buffer_floats(blockDim.x, blockDim.y, blockDim.z);
+  const int bfl = rhs_buffer_floats(kTileX, ty, tz);
   if (tid == 0) {
     mbar_init(&s_bar[0], 1);
     mbar_init(&s_bar[1], 1);
@@ -122,8 +137,8 @@ __global__ void __maxnreg__(96)
   int t0, t1;
   tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tile_at<SINGLE>(W, t);
-    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
+    const Tile tl = tile_at<SINGLE>(W, t, ty, tz);
+    const Lattice L = lattice_at<SINGLE>(W, tl.event);
     const CUtensorMap* map = SINGLE ? &map0 : tmaps + tl.event;
     if (t > t0 && __syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
     if (tid == 0) {
@@ -135,7 +150,7 @@ __global__ void __maxnreg__(96)
 
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
     const bool valid = (i < L.nx) && (j < L.ny) && (k < L.nz);
-    const long long c = valid ? L.idx(i + 2, j + 2, k + 2) : 0;
+    const unsigned c = valid ? L.idx32(i + 2, j + 2, k + 2) : 0u;
     float dq[NQ], uc[4], du[4][4], dv = 0.f;
     Faces<float> Fx, Fy, Fz;
     if (valid) {  // the sources first: du and dv are dead before the component loop (fewer spills)
@@ -169,7 +184,7 @@ __global__ void __maxnreg__(96)
     if (valid && !bad) {  // (a timed-out block leaves at the next tile's barrier)
       const float dt = pr<float>(P).dtau;
 #pragma unroll
-      for (int n = 0; n < NQ; ++n) k_out[n * L.fstride + c] = dq[n] * dt;
+      for (int n = 0; n < NQ; ++n) put(k_out + n * L.fstride, c, dq[n] * dt);
     }
   }
   if (bad) {  // a copy did not complete in time: let the ones in flight land before the block exits
@@ -273,12 +288,13 @@ __device__ __forceinline__ unsigned invert_split(const Params& P, const InvIn& v
 // (FP32 pi storage, stage 2).
 struct UpdInGlobal {
   const UpdIO& io;
-  long long fs, c;
-  __device__ __forceinline__ double q(int n) const { return __ldg(io.q + n * fs + c); }
-  __device__ __forceinline__ float k1(int n) const { return __ldg(io.k1 + n * fs + c); }
-  __device__ __forceinline__ float k2(int n) const { return __ldg(io.k2 + n * fs + c); }
-  __device__ __forceinline__ float qfn(int n) const { return __ldg(io.qf_n + n * fs + c); }
-  __device__ __forceinline__ float qs(int n) const { return __ldg(io.qsf + n * fs + c); }
+  long long fs;
+  unsigned c;
+  __device__ __forceinline__ double q(int n) const { return at(io.q + n * fs, c); }
+  __device__ __forceinline__ float k1(int n) const { return at(io.k1 + n * fs, c); }
+  __device__ __forceinline__ float k2(int n) const { return at(io.k2 + n * fs, c); }
+  __device__ __forceinline__ float qfn(int n) const { return at(io.qf_n + n * fs, c); }
+  __device__ __forceinline__ float qs(int n) const { return at(io.qsf + n * fs, c); }
 };
 
 // the increment added to q^n in FP64: k_1 (stage 1) or (k_1 + k_2)/2 (stage 2)
@@ -307,7 +323,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
                                             unsigned& nit, unsigned& nreg, unsigned& nfb) {
   const bool valid = (i < L.nx) && (j < L.ny) && (k < L.nz);
   const long long fs = L.fstride;
-  const long long c = L.idx(i + 2, j + 2, k + 2);
+  const unsigned c = L.idx32(i + 2, j + 2, k + 2);
   double qn[NQ];  // FP64 new state; components outside the inversion set are formed after it
   float qp[NQ];   // FP32 pi storage: the new pi, Pi (components 4-14)
 #pragma unroll
@@ -346,9 +362,9 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
   const InvIn v = inv_in(gnn, E, Mx, My, Mn, Pi);
   double start;
   if constexpr (LEARNED) {
-    start = learned_start(v, valid ? __ldg(io.z_net + c) : 0.f);
+    start = learned_start(v, valid ? at(io.z_net, c) : 0.f);
   } else {
-    start = valid ? to_f64<float>(__ldg(io.e_guess + c)) : 1.0;
+    start = valid ? to_f64<float>(at(io.e_guess, c)) : 1.0;
   }
 
   if (!valid) return;
@@ -408,7 +424,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
       }
     const float f = regulator_factor<float>(P, go, from_f64<float>(tau_out), eR, P0R, uo, pm, qr[14]);
     if (f < 0.999f) ++nreg;
-    if (STAGE == 2 && io.reg_out) io.reg_out[c] = f;
+    if (STAGE == 2 && io.reg_out) put(io.reg_out, c, f);
     if (f != 1.f) {
       if constexpr (PI32) {  // the FP32 state itself is rescaled (stage 2 reads q* from it)
 #pragma unroll
@@ -416,7 +432,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
       } else if constexpr (STAGE == 1) {
 #pragma unroll
         for (int n = 4; n < 14; ++n) {  // f q* = q^n + (f k_1 + (f - 1) q^n)
-          io.k1[n * fs + c] = fmaf(f, in.k1(n), (f - 1.f) * in.qfn(n));
+          put(io.k1 + n * fs, c, fmaf(f, in.k1(n), (f - 1.f) * in.qfn(n)));
           qr[n] *= f;
         }
         k1_pi_written = true;
@@ -441,7 +457,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
   if constexpr (STORE_K1 && STAGE == 1 && !PI32) {
 #pragma unroll
     for (int n = 0; n < NQ; ++n)
-      if (n < 4 || n > 13 || !k1_pi_written) io.k1[n * fs + c] = in.k1(n);
+      if (n < 4 || n > 13 || !k1_pi_written) put(io.k1 + n * fs, c, in.k1(n));
   }
 #pragma unroll
   for (int n = 0; n < NQ; ++n)
@@ -452,15 +468,15 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
   if constexpr (STAGE == 2) {
 #pragma unroll
     for (int n = 0; n < NQ; ++n)
-      if (!PI32 || n < 4) io.q[n * fs + c] = qn[n];
+      if (!PI32 || n < 4) put(io.q + n * fs, c, qn[n]);
   }
-  for_cell_and_ghosts(P, L, i + 2, j + 2, k + 2, [&](long long t) {
+  for_cell_and_ghosts(P, L, c, i + 2, j + 2, k + 2, [&](unsigned t) {
 #pragma unroll
-    for (int n = 0; n < NQ; ++n) io.qr_out[n * fs + t] = qr[n];
+    for (int n = 0; n < NQ; ++n) put(io.qr_out + n * fs, t, qr[n]);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) io.u_out[m * fs + t] = uo[m];
-    io.e_out[t] = eR;
-    io.p_out[t] = P0R;
+    for (int m = 0; m < 4; ++m) put(io.u_out + m * fs, t, uo[m]);
+    put(io.e_out, t, eR);
+    put(io.p_out, t, P0R);
   });
 }
 
@@ -471,10 +487,10 @@ __global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, 
   int t0, t1;
   tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tile_at<SINGLE>(W, t);
-    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
+    const Tile tl = tile_at<SINGLE>(W, t, (int)blockDim.y, (int)blockDim.z);
+    const Lattice L = lattice_at<SINGLE>(W, tl.event);
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
-    const UpdInGlobal in{io, L.fstride, L.idx(i + 2, j + 2, k + 2)};
+    const UpdInGlobal in{io, L.fstride, L.idx32(i + 2, j + 2, k + 2)};
     update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau_out, st, nit, nreg, nfb);
   }
   if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && (threadIdx.x | threadIdx.y | threadIdx.z) == 0);
@@ -638,22 +654,23 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
 template <int STAGE>
 struct UpdInFused {
   const UpdIO& io;
-  long long fs, c;
+  long long fs;
+  unsigned c;
   const float* sk;  // this stage's k: component n at sk[n * kst]
   int kst;
-  __device__ __forceinline__ double q(int n) const { return __ldg(io.q + n * fs + c); }
+  __device__ __forceinline__ double q(int n) const { return at(io.q + n * fs, c); }
   __device__ __forceinline__ float k1(int n) const {
     if constexpr (STAGE == 1) return sk[n * kst];
-    else return __ldg(io.k1 + n * fs + c);
+    else return at(io.k1 + n * fs, c);
   }
   __device__ __forceinline__ float k2(int n) const { return sk[n * kst]; }
-  __device__ __forceinline__ float qfn(int n) const { return __ldg(io.qf_n + n * fs + c); }
+  __device__ __forceinline__ float qfn(int n) const { return at(io.qf_n + n * fs, c); }
   __device__ __forceinline__ float qs(int) const { return 0.f; }  // (FP32 pi storage is not fused)
 };
 
 // 128 registers (16 warps of 128-thread tiles per SM): with the rhs kernel's 96 the two phases
 // spilled 500 bytes per thread and the launch ran 10% slower.
-template <bool SINGLE, int STAGE, bool TH1, bool LEARNED>
+template <bool SINGLE, int STAGE, bool TH1, bool LEARNED, int TY, int TZ>
 __global__ void __maxnreg__(128)
     fused_kernel(const Params P, const StageIO<float> io, const UpdIO uio, const Work W,
                  const __grid_constant__ CUtensorMap map0, const CUtensorMap* __restrict__ tmaps) {
@@ -661,12 +678,14 @@ __global__ void __maxnreg__(128)
   extern __shared__ __align__(128) float s_raw[];
   __shared__ alignas(8) uint64_t s_bar[2];
   float* const s_q = s_raw + ((32u - ((smem_u32(s_raw) >> 2) & 31u)) & 31u);  // TMA wants 128-byte buffers
-  const int nthr = blockDim.x * blockDim.y * blockDim.z;
-  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int bx = blockDim.x + 4, by = blockDim.y + 4, bz = blockDim.z + 4;
+  const int ty = TY ? TY : (int)blockDim.y, tz = TZ ? TZ : (int)blockDim.z;
+  const int nthr = kTileX * ty * tz;
+  const int tid = threadIdx.x + kTileX * (threadIdx.y + ty * threadIdx.z);
+  constexpr int bx = kTileX + 4;
+  const int by = ty + 4, bz = tz + 4;
   const int vol = bx * by * bz;                  // floats per component in a buffer
   const unsigned box_bytes = 4u * kCompPerBox * vol;
-  const int bfl = rhs_buffer_floats(blockDim.x, blockDim.y, blockDim.z);
+  const int bfl = rhs_buffer_floats(kTileX, ty, tz);
   if (tid == 0) {
     mbar_init(&s_bar[0], 1);
     mbar_init(&s_bar[1], 1);
@@ -693,8 +712,8 @@ __global__ void __maxnreg__(128)
   int t0, t1;
   tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
-    const Tile tl = tile_at<SINGLE>(W, t);
-    const Lattice& L = SINGLE ? W.L0 : W.lats[tl.event];
+    const Tile tl = tile_at<SINGLE>(W, t, ty, tz);
+    const Lattice L = lattice_at<SINGLE>(W, tl.event);
     const CUtensorMap* map = SINGLE ? &map0 : tmaps + tl.event;
     if (t > t0 && __syncthreads_or(bad)) { bad = true; break; }  // every thread is done with both buffers
     if (tid == 0) {
@@ -706,7 +725,7 @@ __global__ void __maxnreg__(128)
 
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
     const bool valid = (i < L.nx) && (j < L.ny) && (k < L.nz);
-    const long long c = valid ? L.idx(i + 2, j + 2, k + 2) : 0;
+    const unsigned c = valid ? L.idx32(i + 2, j + 2, k + 2) : 0u;
     // ---- the right-hand side (as rhs_kernel)
     float dq[NQ], uc[4], du[4][4], dv = 0.f;
     Faces<float> Fx, Fy, Fz;
@@ -747,7 +766,7 @@ __global__ void __maxnreg__(128)
       for (int n = 0; n < NQ; ++n) sk[n * nthr] = dq[n] * dt;
     }
     // ---- the update (as update_kernel), reading k from shared memory
-    const UpdInFused<STAGE> in{uio, L.fstride, L.idx(i + 2, j + 2, k + 2), sk, nthr};
+    const UpdInFused<STAGE> in{uio, L.fstride, L.idx32(i + 2, j + 2, k + 2), sk, nthr};
     update_cell<STAGE, LEARNED, false, UpdInFused<STAGE>, true>(P, L, uio, in, i, j, k, tau_out, st, nit,
                                                                   nreg, nfb);
     fence_proxy_async_smem();  // this thread's generic accesses of the buffer before the next copy into it

@@ -130,7 +130,7 @@ __device__ __forceinline__ bool face_root(const Params& P, R E, R M2, R Pi, R gu
 // it was extrapolated from; v^d = M^d / (E + P0 + Pi) at the root, 0 for a state without one.
 template <typename R, int D, bool TH1>
 __device__ __forceinline__ void face_velocities_inverted(const Params& P, const Lattice& L, const StageIO<R>& io,
-                                                         long long c, int s, R th, R gnn, R& vLm, R& vLp, R& vRm,
+                                                         Idx<R> c, int s, R th, R gnn, R& vLm, R& vLp, R& vRm,
                                                          R& vRp) {
   const long long fs = L.fstride;
   const R h = R(0.5);
@@ -171,12 +171,13 @@ __device__ __forceinline__ void face_velocities_inverted(const Params& P, const 
 template <typename R>
 struct UGlobal {
   const R* u;
-  long long fs, c;
+  long long fs;
+  Idx<R> c;
   int sy, sz;  // row pitch, plane
   __device__ __forceinline__ R operator()(int m, int off) const { return ld<R>(u + m * fs, c + off); }
 };
 template <typename R>
-__device__ __forceinline__ UGlobal<R> u_global(const Lattice& L, const StageIO<R>& io, long long c) {
+__device__ __forceinline__ UGlobal<R> u_global(const Lattice& L, const StageIO<R>& io, Idx<R> c) {
   return UGlobal<R>{io.u_in, L.fstride, c, L.pitch, (int)L.plane};
 }
 
@@ -185,7 +186,7 @@ __device__ __forceinline__ UGlobal<R> u_global(const Lattice& L, const StageIO<R
 // d_d u^mu and v^d_{i+1} - v^d_{i-1}, and the pressure part of S_c (App. B):
 // -d_d (v^d P delta^nu_tau - g^{d nu} P), P = P0 + Pi.
 template <typename R, int D, bool TH1, bool IFACE, typename UA>
-__device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                            const UA& ua, const R (&uc)[4], R inv_gnn, R sfac, R (&dq)[NQ],
                                            R (&du)[4][4], R& dvd, float& amax, Faces<R>& F) {
   const long long fs = L.fstride;
@@ -299,7 +300,8 @@ __device__ __forceinline__ R component_flux(const R* p, int s, R a0, R th, const
   if constexpr (SMEM) {
     a2 = p[-2 * s]; a1 = p[-s]; b1 = p[s]; b2 = p[2 * s];
   } else {
-    a2 = ld<R>(p, -2 * s); a1 = ld<R>(p, -s); b1 = ld<R>(p, s); b2 = ld<R>(p, 2 * s);
+    const long long e = s;
+    a2 = ld<R>(p, -2 * e); a1 = ld<R>(p, -e); b1 = ld<R>(p, e); b2 = ld<R>(p, 2 * e);
   }
   const R d0 = a1 - a2, d1 = a0 - a1, d2 = b1 - a0, d3 = b2 - b1;
   R sm, s0, sp;
@@ -316,7 +318,7 @@ template <typename R, bool SMEM, bool TH1 = false>
 __device__ __forceinline__ void component_rhs(const Params& P, int n, const R* p, int sx, int sy, int sz, R th,
                                               const Faces<R>& Fx, const Faces<R>& Fy, const Faces<R>& Fz,
                                               R (&dq)[NQ]) {
-  const R a0 = SMEM ? p[0] : ld<R>(p, 0);
+  const R a0 = SMEM ? p[0] : ld<R>(p, 0LL);
   R a1x, b1x, a1y, b1y, a1z, b1z;
   R acc = component_flux<R, SMEM, TH1>(p, sx, a0, th, Fx, a1x, b1x, (Fx.c0 + Fy.c0 + Fz.c0) * a0);
   acc = component_flux<R, SMEM, TH1>(p, sy, a0, th, Fy, a1y, b1y, acc);
@@ -423,12 +425,13 @@ struct Stencil13 {
 template <typename R>
 __device__ __forceinline__ Stencil13<R> load_stencil(const R* p, const bool (&on)[3], const int (&s)[3]) {
   Stencil13<R> q;
-  q.a0 = ld<R>(p, 0);
+  q.a0 = ld<R>(p, 0LL);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     q.v[d][0] = q.v[d][1] = q.v[d][2] = q.v[d][3] = R(0);
     if (on[d]) {
-      q.v[d][0] = ld<R>(p, -2 * s[d]); q.v[d][1] = ld<R>(p, -s[d]); q.v[d][2] = ld<R>(p, s[d]); q.v[d][3] = ld<R>(p, 2 * s[d]);
+      const long long e = s[d];
+      q.v[d][0] = ld<R>(p, -2 * e); q.v[d][1] = ld<R>(p, -e); q.v[d][2] = ld<R>(p, e); q.v[d][3] = ld<R>(p, 2 * e);
     }
   }
   return q;
@@ -467,7 +470,7 @@ __device__ __forceinline__ R sum_c0(const Faces<R> (&F)[3], const bool (&on)[3])
 }
 
 template <typename R, bool TH1 = false>
-__device__ __forceinline__ void conserved_fluxes(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void conserved_fluxes(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                                  const Faces<R> (&F)[3], R (&dq)[NQ]) {
   const long long fs = L.fstride;
   const R th = pr<R>(P).theta;
@@ -709,18 +712,18 @@ __device__ __forceinline__ R regulator_factor(const Params& P, R gnn, R sqrt_gnn
 
 // ---------------------------------------------------------------- f) stores with ghosts
 template <typename R>
-__device__ __forceinline__ void store_cell(const StageIO<R>& io, long long fs, long long t, const double (&qn)[NQ],
+__device__ __forceinline__ void store_cell(const StageIO<R>& io, long long fs, Idx<R> t, const double (&qn)[NQ],
                                            const R (&qr)[NQ], const R (&uo)[4], R e, R P0) {
 #pragma unroll
-  for (int n = 0; n < NQ; ++n) io.q_out[n * fs + t] = qn[n];
+  for (int n = 0; n < NQ; ++n) put(io.q_out + n * fs, t, qn[n]);
   if (io.qr_out) {
 #pragma unroll
-    for (int n = 0; n < NQ; ++n) io.qr_out[n * fs + t] = qr[n];
+    for (int n = 0; n < NQ; ++n) put(io.qr_out + n * fs, t, qr[n]);
   }
 #pragma unroll
-  for (int m = 0; m < 4; ++m) io.u_out[m * fs + t] = uo[m];
-  io.e_out[t] = e;
-  io.p_out[t] = P0;
+  for (int m = 0; m < 4; ++m) put(io.u_out + m * fs, t, uo[m]);
+  put(io.e_out, t, e);
+  put(io.p_out, t, P0);
 }
 
 // padded ghost coordinate g in {0, 1, n+2, n+3} that copies the physical padded coordinate p
@@ -729,24 +732,21 @@ __device__ __forceinline__ int ghost_source(int g, int n, int periodic) {
   return (g < 2) ? 2 : n + 1;
 }
 
-// calls put(t) for the element index t of the padded cell (i, j, k) and of every ghost cell that
-// copies it (Eqs. ghostCells_1/2, or the periodic images)
-template <typename F>
-__device__ __forceinline__ void for_cell_and_ghosts(const Params& P, const Lattice& L, int i, int j, int k, F&& put) {
-  put(L.idx(i, j, k));
-  const int nn[3] = {L.nx, L.ny, L.nz};
-  const int pc[3] = {i, j, k};
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    int n = nn[ax];
-    if (pc[ax] > 3 && pc[ax] < n) continue;  // interior cells own no ghost
-    const int gs[4] = {0, 1, n + 2, n + 3};
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      if (ghost_source(gs[g], n, P.periodic) != pc[ax]) continue;
-      int ii = (ax == 0) ? gs[g] : i, jj = (ax == 1) ? gs[g] : j, kk = (ax == 2) ? gs[g] : k;
-      put(L.idx(ii, jj, kk));
-    }
+// calls f(t) for the element index t = t0 of the padded cell (i, j, k) and of every ghost cell that
+// copies it (Eqs. ghostCells_1/2, or the periodic images).  The ghosts of a boundary cell go through one
+// rolled loop: unrolled, its twelve copies of the stores were most of the kernels' code.
+template <typename I, typename F>
+__device__ __forceinline__ void for_cell_and_ghosts(const Params& P, const Lattice& L, I t0, int i, int j, int k, F&& f) {
+  f(t0);
+  if (i > 3 && i < L.nx && j > 3 && j < L.ny && k > 3 && k < L.nz) return;  // interior cells own no ghost
+#pragma unroll 1
+  for (int a = 0; a < 12; ++a) {
+    const int ax = a >> 2, g = a & 3;
+    const int n = (ax == 0) ? L.nx : ((ax == 1) ? L.ny : L.nz), p = (ax == 0) ? i : ((ax == 1) ? j : k);
+    const int pos = (g < 2) ? g : n + g;
+    if (ghost_source(pos, n, P.periodic) != p) continue;
+    const long long step = (ax == 0) ? 1 : ((ax == 1) ? (long long)L.pitch : L.plane);
+    f((I)(t0 + (I)((pos - p) * step)));
   }
 }
 
@@ -755,7 +755,8 @@ __device__ __forceinline__ void store_with_ghosts(const Params& P, const Lattice
                                                   int j, int k, const double (&qn)[NQ], const R (&qr)[NQ],
                                                   const R (&uo)[4], R e, R P0) {
   const long long fs = L.fstride;
-  for_cell_and_ghosts(P, L, i, j, k, [&](long long t) { store_cell<R>(io, fs, t, qn, qr, uo, e, P0); });
+  for_cell_and_ghosts(P, L, cell_idx<R>(L, i, j, k), i, j, k,
+                      [&](Idx<R> t) { store_cell<R>(io, fs, t, qn, qr, uo, e, P0); });
 }
 
 // ---------------------------------------------------------------- a) + b) for one cell
@@ -785,7 +786,7 @@ __device__ __forceinline__ R divergence(const Params& P, const R (&d)[3]) {
 
 // the three directions' face setups; uc returns u^mu at the cell
 template <typename R, bool TH1, bool IFACE, typename UA>
-__device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                            const UA& ua, const CellGeom<R>& G, R (&dq)[NQ], R (&uc)[4],
                                            R (&du)[4][4], R& dv, float& amax, Faces<R>& Fx, Faces<R>& Fy,
                                            Faces<R>& Fz) {
@@ -811,12 +812,12 @@ __device__ __forceinline__ void cell_faces(const Params& P, const Lattice& L, co
 }
 
 template <typename R, bool DIAG = false>
-__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                              const CellGeom<R>& G, const R (&uc)[4], R (&du)[4][4], R dv,
                                              R (&dq)[NQ], R* dg = nullptr);
 
 template <typename R, bool TH1 = false, bool IFACE = false>
-__device__ __forceinline__ void cell_rhs(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void cell_rhs(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                          double tau_src, R (&dq)[NQ], float& amax) {
   const CellGeom<R> G = cell_geom<R>(P, tau_src);
   R uc[4], du[4][4];
@@ -833,7 +834,7 @@ __device__ __forceinline__ void cell_rhs(const Params& P, const Lattice& L, cons
 // |theta|) with J^{mu nu}, J the second-order terms of Eq. (14_moment_terms) (no diffusion); a
 // quantity whose channel is off, or whose denominator vanishes, is 0.
 template <typename R, bool DIAG>
-__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                              const CellGeom<R>& G, const R (&uc)[4], R (&du)[4][4], R dv,
                                              R (&dq)[NQ], R* dg) {
   if constexpr (DIAG) {
@@ -1248,7 +1249,7 @@ __global__ void __launch_bounds__(32, 8)
 enum : int { TM_FACE = 0, TM_DU = 18, TM_DV = 30, TM_PR = 33, TM_ACC = 39, TM_MIX = 54, TM_DIFF = 58, TM_VALUES = 70 };
 
 template <typename R, int D, bool TH1>
-__device__ __forceinline__ void team_faces(const Params& P, const Lattice& L, const StageIO<R>& io, long long c,
+__device__ __forceinline__ void team_faces(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
                                            const CellGeom<R>& G, R (*sm)[32], float& amax) {
   const int lane = threadIdx.x & 31;
   const UGlobal<R> ua = u_global(L, io, c);
