@@ -71,7 +71,7 @@ struct Ctx {
   RootSeg* seg_r = nullptr;
   RootSegM* seg_m = nullptr;
   FaceSeg* seg_face = nullptr;
-  double* d_tau = nullptr;  // three slots, used in rotation with the u buffers: tau^n is in slot cur
+  TauSlot* d_tau = nullptr;  // three slots, used in rotation with the u buffers: tau^n is in slot cur
   unsigned* d_stat = nullptr;
   float* d_mlp = nullptr;
   uint32_t* d_mlp_packed = nullptr;
@@ -343,11 +343,11 @@ __device__ __forceinline__ void cell_coords(const Lattice& L, unsigned o, int& i
 // 26.5 -> 22.7 ms; a 64 x 64 x 48 output to the host (31 fields, diagnostics) 1.1 -> 0.72 ms.
 template <typename R>
 __global__ void __launch_bounds__(256)
-    set_state_kernel(const Params P, const Lattice L, const Primaries in, double tau, double* tau_slot, double* q,
+    set_state_kernel(const Params P, const Lattice L, const Primaries in, double tau, TauSlot* slot, double* q,
                      float* qf, R* U, R* Up, R* E, R* Pb, float* reg, unsigned* status) {
   const unsigned ncp = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
   const unsigned o = blockIdx.x * 256u + threadIdx.x;
-  if (o == 0) *tau_slot = tau;
+  if (o == 0) *slot = tau_slot(tau, P.dtau, P.milne);
   if (o >= ncp) return;
   int i, j, k;
   cell_coords(L, o, i, j, k);
@@ -611,7 +611,7 @@ StageIO<R> make_io(Ctx* c, int stage) {
     io.qr_in = (const R*)io.q_in;
     io.qr_out = nullptr;
   }
-  io.d_tau = c->d_tau + c->cur;
+  io.tau = c->d_tau + c->cur;
   io.tau_next = (stage == 2) ? c->d_tau + c->spare : nullptr;  // the next step's u^n buffer and tau slot
   io.status = c->d_stat;
   io.max_speed_bits = c->d_stat + 1;
@@ -638,7 +638,7 @@ UpdIO make_uio(Ctx* c, int stage) {
   u.e_out = io.e_out;
   u.p_out = io.p_out;
   u.e_guess = io.e_in;
-  u.d_tau = io.d_tau;
+  u.tau = io.tau;
   u.tau_next = io.tau_next;
   u.status = c->d_stat;
   u.counters = (unsigned long long*)(c->d_stat + 4);
@@ -1149,6 +1149,7 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   P.rho_max = o.rho_max;
   P.xi0 = o.xi0;
   P.e_min = o.e_min;
+  P.root_lo = (o.e_min > 0.0) ? o.e_min : 1e-300;
   P.rate_max = (o.tau_relax_min > 0) ? 1.0 / o.tau_relax_min : INFINITY;
   P.ln_rate_max = std::log(P.rate_max);
   fill_pr<double>(P.pd, P);
@@ -1205,7 +1206,7 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->seg_r = (RootSeg*)carve(nseg * sizeof(RootSeg));
   c->seg_m = (RootSegM*)carve(nseg * sizeof(RootSegM));
   c->seg_face = (FaceSeg*)carve(nseg * sizeof(FaceSeg));
-  c->d_tau = (double*)carve(256);
+  c->d_tau = (TauSlot*)carve(256);
   c->d_stat = (unsigned*)carve(256);
   c->d_mlp = (float*)carve(KT_MLP_NPARAM * 4);
   c->d_mlp_packed = (uint32_t*)carve(KT_MLP_PACKED_BYTES);
@@ -1308,7 +1309,7 @@ int kt_set_state_event(kt_ctx* c, int event, double tau, const double* e, const 
   }
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   const unsigned nb = (unsigned)((ncp + 255) / 256);
-  double* slot = c->d_tau + c->cur;
+  TauSlot* slot = c->d_tau + c->cur;
   // the state goes into the buffers that hold u^n and u^{n-1} in the current rotation
   if (c->mixed)
     set_state_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L, in, tau, slot, c->q, c->qf, (float*)c->U[c->cur],
@@ -1560,8 +1561,8 @@ int kt_set_checkpoint(kt_ctx* c, int event, double tau, const double* buf, int o
     }
     CK(cudaGetLastError());
   }
-  double tau_h = tau;
-  CK(cudaMemcpyAsync(c->d_tau + c->cur, &tau_h, 8, cudaMemcpyHostToDevice, c->stream));
+  const TauSlot slot = tau_slot(tau, c->P.dtau, c->P.milne);
+  CK(cudaMemcpyAsync(c->d_tau + c->cur, &slot, sizeof(slot), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->tau = tau;

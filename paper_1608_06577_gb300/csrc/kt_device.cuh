@@ -53,6 +53,17 @@ __device__ __forceinline__ Idx<R> cell_idx(const Lattice& L, int i, int j, int k
   else return L.idx(i, j, k);
 }
 
+// tau^n of a step and what every cell derives from it, written once per step: on the FP64 pipe each of
+// these operations costs every warp as much as one of the root-find's
+struct TauSlot {
+  double tau, tau_out, gnn_out;  // tau^n, tau^{n+1}, g_{eta eta} there (tau^2; 1 in Cartesian coordinates)
+  double unused;
+};
+__host__ __device__ __forceinline__ TauSlot tau_slot(double tau, double dtau, int milne) {
+  const double o = tau + dtau;
+  return TauSlot{tau, o, milne ? o * o : 1.0, 0.0};
+}
+
 // a block-shaped tile of one event: the persistent stage kernel walks a table of these
 struct Tile {
   int event, i0, j0, k0;
@@ -139,6 +150,7 @@ struct Params {
   int mlp_infer;      // learned start: 1 runs the network (KT_INV_LEARNED), 0 starts from e_conf alone
   double rho_max, xi0;
   double e_min;
+  double root_lo;     // lower end of the root-finds' bracket: e_min, or 1e-300
   double rate_max;    // 1 / tau_relax_min (or +inf)
   double ln_rate_max;
   PR<double> pd;

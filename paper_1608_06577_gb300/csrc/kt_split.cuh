@@ -33,8 +33,8 @@ struct UpdIO {
   float* e_out;
   float* p_out;
   const float* e_guess;     // the cell's previous energy density: the plain root-find's start
-  const double* d_tau;      // tau^n
-  double* tau_next;         // stage 2: where tau^{n+1} goes
+  const TauSlot* tau;       // this step's tau
+  TauSlot* tau_next;        // stage 2: where the next step's goes
   unsigned* status;
   unsigned long long* counters;
   float* reg_out;           // stage 2: the regulation factor applied at each cell, or null
@@ -122,8 +122,7 @@ __global__ void __maxnreg__(96)
   float amax = 0.f;
   bool bad = false;
   unsigned issued = 0, done = 0;  // TMA copies issued and waited for (the same in every thread)
-  const double tau_n = io.d_tau[0];
-  const CellGeom<float> G = cell_geom<float>(P, (stage == 1) ? tau_n : tau_n + P.dtau);
+  const CellGeom<float> G = cell_geom<float>(P, (stage == 1) ? io.tau->tau : io.tau->tau_out);
   const float th = pr<float>(P).theta;
   const int sy = bx, sz = bx * by;
   const int own = ((int)threadIdx.z + 2) * sz + ((int)threadIdx.y + 2) * sy + (int)threadIdx.x + 2;
@@ -208,9 +207,15 @@ __device__ __forceinline__ unsigned thr_hi(float t) {
   const unsigned b = __float_as_uint(t);
   return (b >= 0x00800000u && b < 0x7f800000u) ? (b >> 3) + (896u << 20) : 0u;
 }
+// The update kernels are bound by the FP64 pipe (stage 2: 57 instructions per cell at 19 cycles per warp
+// and SM), and the second Newton step needs almost none of it: with |de| < 2^-19 E the new residual
+//   g(e + de) = g + de A + (e + de - E) dP,  dP = c_s^2 de,
+// in single precision is good to a few 2^-24 |de| A, i.e. 3e-13 E A, and dP's next term to 2e-13 E, both
+// inside the threshold's margin; e and P0 take one FP64 addition each.  128^3: updates 206 / 277 ->
+// 192 / 263 us (with tau's squares formed once per step), step 0.906 -> 0.868 ms.
 __device__ __forceinline__ unsigned rootfind_learned(const Params& P, const InvIn& v, double EPi, double e_start,
                                                      double& e, double& P0, unsigned& iters, unsigned& fallbacks) {
-  const double lo = (P.e_min > 0.0) ? P.e_min : 1e-300;
+  const double lo = P.root_lo;
   // (E >= 2^120, beyond where the truncated E and A are valid single-precision values: no
   // acceptance, the plain root-find decides)
   const float tolf = (obits(v.E) < 0x4770000000000000LL) ? 0.99e-10f * v.Ef : 0.f;
@@ -223,8 +228,19 @@ __device__ __forceinline__ unsigned rootfind_learned(const Params& P, const InvI
       return 0u;
     }
     if (kk == 2) break;
-    e = clamp_pos(newton_step(e, r), lo, v.E);
+    const float gf = d2f_trunc(r.g), de = rmul(-gf, __frcp_rn(r.gp));
     ++iters;
+    if (kk == 1 && fabsf(de) < 0x1p-19f * v.Ef && tolf > 0.f) {
+      const float dP = r.c2 * de;
+      const double en = e + f2d_bits(de);
+      if (obits(en) >= obits(lo) && obits(en) <= obits(v.E) &&
+          fabsf(fmaf(r.emf + de, dP, fmaf(de, r.Af, gf))) < tolf * r.Af) {
+        e = en;
+        P0 = r.p0 + f2d_bits(dP);
+        return 0u;
+      }
+    }
+    e = clamp_pos(newton_step(e, r), lo, v.E);
   }
   ++fallbacks;
   return rootfind_plain(P, v.E, EPi, v.M2, v.M2f, e, e, P0, iters);
@@ -319,7 +335,7 @@ __device__ __forceinline__ float pi32_state(const In& in, int n) {
 // to the field array for the second stage, its pi components carrying the regulator's rescaling.
 template <int STAGE, bool LEARNED, bool PI32, typename In, bool STORE_K1 = false>
 __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, const UpdIO& io, const In& in, int i,
-                                            int j, int k, double tau_out, unsigned& st,
+                                            int j, int k, const TauSlot& tau, unsigned& st,
                                             unsigned& nit, unsigned& nreg, unsigned& nfb) {
   const bool valid = (i < L.nx) && (j < L.ny) && (k < L.nz);
   const long long fs = L.fstride;
@@ -358,8 +374,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
     }
   }
 
-  const double gnn = P.milne ? tau_out * tau_out : 1.0;
-  const InvIn v = inv_in(gnn, E, Mx, My, Mn, Pi);
+  const InvIn v = inv_in(tau.gnn_out, E, Mx, My, Mn, Pi);
   double start;
   if constexpr (LEARNED) {
     start = learned_start(v, valid ? at(io.z_net, c) : 0.f);
@@ -413,7 +428,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
   // e) regulator (Eq. regPimunu), after the root-find, on pi only
   bool k1_pi_written = false;  // STORE_K1: the pi components of k_1 were written rescaled
   if (P.regulate) {
-    const float go = P.milne ? from_f64<float>(tau_out * tau_out) : 1.f;
+    const float go = from_f64<float>(tau.gnn_out);
     float pm[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -422,7 +437,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
         pm[a][b] = qr[pix(a, b)];
         pm[b][a] = pm[a][b];
       }
-    const float f = regulator_factor<float>(P, go, from_f64<float>(tau_out), eR, P0R, uo, pm, qr[14]);
+    const float f = regulator_factor<float>(P, go, from_f64<float>(tau.tau_out), eR, P0R, uo, pm, qr[14]);
     if (f < 0.999f) ++nreg;
     if (STAGE == 2 && io.reg_out) put(io.reg_out, c, f);
     if (f != 1.f) {
@@ -483,7 +498,7 @@ __device__ __forceinline__ void update_cell(const Params& P, const Lattice& L, c
 template <bool SINGLE, int STAGE, bool LEARNED, bool PI32>
 __global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, const UpdIO io, const Work W) {
   unsigned st = 0, nit = 0, nreg = 0, nfb = 0;
-  const double tau_out = io.d_tau[0] + P.dtau;
+  const TauSlot tau = *io.tau;
   int t0, t1;
   tile_range(W.ntiles, t0, t1);
   for (int t = t0; t < t1; ++t) {
@@ -491,9 +506,9 @@ __global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, 
     const Lattice L = lattice_at<SINGLE>(W, tl.event);
     const int i = tl.i0 + (int)threadIdx.x, j = tl.j0 + (int)threadIdx.y, k = tl.k0 + (int)threadIdx.z;
     const UpdInGlobal in{io, L.fstride, L.idx32(i + 2, j + 2, k + 2)};
-    update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau_out, st, nit, nreg, nfb);
+    update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau, st, nit, nreg, nfb);
   }
-  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && (threadIdx.x | threadIdx.y | threadIdx.z) == 0);
+  if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && (threadIdx.x | threadIdx.y | threadIdx.z) == 0);
   block_stats(io.status, nullptr, io.counters, st, 0.f, nit, nreg, nfb);
 }
 
@@ -506,13 +521,13 @@ __global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, 
 // differ from q^n by O(dtau).  Run in a launch of its own, at full occupancy, the inference's
 // latency hides behind other warps; inside the register-capped update it could not.
 __global__ void __launch_bounds__(256) mlp_start_kernel(const float* __restrict__ qf, long long fs,
-                                                        const double* __restrict__ d_tau, int milne,
+                                                        const TauSlot* __restrict__ tau_n, int milne,
                                                         const uint32_t* __restrict__ packed,
                                                         float* __restrict__ z_net) {
   __shared__ alignas(16) uint32_t sw[PK_WORDS];
   mlp_load_shared(sw, packed);
   __syncthreads();
-  const float tau = d2f_trunc(d_tau[0]);
+  const float tau = d2f_trunc(tau_n->tau);
   const float gnn = milne ? tau * tau : 1.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long base = (long long)blockIdx.x * blockDim.x; base < fs; base += stride) {  // block-uniform
@@ -588,7 +603,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
   unsigned st = 0, nit = 0, nreg = 0, nfb = 0;
   bool bad = false;
   unsigned issued = 0, done = 0;  // tiles whose copies were issued / waited for (the same in every thread)
-  const double tau_out = io.d_tau[0] + P.dtau;
+  const TauSlot tau = *io.tau;
   int t0, t1;
   tile_range(ntiles, t0, t1);
   auto issue = [&](int t, unsigned slot) {  // thread 0 only: the four (stage 2) or five copies of tile t
@@ -629,7 +644,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
     const UpdInShared<STAGE> in{(const double*)buf, (const float*)(buf + qbytes), (const float*)(buf + qbytes + kbytes),
                                 bc, own};
     update_cell<STAGE, LEARNED, false>(P, L, io, in, tl.i0 + (int)threadIdx.x, tl.j0 + (int)threadIdx.y,
-                                       tl.k0 + (int)threadIdx.z, tau_out, st, nit, nreg, nfb);
+                                       tl.k0 + (int)threadIdx.z, tau, st, nit, nreg, nfb);
     if (nbuf == 1 && t + 1 < t1) {  // single buffer: refill it once every thread is done with it
       if (__syncthreads_or(bad)) { bad = true; break; }
       if (tid == 0) issue(t + 1, 0u);
@@ -640,7 +655,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
     for (; done < issued; ++done)
       mbar_wait(&s_bar[(nbuf == 2) ? (done & 1u) : 0u], (nbuf == 2) ? ((done >> 1) & 1u) : (done & 1u), kWaitPolls);
   }
-  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && tid == 0);
+  if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && tid == 0);
   block_stats(io.status, nullptr, io.counters, st | (bad ? ST_TIMEOUT : 0u), 0.f, nit, nreg, nfb);
 }
 
@@ -696,9 +711,8 @@ __global__ void __maxnreg__(128)
   bool bad = false;
   unsigned issued = 0, done = 0;  // TMA copies issued and waited for (the same in every thread)
   unsigned st = 0, nit = 0, nreg = 0, nfb = 0;
-  const double tau_n = io.d_tau[0];
-  const double tau_out = tau_n + P.dtau;
-  const CellGeom<float> G = cell_geom<float>(P, (STAGE == 1) ? tau_n : tau_out);
+  const TauSlot tau = *io.tau;
+  const CellGeom<float> G = cell_geom<float>(P, (STAGE == 1) ? tau.tau : tau.tau_out);
   const float th = pr<float>(P).theta;
   const int sy = bx, sz = bx * by;
   const int own = ((int)threadIdx.z + 2) * sz + ((int)threadIdx.y + 2) * sy + (int)threadIdx.x + 2;
@@ -767,14 +781,14 @@ __global__ void __maxnreg__(128)
     }
     // ---- the update (as update_kernel), reading k from shared memory
     const UpdInFused<STAGE> in{uio, L.fstride, L.idx32(i + 2, j + 2, k + 2), sk, nthr};
-    update_cell<STAGE, LEARNED, false, UpdInFused<STAGE>, true>(P, L, uio, in, i, j, k, tau_out, st, nit,
+    update_cell<STAGE, LEARNED, false, UpdInFused<STAGE>, true>(P, L, uio, in, i, j, k, tau, st, nit,
                                                                   nreg, nfb);
     fence_proxy_async_smem();  // this thread's generic accesses of the buffer before the next copy into it
   }
   if (bad) {  // a copy did not complete in time: let the ones in flight land before the block exits
     for (; done < issued; ++done) mbar_wait(&s_bar[done & 1u], (done >> 1) & 1u, kWaitPolls);
   }
-  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && tid == 0);
+  if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && tid == 0);
   block_stats(io.status, io.max_speed_bits, io.counters, st | (bad ? ST_TIMEOUT : 0u), amax, nit, nreg, nfb);
 }
 

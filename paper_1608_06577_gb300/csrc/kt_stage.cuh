@@ -32,8 +32,8 @@ struct StageIO {
   const R* p_in;
   R* e_out;
   R* p_out;
-  const double* d_tau;   // tau^n
-  double* tau_next;      // stage 2: where tau^{n+1} goes (another slot than d_tau), else null
+  const TauSlot* tau;    // this step's tau
+  TauSlot* tau_next;     // stage 2: where the next step's goes (another slot), else null
   unsigned* status;
   unsigned* max_speed_bits;
   unsigned long long* counters;  // [0] Newton iterations, [1] regulated cells, [2] fallbacks
@@ -571,7 +571,7 @@ __device__ __forceinline__ double seg_P(const RootSegM& s, double d, float df) {
 // the learned start's Newton steps use it.
 struct Resid {
   double g, A, p0;
-  float gp, Af;
+  float gp, Af, c2, emf;  // A f', A, c_s^2, e - E
 };
 template <bool MIXED>
 __device__ __forceinline__ Resid residual(const Params& P, double e, double E, double EPi, double M2, float M2f) {
@@ -583,9 +583,10 @@ __device__ __forceinline__ Resid residual(const Params& P, double e, double E, d
   r.A = EPi + r.p0;
   const double em = e - E;
   r.g = fma(em, r.A, M2);
-  const float c2 = fmaf(df, fmaf(df, s.b3, s.b2), s.b1);
+  r.c2 = fmaf(df, fmaf(df, s.b3, s.b2), s.b1);
+  r.emf = d2f_trunc(em);
   r.Af = d2f_trunc(r.A);
-  r.gp = r.Af - __fdividef(M2f * c2, r.Af);
+  r.gp = r.Af - __fdividef(M2f * r.c2, r.Af);
   return r;
 }
 
@@ -606,7 +607,7 @@ __device__ __forceinline__ double eos_P_pos(const Params& P, double e) {
 // the exponent lowered by 50 (exact for E >= 2^-972; smaller E stops only at de = 0).
 __device__ __forceinline__ unsigned rootfind_plain(const Params& P, double E, double EPi, double M2, float M2f,
                                                    double start, double& e, double& P0, unsigned& iters) {
-  double lo = (P.e_min > 0.0) ? P.e_min : 1e-300, hi = E;
+  double lo = P.root_lo, hi = E;
   e = (obits(start) >= obits(lo) && obits(start) <= obits(hi)) ? start : hi;
   const long long stop = max(obits(E) - (50LL << 52), 0LL);
   int it;
@@ -1148,8 +1149,8 @@ __device__ __forceinline__ void stage_finish(const Params& P, const Lattice& L, 
 
 // tau^{n+1} for the next step, written by one thread of the second stage into another slot than the one
 // this step's kernels read (a launch of its own cost 2 us per step: 4% of a small grid's)
-__device__ __forceinline__ void advance_tau(const Params& P, const double* d_tau, double* tau_next, bool first) {
-  if (tau_next && first) *tau_next = d_tau[0] + P.dtau;
+__device__ __forceinline__ void advance_tau(const Params& P, const TauSlot* tau, TauSlot* tau_next, bool first) {
+  if (tau_next && first) *tau_next = tau_slot(tau->tau_out, P.dtau, P.milne);
 }
 
 // The contiguous run [t0, t1) of the tile table that this block processes.  Tiles are ordered
@@ -1231,12 +1232,12 @@ __global__ void __launch_bounds__(32, 8)
     first = (unsigned)s.i0;
   }
   const CellAt at = cell_at(L, first + threadIdx.x);
-  const double tau_n = io.d_tau[0], tau_out = tau_n + P.dtau;
+  const double tau_n = io.tau->tau, tau_out = io.tau->tau_out;
   R dq[NQ];
   cell_rhs<R, TH1, IFACE>(P, L, io, at.c, (STAGE == 1) ? tau_n : tau_out, dq, amax);
   stage_finish<R, STAGE>(P, L, io, at, tau_out, dq, st, nit, nreg);
   __syncwarp();
-  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
+  if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
   warp_stats(io, st, amax, nit, nreg);
 }
 
@@ -1288,7 +1289,7 @@ __global__ void __launch_bounds__(128, 2)
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const CellAt at = cell_at(L, first + lane);
-  const double tau_n = io.d_tau[0], tau_out = tau_n + P.dtau;
+  const double tau_n = io.tau->tau, tau_out = io.tau->tau_out;
   const CellGeom<R> G = cell_geom<R>(P, (STAGE == 1) ? tau_n : tau_out);
   const long long fs = L.fstride, c = at.c;
   const bool on[3] = {L.nx > 1, L.ny > 1, L.nz > 1};
@@ -1356,7 +1357,7 @@ __global__ void __launch_bounds__(128, 2)
   cell_sources<R>(P, L, io, c, G, uc, du, divergence<R>(P, d), dq);
   stage_finish<R, STAGE>(P, L, io, at, tau_out, dq, st, nit, nreg);
   __syncwarp();
-  if (STAGE == 2) advance_tau(P, io.d_tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
+  if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
   warp_stats(io, st, amax, nit, nreg);
 }
 
