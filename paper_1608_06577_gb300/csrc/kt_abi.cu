@@ -319,8 +319,6 @@ void build_mixed_root_segments(const std::vector<RootSeg>& sr, std::vector<RootS
 }
 
 // ------------------------------------------------------------------ small kernels
-__device__ __forceinline__ double gnn_at(const Params& P, double tau) { return P.milne ? tau * tau : 1.0; }
-
 // The primaries of kt_set_state: packed physical arrays on the device, null where not given
 struct Primaries {
   const double *e, *u, *pi, *Pi, *u_prev;
@@ -341,23 +339,23 @@ __device__ __forceinline__ void cell_coords(const Lattice& L, unsigned o, int& i
 // themselves (host arrays come through the staging area).  With the gather below, set and get of a 128^3
 // event on the device: six learned steps between them 7.13 -> 6.79 ms, six steps of a 16-event batch
 // 26.5 -> 22.7 ms; a 64 x 64 x 48 output to the host (31 fields, diagnostics) 1.1 -> 0.72 ms.
+constexpr int kSetThreads = 128;
 template <typename R>
-__global__ void __launch_bounds__(256)
-    set_state_kernel(const Params P, const Lattice L, const Primaries in, double tau, TauSlot* slot, double* q,
-                     float* qf, R* U, R* Up, R* E, R* Pb, float* reg, unsigned* status) {
+__global__ void __launch_bounds__(kSetThreads, 4)
+    set_state_kernel(const Params P, const Lattice L, const Primaries in, double tau, double g, double gp, TauSlot* slot,
+                     double* q, float* qf, R* U, R* Up, R* E, R* Pb, float* reg, unsigned* status) {
   const unsigned ncp = (unsigned)L.nx * (unsigned)L.ny * (unsigned)L.nz;
-  const unsigned o = blockIdx.x * 256u + threadIdx.x;
+  const unsigned o = blockIdx.x * kSetThreads + threadIdx.x;
   if (o == 0) *slot = tau_slot(tau, P.dtau, P.milne);
   if (o >= ncp) return;
   int i, j, k;
   cell_coords(L, o, i, j, k);
   const double e = in.e[o];
   double u4[4] = {1.0, 0.0, 0.0, 0.0}, up4[4], pi[10];
-  const double g = gnn_at(P, tau);
   if (in.u) {
 #pragma unroll
     for (int m = 0; m < 3; ++m) u4[m + 1] = in.u[(size_t)m * ncp + o];
-    u4[0] = sqrt(1.0 + u4[1] * u4[1] + u4[2] * u4[2] + g * u4[3] * u4[3]);
+    u4[0] = sqrt(fma(g * u4[3], u4[3], fma(u4[2], u4[2], fma(u4[1], u4[1], 1.0))));
   }
 #pragma unroll
   for (int m = 0; m < 10; ++m) pi[m] = in.pi ? in.pi[(size_t)m * ncp + o] : 0.0;
@@ -367,8 +365,7 @@ __global__ void __launch_bounds__(256)
   if (in.u_prev) {
 #pragma unroll
     for (int m = 0; m < 3; ++m) up4[m + 1] = in.u_prev[(size_t)m * ncp + o];
-    const double gp = gnn_at(P, tau - P.dtau);
-    up4[0] = sqrt(1.0 + up4[1] * up4[1] + up4[2] * up4[2] + gp * up4[3] * up4[3]);
+    up4[0] = sqrt(fma(gp * up4[3], up4[3], fma(up4[2], up4[2], fma(up4[1], up4[1], 1.0))));
   }
   const double P0 = eos_P<double>(P, e), Pt = P0 + Pi, w = (e + Pt) * u4[0];
   double qn[NQ];
@@ -386,8 +383,18 @@ __global__ void __launch_bounds__(256)
   if (bad) atomicOr(status, ST_NONFINITE);
   // the inversion of Eq. (eInferred) needs E = T^{tau tau} - pi^{tau tau} > 0 and M^2 < E^2 with
   // M^i = T^{tau i} - pi^{tau i}, M^2 = M_x^2 + M_y^2 + g_{eta eta} M_eta^2 (Sec. 2.4)
-  const double Ei = qn[0] - qn[4], Mx = qn[1] - qn[5], My = qn[2] - qn[6], Mn = qn[3] - qn[7];
-  if (!bad && !(pos(Ei) && obits(Mx * Mx + My * My + g * Mn * Mn) < obits(Ei * Ei))) atomicOr(status, ST_INVERSION);
+  // Decided in single precision where that is certain: E and M within 2^60 of one, M^2 < 0.99 E^2 and a
+  // pi^{tau mu} no larger than E, so that the difference's rounding stays far inside the margin.
+  const float Ef = d2f_trunc(qn[0]) - d2f_trunc(qn[4]), gf = d2f_trunc(g);
+  const float mx = d2f_trunc(qn[1]) - d2f_trunc(qn[5]), my = d2f_trunc(qn[2]) - d2f_trunc(qn[6]),
+              mn = d2f_trunc(qn[3]) - d2f_trunc(qn[7]);
+  const bool sure = Ef > 0x1p-60f && Ef < 0x1p60f && fmaf(gf * mn, mn, fmaf(my, my, mx * mx)) < 0.99f * Ef * Ef &&
+                    fabsf(d2f_trunc(qn[4])) < Ef && fabsf(d2f_trunc(qn[5])) < Ef && fabsf(d2f_trunc(qn[6])) < Ef &&
+                    gf * d2f_trunc(qn[7]) * d2f_trunc(qn[7]) < Ef * Ef && fabsf(d2f_trunc(qn[0])) < 0x1p60f;
+  if (!bad && !sure) {
+    const double Ei = qn[0] - qn[4], Mx = qn[1] - qn[5], My = qn[2] - qn[6], Mn = qn[3] - qn[7];
+    if (!(pos(Ei) && obits(Mx * Mx + My * My + g * Mn * Mn) < obits(Ei * Ei))) atomicOr(status, ST_INVERSION);
+  }
   const long long fs = L.fstride;
   reg[L.idx(i, j, k)] = 1.f;  // no regulation recorded yet
   float qs[NQ];
@@ -1308,15 +1315,16 @@ int kt_set_state_event(kt_ctx* c, int event, double tau, const double* e, const 
     CK(up(in.u_prev, 15, 3));
   }
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
-  const unsigned nb = (unsigned)((ncp + 255) / 256);
+  const unsigned nb = (unsigned)((ncp + kSetThreads - 1) / kSetThreads);
+  const double g = c->P.milne ? tau * tau : 1.0, gp = c->P.milne ? (tau - c->P.dtau) * (tau - c->P.dtau) : 1.0;
   TauSlot* slot = c->d_tau + c->cur;
   // the state goes into the buffers that hold u^n and u^{n-1} in the current rotation
   if (c->mixed)
-    set_state_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L, in, tau, slot, c->q, c->qf, (float*)c->U[c->cur],
+    set_state_kernel<float><<<nb, kSetThreads, 0, c->stream>>>(c->P, L, in, tau, g, gp, slot, c->q, c->qf, (float*)c->U[c->cur],
                                                        (float*)c->U[c->prev], (float*)c->E[0], (float*)c->Pb[0],
                                                        c->reg, c->d_stat);
   else
-    set_state_kernel<double><<<nb, 256, 0, c->stream>>>(c->P, L, in, tau, slot, c->q, nullptr, (double*)c->U[c->cur],
+    set_state_kernel<double><<<nb, kSetThreads, 0, c->stream>>>(c->P, L, in, tau, g, gp, slot, c->q, nullptr, (double*)c->U[c->cur],
                                                         (double*)c->U[c->prev], (double*)c->E[0], (double*)c->Pb[0],
                                                         c->reg, c->d_stat);
   CK(cudaGetLastError());
