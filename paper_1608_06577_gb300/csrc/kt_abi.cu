@@ -67,10 +67,10 @@ struct Ctx {
   void* Pb[2] = {};
   double* stage = nullptr;  // staging: 18 packed fields of the largest event
   EosSeg<double>* seg_d = nullptr;
-  EosSeg<float>* seg_f = nullptr;
   RootSeg* seg_r = nullptr;
   RootSegM* seg_m = nullptr;
   FaceSeg* seg_face = nullptr;
+  SourceSeg* seg_src = nullptr;
   TauSlot* d_tau = nullptr;  // three slots, used in rotation with the u buffers: tau^n is in slot cur
   unsigned* d_stat = nullptr;
   float* d_mlp = nullptr;
@@ -202,10 +202,10 @@ size_t state_bytes(const std::vector<Lattice>& lat, long long gs, size_t max_cel
   b += align_up(4 * fs * es, 256);             // E[2], P[2]
   b += align_up(18 * max_cells * 8, 256);      // staging
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(EosSeg<double>), 256);
-  b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(EosSeg<float>), 256);
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(RootSeg), 256);
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(RootSegM), 256);
   b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(FaceSeg), 256);
+  b += align_up((size_t)(eos_n > 0 ? eos_n : 1) * sizeof(SourceSeg), 256);
   b += 256;                                    // tau
   b += 256;                                    // stats
   b += align_up(KT_MLP_NPARAM * 4, 256);       // MLP weights
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kSetThreads, 4)
     for (int m = 0; m < 3; ++m) up4[m + 1] = in.u_prev[(size_t)m * ncp + o];
     up4[0] = sqrt(fma(gp * up4[3], up4[3], fma(up4[2], up4[2], fma(up4[1], up4[1], 1.0))));
   }
-  const double P0 = eos_P<double>(P, e), Pt = P0 + Pi, w = (e + Pt) * u4[0];
+  const double P0 = eos_P(P, e), Pt = P0 + Pi, w = (e + Pt) * u4[0];
   double qn[NQ];
   qn[0] = fma(w, u4[0], -Pt) + pi[0];
 #pragma unroll
@@ -1209,10 +1209,10 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->stage = (double*)carve(18 * c->max_cells * 8);
   int nseg = P.eos_n > 0 ? P.eos_n : 1;
   c->seg_d = (EosSeg<double>*)carve(nseg * sizeof(EosSeg<double>));
-  c->seg_f = (EosSeg<float>*)carve(nseg * sizeof(EosSeg<float>));
   c->seg_r = (RootSeg*)carve(nseg * sizeof(RootSeg));
   c->seg_m = (RootSegM*)carve(nseg * sizeof(RootSegM));
   c->seg_face = (FaceSeg*)carve(nseg * sizeof(FaceSeg));
+  c->seg_src = (SourceSeg*)carve(nseg * sizeof(SourceSeg));
   c->d_tau = (TauSlot*)carve(256);
   c->d_stat = (unsigned*)carve(256);
   c->d_mlp = (float*)carve(KT_MLP_NPARAM * 4);
@@ -1233,10 +1233,10 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
     c->grid_mlp = (int)std::max(1LL, std::min((long long)std::max(1, nb) * sms, (long long)((fs + 255) / 256)));
   }
   P.seg_d = c->seg_d;
-  P.seg_f = c->seg_f;
   P.seg_r = c->seg_r;
   P.seg_m = c->seg_m;
   P.seg_face = c->seg_face;
+  P.seg_src = c->seg_src;
 
   CK(cudaMemsetAsync(qq, 0, 30 * fs * 8, c->stream));
   CK(cudaMemsetAsync(ep, 0, 4 * fs * c->esz, c->stream));
@@ -1262,13 +1262,16 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
     std::vector<RootSegM> sm;
     build_mixed_root_segments(sr, sm);
     CK(cudaMemcpyAsync(c->seg_d, sd.data(), sd.size() * sizeof(sd[0]), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(c->seg_f, sf.data(), sf.size() * sizeof(sf[0]), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->seg_r, sr.data(), sr.size() * sizeof(sr[0]), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->seg_m, sm.data(), sm.size() * sizeof(sm[0]), cudaMemcpyHostToDevice, c->stream));
     std::vector<FaceSeg> sface(sr.size());
     for (size_t i = 0; i < sr.size(); ++i)
       sface[i] = FaceSeg{(float)sr[i].e0, (float)sr[i].e1, (float)sr[i].P0, (float)sr[i].a1,
                          (float)sr[i].a2, (float)sr[i].a3, 0.f,             0.f};
+    std::vector<SourceSeg> ssrc(sf.size());
+    for (size_t i = 0; i < sf.size(); ++i)
+      ssrc[i] = SourceSeg{sf[i].e0, sf[i].inv_de, sf[i].l0, sf[i].dl, sf[i].T0, sf[i].mT, sf[i].cT2, sf[i].cT3};
+    CK(cudaMemcpyAsync(c->seg_src, ssrc.data(), ssrc.size() * sizeof(SourceSeg), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->seg_face, sface.data(), sface.size() * sizeof(FaceSeg), cudaMemcpyHostToDevice, c->stream));
   }
   if (o.mlp_weights) {

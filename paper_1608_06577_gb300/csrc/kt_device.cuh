@@ -106,6 +106,12 @@ struct alignas(32) FaceSeg {
   float e0, e1, P0, a1, a2, a3, unused0, unused1;
 };
 
+// The single-precision record of the same interval for the sources' T and ln(1/3 - c_s^2), one sector
+// (eight loads from EosSeg before)
+struct alignas(32) SourceSeg {
+  float e0, inv_de, l0, dl, T0, mT, cT2, cT3;
+};
+
 struct Coef {
   int kind;       // 0 const, 1 gauss
   double c0, c1, c2;
@@ -138,9 +144,9 @@ struct Params {
   int eos_n;
   float lne0, inv_h;  // index guess: (ln e - ln e_0) * inv_h
   const EosSeg<double>* seg_d;
-  const EosSeg<float>* seg_f;
   const RootSeg* seg_r;
   const FaceSeg* seg_face;  // the same intervals for the face root-finds (KT_IFACE_INVERT, FP32)
+  const SourceSeg* seg_src;  // the same intervals for the FP32 sources
   const RootSegM* seg_m;  // the same intervals for the mixed-precision root-find
   Coef eta, zeta;
   int shear_on, bulk_on;
@@ -161,55 +167,27 @@ template <typename R> __device__ __forceinline__ const PR<R>& pr(const Params& P
 template <> __device__ __forceinline__ const PR<double>& pr<double>(const Params& P) { return P.pd; }
 template <> __device__ __forceinline__ const PR<float>& pr<float>(const Params& P) { return P.pf; }
 
-template <typename R> __device__ __forceinline__ const EosSeg<R>* eos_table(const Params& P);
-template <> __device__ __forceinline__ const EosSeg<double>* eos_table<double>(const Params& P) { return P.seg_d; }
-template <> __device__ __forceinline__ const EosSeg<float>* eos_table<float>(const Params& P) { return P.seg_f; }
-
 // Interval search: a single-precision log guess, corrected so that e_i <= e < e_{i+1} exactly
 // (clamped to the first / last interval outside the table).
-template <typename R>
-__device__ __forceinline__ int eos_interval(const Params& P, const EosSeg<R>* seg, R e) {
-  int n1 = P.eos_n - 2;
-  float ef;
-  if constexpr (sizeof(R) == 8) ef = d2f_trunc(e); else ef = e;
-  float g = (__logf(ef) - P.lne0) * P.inv_h;
+__device__ __forceinline__ int eos_interval(const Params& P, const EosSeg<double>* seg, double e) {
+  const int n1 = P.eos_n - 2;
+  const float g = (__logf(d2f_trunc(e)) - P.lne0) * P.inv_h;
   int i = (g > 0.f) ? (int)g : 0;  // NaN compares false -> 0
   i = min(i, n1);
-  if constexpr (sizeof(R) == 8) {  // nodes are positive: compare bit patterns (e <= 0 orders below all)
-    const long long b = __double_as_longlong(e);
+  const long long b = __double_as_longlong(e);  // nodes are positive: compare bit patterns (e <= 0 orders below all)
 #pragma unroll 1
-    for (int it = 0; it < 64 && i > 0 && b < __double_as_longlong(seg[i].e0); ++it) --i;
+  for (int it = 0; it < 64 && i > 0 && b < __double_as_longlong(seg[i].e0); ++it) --i;
 #pragma unroll 1
-    for (int it = 0; it < 64 && i < n1 && b >= __double_as_longlong(seg[i + 1].e0); ++it) ++i;
-  } else {
-#pragma unroll 1
-    for (int it = 0; it < 64 && i > 0 && e < seg[i].e0; ++it) --i;
-#pragma unroll 1
-    for (int it = 0; it < 64 && i < n1 && e >= seg[i + 1].e0; ++it) ++i;
-  }
+  for (int it = 0; it < 64 && i < n1 && b >= __double_as_longlong(seg[i + 1].e0); ++it) ++i;
   return i;
 }
 
-// P0(e), c_s^2(e) (for the root-find)
-template <typename R>
-__device__ __forceinline__ void eos_P_cs2(const Params& P, R e, R& P0, R& cs2) {
-  if (!P.eos_table) {
-    P0 = e * R(1.0 / 3.0);
-    cs2 = R(1.0 / 3.0);
-    return;
-  }
-  const EosSeg<R>* seg = eos_table<R>(P);
-  const EosSeg<R>& s = seg[eos_interval<R>(P, seg, e)];
-  R t = (e - s.e0) * s.inv_de;
-  P0 = fma(t, fma(t, fma(t, s.cP3, s.cP2), s.mP), s.P0);
-  cs2 = fma(t, fma(t, R(3) * s.cP3, R(2) * s.cP2), s.mP) * s.inv_de;
-}
-
-template <typename R>
-__device__ __forceinline__ R eos_P(const Params& P, R e) {
-  R p, c;
-  eos_P_cs2<R>(P, e, p, c);
-  return p;
+// P0(e)
+__device__ __forceinline__ double eos_P(const Params& P, double e) {
+  if (!P.eos_table) return e * (1.0 / 3.0);
+  const EosSeg<double>& s = P.seg_d[eos_interval(P, P.seg_d, e)];
+  const double t = (e - s.e0) * s.inv_de;
+  return fma(t, fma(t, fma(t, s.cP3, s.cP2), s.mP), s.P0);
 }
 
 // T(e) and ln(1/3 - c_s^2)(e) (for the transport coefficients)
@@ -220,22 +198,23 @@ __device__ __forceinline__ void eos_T_lnd(const Params& P, R e, R& T, R& lnd) {
     lnd = -R(INFINITY);
     return;
   }
-  const EosSeg<R>* seg = eos_table<R>(P);
   // FP64: the exact interval.  FP32 (the mixed-precision sources): the interval of the
   // single-precision log guess alone; next to a node that may be the neighbouring interval,
   // whose cubic matches value and slope at the node, so the difference stays far below FP32
   // rounding, and the dependent table loads of the correction are saved.
-  int i;
   if constexpr (sizeof(R) == 8) {
-    i = eos_interval<R>(P, seg, e);
+    const EosSeg<double>& s = P.seg_d[eos_interval(P, P.seg_d, e)];
+    R t = (e - s.e0) * s.inv_de;
+    T = fma(t, fma(t, fma(t, s.cT3, s.cT2), s.mT), s.T0);
+    lnd = fma(t, s.dl, s.l0);
   } else {
     const float g = (__logf(e) - P.lne0) * P.inv_h;
-    i = min((g > 0.f) ? (int)g : 0, P.eos_n - 2);
+    const float4* p = reinterpret_cast<const float4*>(P.seg_src + min((g > 0.f) ? (int)g : 0, P.eos_n - 2));
+    const float4 a = __ldg(p), b = __ldg(p + 1);
+    const float t = (e - a.x) * a.y;
+    T = fmaf(t, fmaf(t, fmaf(t, b.w, b.z), b.y), b.x);
+    lnd = fmaf(t, a.w, a.z);
   }
-  const EosSeg<R>& s = seg[i];
-  R t = (e - s.e0) * s.inv_de;
-  T = fma(t, fma(t, fma(t, s.cT3, s.cT2), s.mT), s.T0);
-  lnd = fma(t, s.dl, s.l0);
 }
 
 // x / 2 by its exponent; |x| < 2^-1021 gives 0

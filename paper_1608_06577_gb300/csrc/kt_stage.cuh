@@ -652,7 +652,7 @@ __device__ __forceinline__ unsigned invert_fp64(const Params& P, double tau, con
   if (!(obits(E) > 0) || !finite(E) || !finite(M2) || !(obits(M2) < obits(E * E))) {
     st = ST_INVERSION;
     e = (P.e_min > 0.0) ? P.e_min : 1e-30;
-    P0 = eos_P<double>(P, e);
+    P0 = eos_P(P, e);
   } else if (!P.eos_table) {  // (bulk pressure is evolved with a table EOS only)
     const double M = sqrt(M2);  // conformal closed form e = sqrt(4E^2 - 3M^2) - E, cancellation-free
     e = vdiv(3.0 * (E - M) * (E + M), sqrt(fma(4.0 * E, E, -3.0 * M2)) + E);
