@@ -189,7 +189,7 @@ __global__ void __maxnreg__(96)
   if (bad) {  // a copy did not complete in time: let the ones in flight land before the block exits
     for (; done < issued; ++done) mbar_wait(&s_bar[done & 1u], (done >> 1) & 1u, kWaitPolls);
   }
-  block_stats(io.status, io.max_speed_bits, io.counters, bad ? ST_TIMEOUT : 0u, amax, 0u, 0u, 0u);
+  block_stats<true, false>(io.status, io.max_speed_bits, io.counters, bad ? ST_TIMEOUT : 0u, amax, 0u, 0u, 0u);
 }
 
 // ------------------------------------------------------------- d) the root-find (Sec. 2.4)
@@ -509,7 +509,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 64 : 80) update_kernel(const Params P, 
     update_cell<STAGE, LEARNED, PI32>(P, L, io, in, i, j, k, tau, st, nit, nreg, nfb);
   }
   if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && (threadIdx.x | threadIdx.y | threadIdx.z) == 0);
-  block_stats(io.status, nullptr, io.counters, st, 0.f, nit, nreg, nfb);
+  block_stats<false, true>(io.status, nullptr, io.counters, st, 0.f, nit, nreg, nfb);
 }
 
 // ---------------------------------------------------------------- the network, once per step
@@ -656,7 +656,7 @@ __global__ void __maxnreg__(STAGE == 1 ? 72 : 96)
       mbar_wait(&s_bar[(nbuf == 2) ? (done & 1u) : 0u], (nbuf == 2) ? ((done >> 1) & 1u) : (done & 1u), kWaitPolls);
   }
   if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && tid == 0);
-  block_stats(io.status, nullptr, io.counters, st | (bad ? ST_TIMEOUT : 0u), 0.f, nit, nreg, nfb);
+  block_stats<false, true>(io.status, nullptr, io.counters, st | (bad ? ST_TIMEOUT : 0u), 0.f, nit, nreg, nfb);
 }
 
 // ---------------------------------------------------------------- fused stage (one launch per stage)
@@ -789,7 +789,7 @@ __global__ void __maxnreg__(128)
     for (; done < issued; ++done) mbar_wait(&s_bar[done & 1u], (done >> 1) & 1u, kWaitPolls);
   }
   if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && tid == 0);
-  block_stats(io.status, io.max_speed_bits, io.counters, st | (bad ? ST_TIMEOUT : 0u), amax, nit, nreg, nfb);
+  block_stats<true, true>(io.status, io.max_speed_bits, io.counters, st | (bad ? ST_TIMEOUT : 0u), amax, nit, nreg, nfb);
 }
 
 }  // namespace kt

@@ -389,8 +389,17 @@ __device__ __forceinline__ void component_rhs_xy(const Params& P, int n, const f
   up2(D1, d1x, d1y);
   up2(D2, d2x, d2y);
   up2(D3, d3x, d3y);
-  three_slopes<float, true>(d0x, d1x, d2x, d3x, 1.f, smx, s0x, spx);
-  three_slopes<float, true>(d0y, d1y, d2y, d3y, 1.f, smy, s0y, spy);
+  // three_slopes for both directions, the lower bounds as pairs
+  const float h1x = fmaxf(d1x, 0.f), h1y = fmaxf(d1y, 0.f), h2x = fmaxf(d2x, 0.f), h2y = fmaxf(d2y, 0.f);
+  float l1x, l1y, l2x, l2y;
+  up2(sub2(D1, pk2(h1x, h1y)), l1x, l1y);
+  up2(sub2(D2, pk2(h2x, h2y)), l2x, l2y);
+  smx = fminf(fmaxf(d0x, l1x), h1x);
+  smy = fminf(fmaxf(d0y, l1y), h1y);
+  s0x = fminf(fmaxf(d1x, l2x), h2x);
+  s0y = fminf(fmaxf(d1y, l2y), h2y);
+  spx = fminf(fmaxf(d3x, l2x), h2x);
+  spy = fminf(fmaxf(d3y, l2y), h2y);
   unsigned long long acc = mul2(W.wLm, fma2(pk2(0.5f, 0.5f), pk2(smx, smy), A1));
   acc = fma2(W.wRp, fma2(pk2(-0.5f, -0.5f), pk2(spx, spy), B1), acc);
   acc = fma2(W.hdW, pk2(s0x, s0y), acc);
@@ -1165,33 +1174,39 @@ __device__ __forceinline__ void tile_range(int ntiles, int& t0, int& t1) {
 // ---------------------------------------------------------------- per-launch statistics
 // status bits OR-ed, the largest local speed (float bits, all non-negative), and the Newton /
 // regulated / fallback counters: warp reductions, then one set of atomics per block.  Every
-// thread of the block calls this once, after its last cell.
+// thread of the block calls this once, after its last cell.  SPEED, COUNTS: which of them the kernel has.
+template <bool SPEED, bool COUNTS>
 __device__ __forceinline__ void block_stats(unsigned* status, unsigned* max_speed_bits,
                                             unsigned long long* counters, unsigned st, float amax, unsigned nit,
                                             unsigned nreg, unsigned nfb) {
-  __shared__ unsigned s_st[32], s_max[32], s_it[32], s_reg[32], s_fb[32];
+  __shared__ unsigned s_stat[5];
   const unsigned full = 0xffffffffu;
-  unsigned w_st = __reduce_or_sync(full, st);
-  unsigned w_max = __reduce_max_sync(full, __float_as_uint(amax));
-  unsigned w_it = __reduce_add_sync(full, nit);
-  unsigned w_reg = __reduce_add_sync(full, nreg);
-  unsigned w_fb = __reduce_add_sync(full, nfb);
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int warp = tid >> 5, nwarps = (blockDim.x * blockDim.y * blockDim.z + 31) >> 5;
+  if (tid < 5) s_stat[tid] = 0u;
+  __syncthreads();
+  const unsigned w_st = __reduce_or_sync(full, st);
+  unsigned w_max = 0, w_it = 0, w_reg = 0, w_fb = 0;
+  if (SPEED) w_max = __reduce_max_sync(full, __float_as_uint(amax));
+  if (COUNTS) {
+    w_it = __reduce_add_sync(full, nit);
+    w_reg = __reduce_add_sync(full, nreg);
+    w_fb = __reduce_add_sync(full, nfb);
+  }
   if ((tid & 31) == 0) {
-    s_st[warp] = w_st; s_max[warp] = w_max; s_it[warp] = w_it; s_reg[warp] = w_reg; s_fb[warp] = w_fb;
+    if (w_st) atomicOr(&s_stat[0], w_st);
+    if (SPEED) atomicMax(&s_stat[1], w_max);
+    if (COUNTS) {
+      atomicAdd(&s_stat[2], w_it);
+      if (w_reg) atomicAdd(&s_stat[3], w_reg);
+      if (w_fb) atomicAdd(&s_stat[4], w_fb);
+    }
   }
   __syncthreads();
-  if (tid == 0) {
-    unsigned a = 0, b = 0, cI = 0, d = 0, fb = 0;
-    for (int w = 0; w < nwarps; ++w) {
-      a |= s_st[w]; b = max(b, s_max[w]); cI += s_it[w]; d += s_reg[w]; fb += s_fb[w];
-    }
-    if (a) atomicOr(status, a);
-    if (max_speed_bits) atomicMax(max_speed_bits, b);
-    if (cI) atomicAdd(counters + 0, (unsigned long long)cI);
-    if (d) atomicAdd(counters + 1, (unsigned long long)d);
-    if (fb) atomicAdd(counters + 2, (unsigned long long)fb);
+  if (tid < 5) {
+    const unsigned v = s_stat[tid];
+    if (tid == 0 && v) atomicOr(status, v);
+    if (SPEED && tid == 1) atomicMax(max_speed_bits, v);
+    if (COUNTS && tid >= 2 && v) atomicAdd(counters + tid - 2, (unsigned long long)v);
   }
 }
 
