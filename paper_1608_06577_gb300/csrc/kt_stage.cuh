@@ -843,10 +843,50 @@ __device__ __forceinline__ void cell_rhs(const Params& P, const Lattice& L, cons
 // sqrt(pi.pi)/P0, |Pi|/P0, sqrt(J^{mu nu} J_{mu nu})/(2 eta sqrt(sigma.sigma)) and |J|/(zeta
 // |theta|) with J^{mu nu}, J the second-order terms of Eq. (14_moment_terms) (no diffusion); a
 // quantity whose channel is off, or whose denominator vanishes, is 0.
-template <typename R, bool DIAG>
-__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
-                                             const CellGeom<R>& G, const R (&uc)[4], R (&du)[4][4], R dv,
-                                             R (&dq)[NQ], R* dg) {
+//
+// The transport coefficients depend on e alone and nothing here reads the fluxes, so a kernel with warps
+// to spare computes both beside them: `out` says where the terms go and may bring the coefficients.
+template <typename R>
+struct Transport {
+  R T, lnd, es, rate_pi, rate_Pi, d;  // d = 1/3 - c_s^2
+};
+// T(e) and ln(1/3 - c_s^2)(e) are given; the rates are bounded by the step
+template <typename R>
+__device__ __forceinline__ void shear_transport(const Params& P, Transport<R>& tr) {
+  tr.es = eta_over_s<R>(P, tr.T);
+  const R rate = (tr.es > R(0)) ? ((P.eta.kind == 0) ? tr.T * pr<R>(P).eta_inv_5c0 : sdiv(tr.T, R(5) * tr.es)) : R(INFINITY);
+  tr.rate_pi = nmin(rate, pr<R>(P).rate_max);
+}
+template <typename R>
+__device__ __forceinline__ void bulk_transport(const Params& P, Transport<R>& tr) {
+  tr.d = sexp(tr.lnd);
+  // 1/tau_Pi = 15 (1/3 - c_s^2)^2 T / (zeta/s): both factors span hundreds of e-folds away from the
+  // transition, so their quotient is formed in the exponent (Eq. (zetas), bounded below, divides)
+  R rate;
+  if (P.zeta.kind == 2) {
+    const R z = pr<R>(P).zeta_c0 * zeta_over_s_paper<R>(tr.T * pr<R>(P).zeta_inv_c1);
+    rate = (z > R(0)) ? sdiv(R(15) * tr.d * tr.d * tr.T, z) : R(INFINITY);
+  } else {
+    rate = R(15) * tr.T * sexp(fma(R(2), tr.lnd, -ln_zeta_over_s<R>(P, tr.T)));
+  }
+  tr.rate_Pi = nmin(rate, pr<R>(P).rate_max);
+}
+// the terms added to dq at once, the coefficients formed where they are used
+template <typename R>
+struct SourceDirect {
+  static constexpr bool kHasTransport = false;
+  Transport<R> tr;
+  R (&dq)[NQ];
+  __device__ __forceinline__ void conserved(int n, R it, R qn) { dq[n] = fma(-it, qn, dq[n]); }
+  __device__ __forceinline__ void energy(R x) { dq[0] -= x; }
+  __device__ __forceinline__ void shear(int n, R iu0, R s) { dq[n] = fma(iu0, s, dq[n]); }
+  __device__ __forceinline__ void bulk(R x) { dq[14] += x; }
+};
+
+template <typename R, bool DIAG, typename Out>
+__device__ __forceinline__ void cell_sources_to(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
+                                                const CellGeom<R>& G, const R (&uc)[4], R (&du)[4][4], R dv,
+                                                Out& out, R* dg) {
   if constexpr (DIAG) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) dg[k] = R(0);
@@ -876,10 +916,10 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
   // geometric sources of the conservation laws, Eqs. (dT001)-(dT0i1)
   {
     R Tnn = (ec + Pt) * uc[3] * uc[3] + Pt * inv_gnn + pi[3][3];
-    dq[0] -= ld<R>(q, c) * it + tg * Tnn;
-    dq[1] -= ld<R>(q + fs, c) * it;
-    dq[2] -= ld<R>(q + 2 * fs, c) * it;
-    dq[3] -= R(3) * ld<R>(q + 3 * fs, c) * it;
+    out.energy(fma(tg, Tnn, rmul(ld<R>(q, c), it)));
+    out.conserved(1, it, ld<R>(q + fs, c));
+    out.conserved(2, it, ld<R>(q + 2 * fs, c));
+    out.conserved(3, it, rmul(R(3), ld<R>(q + 3 * fs, c)));
   }
 
   if (P.shear_on || P.bulk_on) {
@@ -944,15 +984,13 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
     const R ps = fma(gnn, fma(gnn, pi[3][3] * sig[3][3], R(2) * psn), fma(R(2), pso, psd));
 
     // transport coefficients (Sec. 2.2) from T(e), ln(1/3 - c_s^2)(e)
-    R T, lnd;
-    eos_T_lnd<R>(P, ec, T, lnd);
+    Transport<R>& tr = out.tr;
+    if constexpr (!Out::kHasTransport) eos_T_lnd<R>(P, ec, tr.T, tr.lnd);
     const R iu0 = sdiv(R(1), uc[0]);
 
     if (P.shear_on) {
       const R eta_tp = (ec + P0c) * R(0.2);
-      const R es = eta_over_s<R>(P, T);
-      R rate_pi = (es > R(0)) ? ((P.eta.kind == 0) ? T * pr<R>(P).eta_inv_5c0 : sdiv(T, R(5) * es)) : R(INFINITY);
-      rate_pi = nmin(rate_pi, pr<R>(P).rate_max);
+      if constexpr (!Out::kHasTransport) shear_transport<R>(P, tr);
       const R tp3 = pr<R>(P).tpp * ps * R(1.0 / 3.0);
       const R csig = fma(R(1.2), Pic, R(2) * eta_tp);
       if constexpr (DIAG) {  // sums over the full tensor: off-diagonal pairs count twice
@@ -973,12 +1011,12 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
             dg[4] += X * X * w;
             xs += sig[a][b] * sig[a][b] * w;
           }
-        dg[0] = sdiv(R(5) * es, T) * theta;
+        dg[0] = sdiv(R(5) * tr.es, tr.T) * theta;
         dg[4] = (xs > R(0)) ? sdiv(sqrt(dg[4]), R(2) * eta_tp * sqrt(xs)) : R(0);
       }
       // M^b_l = g_{ll} Y^{bl} - K^b_l, and on its diagonal half of the coefficient of pi^{ab}:
       // -1/tau_pi - 4 theta/3 (delta_pipi) + u^tau d_i v^i (S_pi's pi d_i v^i, taken inside the 1/u^tau)
-      const R hc = rmul(R(0.5), fma(uc[0], dv, fma(R(-4.0 / 3.0), theta, -rate_pi)));
+      const R hc = rmul(R(0.5), fma(uc[0], dv, fma(R(-4.0 / 3.0), theta, -tr.rate_pi)));
       R M[4][4];
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
@@ -1000,34 +1038,24 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
         R h = fma(pi[a][0], M[a][0], fma(pi[a][1], M[a][1], fma(pi[a][2], M[a][2], pi[a][3] * M[a][3])));
         const R dg0 = (a == 0) ? tp3 : ((a == 3) ? gup[3] * tp3 : -tp3);
         h = fma(R(2), h, fma(csig, sig[a][a], fma(-tpu, uc[a], dg0)));
-        dq[pix(a, a)] = fma(iu0, h, dq[pix(a, a)]);
+        out.shear(pix(a, a), iu0, h);
 #pragma unroll
         for (int b = a + 1; b < 4; ++b) {
           R s = fma(csig, sig[a][b], -(tpu * uc[b]));
 #pragma unroll
           for (int l = 0; l < 4; ++l) s = fma(pi[a][l], M[b][l], fma(pi[b][l], M[a][l], s));
-          dq[pix(a, b)] = fma(iu0, s, dq[pix(a, b)]);
+          out.shear(pix(a, b), iu0, s);
         }
       }
     }
     if (P.bulk_on) {
-      const R d = sexp(lnd);
-      const R d15 = R(15) * d * d;
-      // 1/tau_Pi = 15 (1/3 - c_s^2)^2 T / (zeta/s): both factors span hundreds of e-folds away from the
-      // transition, so their quotient is formed in the exponent (Eq. (zetas), bounded below, divides)
-      R rate_Pi;
-      if (P.zeta.kind == 2) {
-        const R z = pr<R>(P).zeta_c0 * zeta_over_s_paper<R>(T * pr<R>(P).zeta_inv_c1);
-        rate_Pi = (z > R(0)) ? sdiv(d15 * T, z) : R(INFINITY);
-      } else {
-        rate_Pi = R(15) * T * sexp(fma(R(2), lnd, -ln_zeta_over_s<R>(P, T)));
-      }
-      rate_Pi = nmin(rate_Pi, pr<R>(P).rate_max);
-      const R zt = d15 * (ec + P0c);
-      const R IPi = R(2.0 / 3.0) * Pic * theta - R(1.6) * d * ps;
-      dq[14] += (-zt * theta - rate_Pi * Pic - IPi) * iu0 + Pic * dv;
+      if constexpr (!Out::kHasTransport) bulk_transport<R>(P, tr);
+      const R d = tr.d;
+      const R zt = R(15) * d * d * (ec + P0c);
+      const R IPi = fma(R(2.0 / 3.0) * Pic, theta, -(R(1.6) * d * ps));
+      out.bulk(fma(fma(-tr.rate_Pi, Pic, fma(-zt, theta, -IPi)), iu0, rmul(Pic, dv)));
       if constexpr (DIAG) {
-        const R lrate = R(2.70805020110221) + R(2) * lnd + slog(T) - ln_zeta_over_s<R>(P, T);  // ln 15 + ...
+        const R lrate = R(2.70805020110221) + R(2) * tr.lnd + slog(tr.T) - ln_zeta_over_s<R>(P, tr.T);  // ln 15 + ...
         dg[1] = sexp(-lrate) * theta;
         dg[5] = (theta != R(0)) ? sdiv(fabs(IPi), zt * fabs(theta)) : R(0);
       }
@@ -1037,6 +1065,14 @@ __device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, 
       dg[3] = sdiv(fabs(Pic), P0c);
     }
   }
+}
+
+template <typename R, bool DIAG>
+__device__ __forceinline__ void cell_sources(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
+                                             const CellGeom<R>& G, const R (&uc)[4], R (&du)[4][4], R dv,
+                                             R (&dq)[NQ], R* dg) {
+  SourceDirect<R> out{Transport<R>{}, dq};
+  cell_sources_to<R, DIAG>(P, L, io, c, G, uc, du, dv, out, dg);
 }
 
 // The inversion's inputs at one cell (Eqs. eInferred-uiInferred): E = T^tt - pi^tt,
@@ -1259,10 +1295,30 @@ __global__ void __launch_bounds__(32, 8)
 // ---------------------------------------------------------------- the same for grids with few cells (FP64)
 // With fewer strips than the chip has FP64 issue slots (four warps per SM) the kernel above is a serial
 // chain of ~1,500 FP64 instructions at 64 cycles each while most units idle.  Here four warps share a
-// strip: one axis each for the face setup (warps 0-2), every fourth component each for the fluxes, then
-// warp 0 adds up and runs the sources and the update.  Values pass through shared memory and are added in
-// the order of the one-warp kernel, so both give the same bits.
-enum : int { TM_FACE = 0, TM_DU = 18, TM_DV = 30, TM_PR = 33, TM_ACC = 39, TM_MIX = 54, TM_DIFF = 58, TM_VALUES = 70 };
+// strip.  Warps 0-2 take one axis each for the face setup and then every third component of the fluxes;
+// warp 3 meanwhile computes the transport coefficients and then the sources (as long a chain as five
+// components); warp 0 adds up and runs the update.  Values pass through shared memory and are added in
+// the order of the one-warp kernel, so both give the same bits.  Gubser grid 32 x 32 x 8 (256 strips), 20
+// steps: 2.24 ms with the sources in warp 0 after the fluxes, 2.05 ms beside them (start of both: 3.39
+// ms with one warp per strip); shock tube of 7 strips, 80 steps, 3.50 ms with one warp, 2.94 ms here.
+enum : int { TM_FACE = 0, TM_DU = 18, TM_DV = 30, TM_PR = 33, TM_ACC = 39, TM_MIX = 54, TM_DIFF = 58, TM_SRC = 70,
+             TM_IU0 = 85, TM_VALUES = 86 };
+
+// the source terms left in shared memory for warp 0 (rows 1-3: the components they multiply)
+template <typename R>
+struct SourceShared {
+  static constexpr bool kHasTransport = true;
+  Transport<R> tr;
+  R (*sm)[32];
+  int lane;
+  __device__ __forceinline__ void conserved(int n, R, R qn) { sm[TM_SRC + n][lane] = qn; }
+  __device__ __forceinline__ void energy(R x) { sm[TM_SRC][lane] = x; }
+  __device__ __forceinline__ void shear(int n, R iu0, R s) {
+    sm[TM_SRC + n][lane] = s;
+    sm[TM_IU0][lane] = iu0;
+  }
+  __device__ __forceinline__ void bulk(R x) { sm[TM_SRC + 14][lane] = x; }
+};
 
 template <typename R, int D, bool TH1>
 __device__ __forceinline__ void team_faces(const Params& P, const Lattice& L, const StageIO<R>& io, Idx<R> c,
@@ -1310,12 +1366,29 @@ __global__ void __launch_bounds__(128, 2)
   const bool on[3] = {L.nx > 1, L.ny > 1, L.nz > 1};
   const int s[3] = {1, L.pitch, (int)L.plane};
   const R* p = io.qr_in + c;
-  Stencil13<R> q = load_stencil<R>(p + warp * fs, on, s);  // in flight during the face setup
+  Stencil13<R> q;
+  SourceShared<R> src{Transport<R>{}, sm, lane};
+  if (warp < 3) q = load_stencil<R>(p + warp * fs, on, s);  // in flight during the face setup
   if (warp == 0) team_faces<R, 0, TH1>(P, L, io, c, G, sm, amax);
   else if (warp == 1) team_faces<R, 1, TH1>(P, L, io, c, G, sm, amax);
   else if (warp == 2) team_faces<R, 2, TH1>(P, L, io, c, G, sm, amax);
+  else if (P.shear_on || P.bulk_on) {
+    eos_T_lnd<R>(P, ld<R>(io.e_in, c), src.tr.T, src.tr.lnd);
+    if (P.shear_on) shear_transport<R>(P, src.tr);
+    if (P.bulk_on) bulk_transport<R>(P, src.tr);
+  }
   __syncthreads();
-  {
+  if (warp == 3) {
+    const R d[3] = {sm[TM_DV][lane], sm[TM_DV + 1][lane], sm[TM_DV + 2][lane]};
+    R uc[4], du[4][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      uc[m] = ld<R>(io.u_in + m * fs, c);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) du[a + 1][m] = sm[TM_DU + 4 * a + m][lane];
+    }
+    cell_sources_to<R, false>(P, L, io, c, G, uc, du, divergence<R>(P, d), src, nullptr);
+  } else {
     Faces<R> F[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d)
@@ -1323,8 +1396,8 @@ __global__ void __launch_bounds__(128, 2)
                       sm[TM_FACE + 6 * d + 3][lane], sm[TM_FACE + 6 * d + 4][lane], sm[TM_FACE + 6 * d + 5][lane], s[d]};
     const R c0 = sum_c0<R>(F, on), th = pr<R>(P).theta;
 #pragma unroll 1
-    for (int n = warp; n < NQ; n += 4) {
-      const Stencil13<R> next = load_stencil<R>(p + min(n + 4, NQ - 1) * fs, on, s);
+    for (int n = warp; n < NQ; n += 3) {
+      const Stencil13<R> next = load_stencil<R>(p + min(n + 3, NQ - 1) * fs, on, s);
       R acc = R(-0.0), mix = R(-0.0);  // (adding -0 changes nothing)
       const bool any = stencil_nonzero<R>(q);
       if (any) stencil_flux<R, TH1>(q, c0, on, F, th, n >= 4 && n <= 7, acc, mix);
@@ -1344,7 +1417,7 @@ __global__ void __launch_bounds__(128, 2)
     warp_stats(io, 0u, amax, 0u, 0u);
     return;
   }
-  R dq[NQ], uc[4], du[4][4];
+  R dq[NQ];
 #pragma unroll
   for (int n = 0; n < NQ; ++n) dq[n] = R(-0.0);
 #pragma unroll
@@ -1362,14 +1435,16 @@ __global__ void __launch_bounds__(128, 2)
     dq[n] += sm[TM_ACC + n][lane];
     if (n >= 4 && n <= 7) dq[n - 4] += sm[TM_MIX + n - 4][lane];
   }
-  const R d[3] = {sm[TM_DV][lane], sm[TM_DV + 1][lane], sm[TM_DV + 2][lane]};
+  SourceDirect<R> out{Transport<R>{}, dq};
+  const R it = P.milne ? G.tau * G.inv_gnn : R(0);
+  out.energy(sm[TM_SRC][lane]);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    uc[m] = ld<R>(io.u_in + m * fs, c);
+  for (int n = 1; n < 4; ++n) out.conserved(n, it, sm[TM_SRC + n][lane]);
+  if (P.shear_on) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) du[a + 1][m] = sm[TM_DU + 4 * a + m][lane];
+    for (int n = 4; n < 14; ++n) out.shear(n, sm[TM_IU0][lane], sm[TM_SRC + n][lane]);
   }
-  cell_sources<R>(P, L, io, c, G, uc, du, divergence<R>(P, d), dq);
+  if (P.bulk_on) out.bulk(sm[TM_SRC + 14][lane]);
   stage_finish<R, STAGE>(P, L, io, at, tau_out, dq, st, nit, nreg);
   __syncwarp();
   if (STAGE == 2) advance_tau(P, io.tau, io.tau_next, blockIdx.x == 0 && threadIdx.x == 0);
