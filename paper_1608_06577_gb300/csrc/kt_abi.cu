@@ -1352,14 +1352,17 @@ int kt_set_state(kt_ctx* c, double tau, const double* e, const double* u, const 
 
 namespace {
 
-// One packed row of an event going out: the field component, whether it is float, the destination.
+// One packed row of an event going out: the field component, whether it is float, the destination, and
+// which of the caller's arrays that is in.
 struct Row {
   const void* f;
   int f32;
   double* dst;
+  int array;
 };
 // Rows to the caller's arrays: on the device in one launch per kRows rows, to the host through the staging
-// area with one copy per run of adjoining destinations.
+// area with one copy per caller's array (its rows adjoin).  Two arrays that happen to adjoin are copied
+// apart all the same: each may be a pinned allocation of its own, and a copy across both is refused.
 int gather_rows(Ctx* c, const Lattice& L, const std::vector<Row>& rows, int on_device) {
   const size_t ncp = (size_t)L.nx * L.ny * L.nz;
   for (size_t b = 0; b < rows.size(); b += kRows) {
@@ -1376,7 +1379,7 @@ int gather_rows(Ctx* c, const Lattice& L, const std::vector<Row>& rows, int on_d
     if (on_device) continue;
     for (int r = 0; r < g.n;) {
       int m = 1;
-      while (r + m < g.n && rows[b + r + m].dst == rows[b + r].dst + m * ncp) ++m;
+      while (r + m < g.n && rows[b + r + m].array == rows[b + r].array) ++m;
       CK(cudaMemcpyAsync(rows[b + r].dst, c->stage + r * ncp, m * ncp * 8, cudaMemcpyDeviceToHost, c->stream));
       r += m;
     }
@@ -1481,16 +1484,16 @@ int kt_get_state_event(kt_ctx* c, int event, double* tau, double* e, double* u, 
   const long long fs = c->gs;
   std::vector<Row> rows;
   const char* Ucur = (const char*)c->U[c->cur];
-  if (e) rows.push_back({c->E[0], c->mixed, e});
-  if (u) for (int m = 0; m < 4; ++m) rows.push_back({Ucur + (size_t)m * fs * c->esz, c->mixed, u + m * ncp});
+  if (e) rows.push_back({c->E[0], c->mixed, e, 0});
+  if (u) for (int m = 0; m < 4; ++m) rows.push_back({Ucur + (size_t)m * fs * c->esz, c->mixed, u + m * ncp, 1});
   // component n of q: FP64, or (KT_STORE_PI_FP32, n >= 4) the FP32 state
-  auto qrow = [&](int n, double* dst) {
-    if (c->pi32 && n >= 4) rows.push_back({c->qf + (size_t)n * fs, 1, dst});
-    else rows.push_back({c->q + (size_t)n * fs, 0, dst});
+  auto qrow = [&](int n, double* dst, int array) {
+    if (c->pi32 && n >= 4) rows.push_back({c->qf + (size_t)n * fs, 1, dst, array});
+    else rows.push_back({c->q + (size_t)n * fs, 0, dst, array});
   };
-  if (pi) for (int m = 0; m < 10; ++m) qrow(4 + m, pi + m * ncp);
-  if (Pi) qrow(14, Pi);
-  if (q) for (int n = 0; n < NQ; ++n) qrow(n, q + n * ncp);
+  if (pi) for (int m = 0; m < 10; ++m) qrow(4 + m, pi + m * ncp, 2);
+  if (Pi) qrow(14, Pi, 3);
+  if (q) for (int n = 0; n < NQ; ++n) qrow(n, q + n * ncp, 4);
   const int rc = gather_rows(c, L, rows, on_device);
   if (rc != KT_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));
@@ -1540,7 +1543,7 @@ int kt_get_checkpoint(kt_ctx* c, int event, double* tau, double* buf, int on_dev
   const size_t ncp = (size_t)L.nx * L.ny * L.nz;
   static_assert(KT_CHECKPOINT_ROWS == 41, "checkpoint layout");
   std::vector<Row> rows;
-  for (const CkptRow& r : checkpoint_rows(c)) rows.push_back({r.f, r.is_r == 2 || (r.is_r && c->mixed), buf + rows.size() * ncp});
+  for (const CkptRow& r : checkpoint_rows(c)) rows.push_back({r.f, r.is_r == 2 || (r.is_r && c->mixed), buf + rows.size() * ncp, 0});
   const int rc = gather_rows(c, L, rows, on_device);
   if (rc != KT_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));

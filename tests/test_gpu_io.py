@@ -56,3 +56,34 @@ def test_device_and_host_io_agree(mode, shape, baseline_eos):
         s = c.get_state()
         assert np.array_equal(s["e"], p.e) and np.array_equal(s["u"][1:], p.u)
         assert np.array_equal(s["pi"], p.pi) and np.array_equal(s["Pi"], p.Pi)
+
+
+def test_host_arrays_that_adjoin(baseline_eos):
+    """Output arrays pinned one by one that follow one another in memory: no copy spans two of them."""
+    import ctypes as C
+    import mmap
+    import torch
+    from paper_1608_06577_gb300 import KT
+    p = hotspot_problem(nx=16, ny=16, neta=32, nhot=5, seed=3, r_max=0.8, eos_table=baseline_eos)
+    n = p.ncells
+    sizes = {"e": (n,), "u": (4, n), "pi": (10, n), "Pi": (n,)}
+    buf = mmap.mmap(-1, 16 * n * 8)
+    assert (n * 8) % mmap.PAGESIZE == 0
+    base = C.addressof(C.c_char.from_buffer(buf))
+    out, at, rt, pinned = {}, 0, torch.cuda.cudart(), []
+    try:
+        for f, s in sizes.items():
+            nb = int(np.prod(s)) * 8
+            out[f] = np.frombuffer(buf, dtype=np.float64, count=nb // 8, offset=at).reshape(s)
+            assert int(rt.cudaHostRegister(base + at, nb, 0)) == 0
+            pinned.append(base + at)
+            at += nb
+        a = KT(p, precision=1)
+        a.set_problem_state()
+        ref = a.get_state()
+        got = a.get_state(fields=tuple(sizes), out=out)
+        for f in sizes:
+            assert np.array_equal(got[f], ref[f]), f
+    finally:
+        for q in pinned:
+            rt.cudaHostUnregister(q)
