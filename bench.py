@@ -48,8 +48,9 @@ BYTES_PER_CELL = {"fp64": 856, "mixed": 1088, "learned": 1128}
 ALG_BYTES_PER_CELL = {"fp64": 856, "mixed": 728, "learned": 728}
 # FP64 add/multiply/FMA instructions per cell and RK2 step of the FP64 mode (ncu counts of the two
 # fused stage kernels), and GB300's FP64 rate: 2 FMA per SM and clock (152 SMs; 1.25 TFLOP/s at
-# 2.07 GHz nominal), taken at the SM clock sampled during the timed steps
-FP64_INST_PER_CELL_STEP = 1799 + 1828
+# 2.07 GHz nominal), taken at the SM clock sampled during the timed steps.  (Measured, an SM takes one
+# FP64 warp instruction per 19.05 cycles, not 16: 0.84 of this peak is the real ceiling.)
+FP64_INST_PER_CELL_STEP = 1478 + 1509
 FP64_FMA_PER_SM_CLK = 2
 N_SM = 152
 # per launch slot of kt_time_kernels (bytes per cell); FP64: the fused stage kernels
@@ -73,15 +74,15 @@ LAUNCHES_PER_STEP = {"fp64": 2, "mixed": 4}  # (+ 1 for the network, learned sta
 # kernel ncu captures of the 96^3 learned workload, per cell times the 128^3 cells (average over
 # the two stages of each kernel; the update and fused kernels captured on 32x2x2 tiles, one block
 # per tile).  Only that mode (workload EOS) has a capture.
-MEASURED_TRAFFIC = {("learned", 128): {"rhs_kernel": 311.2e6, "update_kernel": 756.7e6, "fused_kernel": 827.8e6,
+MEASURED_TRAFFIC = {("learned", 128): {"rhs_kernel": 312.8e6, "update_kernel": 745.2e6, "fused_kernel": 821.8e6,
                                         "mlp_start_kernel": 85.4e6}}
 # Warp instructions per 32 cells of each launch slot (ncu smsp__inst_executed.sum over the warps of
 # one-kernel captures of the 96^3 learned workload, current kernels), for each kernel's fraction of
 # the SMs' issue rate: one warp instruction per scheduler and clock, 4 schedulers per SM.  The
 # kernels are bound by instruction issue and latency rather than by HBM.
-INST_PER_WARP = {"learned": {"learned_start": 259, "stage1_rhs": 2811, "stage2_rhs": 2811, "stage1_update": 1621,
-                             "stage2_update": 1914}}
-INST_PER_WARP_FUSED = {"learned": {"learned_start": 259, "stage1_rhs": 4319, "stage2_rhs": 4622}}  # fused launches
+INST_PER_WARP = {"learned": {"learned_start": 291, "stage1_rhs": 2556, "stage2_rhs": 2556, "stage1_update": 1706,
+                             "stage2_update": 2005}}
+INST_PER_WARP_FUSED = {"learned": {"learned_start": 291, "stage1_rhs": 4025, "stage2_rhs": 4372}}  # fused launches
 ISSUE_PER_SM_CLK = 4
 REPEATS = 3  # timed runs of K steps per mode; the median is reported
 
