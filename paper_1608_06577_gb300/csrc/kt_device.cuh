@@ -222,44 +222,43 @@ __device__ __forceinline__ double half_bits(double x) {
   const int hi = __double2hiint(x);
   return ((hi & 0x7ff00000) > 0x00100000) ? __hiloint2double(hi - 0x00100000, __double2loint(x)) : 0.0;
 }
-__device__ __forceinline__ float half_bits(float x) { return 0.5f * x; }
 
 // Generalised minmod of (theta dl, (dl + dr)/2, theta dr), Sec. 3.1, with sgn(0) = 0, from the
 // one-sided differences dl = q_i - q_{i-1}, dr = q_{i+1} - q_i: the three arguments share a sign
 // exactly when dl and dr do, and then the result is that sign times the smallest magnitude.
 // This is the slope times the cell size.
-// FP64: the signs and magnitudes are compared as integers (the magnitudes of doubles order like
-// their bit patterns), so only the theta branch does FP64 arithmetic.  FP32 with theta = 1: the
-// median of (dl, dr, 0) by four min/max instructions.  (FP32 theta != 1 tests the sign by the
-// product, which loses slopes whose one-sided differences multiply below ~1e-45.)
+// FP64 only: the signs and magnitudes are compared as integers (the magnitudes of doubles order like
+// their bit patterns), so only the theta branch does FP64 arithmetic.
 // (half_bits halves the sum in its exponent, off the FP64 pipe.)
 // TH1: theta = 1, where (|dl| + |dr|)/2 >= min(|dl|, |dr|) never decides.
 template <typename R, bool TH1 = false>
 __device__ __forceinline__ R limited_slope_d(R dl, R dr, R theta) {
-  if constexpr (sizeof(R) == 8) {
-    const long long bl = __double_as_longlong(dl), br = __double_as_longlong(dr);
-    const long long ml = bl & 0x7fffffffffffffffLL, mr = br & 0x7fffffffffffffffLL;
-    R m = (ml < mr) ? dl : dr;  // the smaller magnitude (0 if either is 0), with the shared sign
-    if constexpr (!TH1) {
-      const R m1 = theta * m, m2 = half_bits(dl + dr);
-      m = ((__double_as_longlong(m1) & 0x7fffffffffffffffLL) < (__double_as_longlong(m2) & 0x7fffffffffffffffLL))
-              ? m1 : m2;
-    }
-    return ((bl ^ br) >= 0) ? m : R(0);
-  } else if constexpr (TH1) {
-    return fmaxf(fminf(dl, dr), fminf(fmaxf(dl, dr), 0.f));
-  } else {
-    R mn = fmin(theta * fabs(dl), theta * fabs(dr));
-    mn = fmin(mn, R(0.5) * fabs(dl + dr));
-    return (dl * dr > R(0)) ? copysign(mn, dl) : R(0);
+  static_assert(sizeof(R) == 8, "three_slopes limits in FP32");
+  const long long bl = __double_as_longlong(dl), br = __double_as_longlong(dr);
+  const long long ml = bl & 0x7fffffffffffffffLL, mr = br & 0x7fffffffffffffffLL;
+  R m = (ml < mr) ? dl : dr;  // the smaller magnitude (0 if either is 0), with the shared sign
+  if constexpr (!TH1) {
+    const R m1 = theta * m, m2 = half_bits(dl + dr);
+    m = ((__double_as_longlong(m1) & 0x7fffffffffffffffLL) < (__double_as_longlong(m2) & 0x7fffffffffffffffLL))
+            ? m1 : m2;
   }
+  return ((bl ^ br) >= 0) ? m : R(0);
 }
 
 // The three slopes of a five-point stencil, s_{i-1}, s_i, s_{i+1}, from its one-sided differences
 // d0..d3.  FP32 with theta = 1: minmod(a, b) = clamp(a, min(0, b), max(0, b)) (zero when the signs
 // differ or either is zero, else the smaller magnitude), so s_i and s_{i+1} share the bounds from
 // d2: eight min/max instructions for the three, with min(x, 0) formed as x - max(x, 0) (exact) on the
-// FMA pipe, where the ALU pipe that runs min/max is the busier one.  Otherwise limited_slope_d for each.
+// FMA pipe, where the ALU pipe that runs min/max is the busier one.  FP32 otherwise: the mean of two
+// differences clamped to the intersection of [min(0, theta d), max(0, theta d)] of both, which is {0} when
+// the signs differ.  FP64: limited_slope_d for each.
+__device__ __forceinline__ void slope_bounds(float td, float& hi, float& lo) {
+  hi = fmaxf(td, 0.f);
+  lo = td - hi;
+}
+__device__ __forceinline__ float clamp_slope(float c, float ha, float la, float hb, float lb) {
+  return fminf(fminf(fmaxf(fmaxf(c, la), lb), ha), hb);
+}
 template <typename R, bool TH1>
 __device__ __forceinline__ void three_slopes(R d0, R d1, R d2, R d3, R th, R& sm, R& s0, R& sp) {
   if constexpr (sizeof(R) == 4 && TH1) {
@@ -267,6 +266,15 @@ __device__ __forceinline__ void three_slopes(R d0, R d1, R d2, R d3, R th, R& sm
     sm = fminf(fmaxf(d0, lo1), hi1);
     s0 = fminf(fmaxf(d1, lo2), hi2);
     sp = fminf(fmaxf(d3, lo2), hi2);
+  } else if constexpr (sizeof(R) == 4) {
+    R h0, h1, h2, h3, l0, l1, l2, l3;
+    slope_bounds(__fmul_rn(th, d0), h0, l0);
+    slope_bounds(__fmul_rn(th, d1), h1, l1);
+    slope_bounds(__fmul_rn(th, d2), h2, l2);
+    slope_bounds(__fmul_rn(th, d3), h3, l3);
+    sm = clamp_slope(0.5f * (d0 + d1), h0, l0, h1, l1);
+    s0 = clamp_slope(0.5f * (d1 + d2), h1, l1, h2, l2);
+    sp = clamp_slope(0.5f * (d2 + d3), h2, l2, h3, l3);
   } else {
     sm = limited_slope_d<R, TH1>(d0, d1, th);
     s0 = limited_slope_d<R, TH1>(d1, d2, th);

@@ -157,7 +157,7 @@ __global__ void __maxnreg__(96)
       cell_sources<float>(P, L, io, c, G, uc, du, dv, dq);
     }
 
-    const FacesXY Wxy = faces_xy(Fx, Fy);  // theta = 1: the x and y fluxes in paired instructions
+    const FacesXY Wxy = faces_xy(Fx, Fy);  // the x and y fluxes in paired instructions
 #pragma unroll  // unrolled: the component index, the rows it feeds and every branch become constants
     for (int g = 0; g < kGroups; ++g) {
       if (g + 1 < kGroups) {
@@ -171,13 +171,8 @@ __global__ void __maxnreg__(96)
       if (valid) {
 #pragma unroll
         for (int m = 0; m < kCompPerBox; ++m)
-          if (kCompPerBox * g + m < NQ) {
-            if constexpr (TH1)
-              component_rhs_xy(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, sy, sz, Wxy, Fx, Fy, Fz, dq);
-            else
-              component_rhs<float, true, TH1>(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, 1, sy, sz, th,
-                                              Fx, Fy, Fz, dq);
-          }
+          if (kCompPerBox * g + m < NQ)
+            component_rhs_xy<TH1>(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, sy, sz, Wxy, Fx, Fy, Fz, th, dq);
       }
     }
     if (valid && !bad) {  // (a timed-out block leaves at the next tile's barrier)
@@ -761,13 +756,8 @@ __global__ void __maxnreg__(128)
       if (valid) {
 #pragma unroll
         for (int m = 0; m < kCompPerBox; ++m)
-          if (kCompPerBox * g + m < NQ) {
-            if constexpr (TH1)
-              component_rhs_xy(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, sy, sz, Wxy, Fx, Fy, Fz, dq);
-            else
-              component_rhs<float, true, TH1>(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, 1, sy, sz, th,
-                                              Fx, Fy, Fz, dq);
-          }
+          if (kCompPerBox * g + m < NQ)
+            component_rhs_xy<TH1>(P, kCompPerBox * g + m, s_q + b * bfl + m * vol + own, sy, sz, Wxy, Fx, Fy, Fz, th, dq);
       }
     }
     if (__syncthreads_or(bad)) { bad = true; break; }  // the update runs for every tile of every block, or none

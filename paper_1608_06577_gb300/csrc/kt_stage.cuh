@@ -290,51 +290,21 @@ __device__ __forceinline__ void add_row(R (&dq)[NQ], int r, R v) {
   }
 }
 
-// one component along one direction: generalised-minmod reconstruction from the five-point
-// stencil p[-2s..2s] (a0 = p[0] given; global memory, or shared memory if SMEM) and the flux
-// difference -(H_R - H_L)/dx without its q_i term, added to acc; a1, b1 return the neighbours for
-// the central differences of S_c
-template <typename R, bool SMEM, bool TH1 = false>
-__device__ __forceinline__ R component_flux(const R* p, int s, R a0, R th, const Faces<R>& F, R& a1, R& b1, R acc) {
-  R a2, b2;
-  if constexpr (SMEM) {
-    a2 = p[-2 * s]; a1 = p[-s]; b1 = p[s]; b2 = p[2 * s];
-  } else {
-    const long long e = s;
-    a2 = ld<R>(p, -2 * e); a1 = ld<R>(p, -e); b1 = ld<R>(p, e); b2 = ld<R>(p, 2 * e);
-  }
-  const R d0 = a1 - a2, d1 = a0 - a1, d2 = b1 - a0, d3 = b2 - b1;
-  R sm, s0, sp;
-  three_slopes<R, TH1>(d0, d1, d2, d3, th, sm, s0, sp);
-  acc = fma(F.wLm, fma(R(0.5), sm, a1), acc);
-  acc = fma(F.wRp, fma(R(-0.5), sp, b1), acc);
+// one component along one direction: generalised-minmod reconstruction from the five-point FP32
+// stencil p[-2s..2s] in shared memory (a0 = p[0] given) and the flux difference -(H_R - H_L)/dx without
+// its q_i term, added to acc; a1, b1 return the neighbours for the central differences of S_c
+template <bool TH1>
+__device__ __forceinline__ float component_flux(const float* p, int s, float a0, float th, const Faces<float>& F,
+                                                float& a1, float& b1, float acc) {
+  const float a2 = p[-2 * s], b2 = p[2 * s];
+  a1 = p[-s];
+  b1 = p[s];
+  const float d0 = a1 - a2, d1 = a0 - a1, d2 = b1 - a0, d3 = b2 - b1;
+  float sm, s0, sp;
+  three_slopes<float, TH1>(d0, d1, d2, d3, th, sm, s0, sp);
+  acc = fma(F.wLm, fma(0.5f, sm, a1), acc);
+  acc = fma(F.wRp, fma(-0.5f, sp, b1), acc);
   return fma(F.hdW, s0, acc);
-}
-
-// Component n (warp-uniform) of the 15 conserved components, at a cell whose stencil starts at
-// p with strides sx, sy, sz: -div H in x, y, eta and the remaining S_c terms
-// -d_d(-v^d pi^{tau nu} + pi^{d nu}) by central differences, added to dq.
-template <typename R, bool SMEM, bool TH1 = false>
-__device__ __forceinline__ void component_rhs(const Params& P, int n, const R* p, int sx, int sy, int sz, R th,
-                                              const Faces<R>& Fx, const Faces<R>& Fy, const Faces<R>& Fz,
-                                              R (&dq)[NQ]) {
-  const R a0 = SMEM ? p[0] : ld<R>(p, 0LL);
-  R a1x, b1x, a1y, b1y, a1z, b1z;
-  R acc = component_flux<R, SMEM, TH1>(p, sx, a0, th, Fx, a1x, b1x, (Fx.c0 + Fy.c0 + Fz.c0) * a0);
-  acc = component_flux<R, SMEM, TH1>(p, sy, a0, th, Fy, a1y, b1y, acc);
-  acc = component_flux<R, SMEM, TH1>(p, sz, a0, th, Fz, a1z, b1z, acc);
-  add_row(dq, n, acc);
-  if (n >= 4 && n <= 13) {  // pi components
-    const int r0 = cross_row<0>(n, true);
-    if (r0 >= 0)
-      add_row(dq, r0, (Fx.vpl_h * b1x - Fx.vmi_h * a1x) + (Fy.vpl_h * b1y - Fy.vmi_h * a1y) +
-                          (Fz.vpl_h * b1z - Fz.vmi_h * a1z));
-    const int rx = cross_row<0>(n, false), ry = cross_row<1>(n, false), rz = cross_row<2>(n, false);
-    const R* hinv = pr<R>(P).half_inv_d;  // kernel parameters: no registers held across the loop
-    if (rx >= 0) add_row(dq, rx, -(b1x - a1x) * hinv[0]);
-    if (ry >= 0) add_row(dq, ry, -(b1y - a1y) * hinv[1]);
-    if (rz >= 0) add_row(dq, rz, -(b1z - a1z) * hinv[2]);
-  }
 }
 
 // ---- paired FP32 arithmetic (the f32x2 instructions of the sm_100 family): two independent
@@ -350,6 +320,11 @@ __device__ __forceinline__ void up2(unsigned long long v, float& lo, float& hi) 
 __device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
   unsigned long long r;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
@@ -371,13 +346,16 @@ __device__ __forceinline__ FacesXY faces_xy(const Faces<float>& Fx, const Faces<
   return FacesXY{pk2(Fx.wLm, Fy.wLm), pk2(Fx.wRp, Fy.wRp), pk2(Fx.hdW, Fy.hdW)};
 }
 
-// component_rhs for the FP32 stencil in shared memory with theta = 1, the x and y directions
-// computed as pairs: the differences and the five multiply-adds of the two directions share
-// instructions; the limiter's min/max and the eta direction stay scalar.
-// The same arithmetic as component_rhs, summed x + y, then eta.
+// Component n (warp-uniform) of the 15 conserved components, at a cell whose FP32 stencil starts at p in
+// shared memory with strides 1, sy, sz: -div H in x, y, eta and the remaining S_c terms
+// -d_d(-v^d pi^{tau nu} + pi^{d nu}) by central differences, added to dq.  The x and y directions are
+// computed as pairs: the differences, bounds and five multiply-adds of the two share instructions; the
+// limiter's min/max and the eta direction stay scalar.  With theta != 1 (96 x 96 x 64, theta = 1.3) the
+// right-hand side took 82 us per launch with scalar directions and a sign test per slope, 76 us so.
+template <bool TH1>
 __device__ __forceinline__ void component_rhs_xy(const Params& P, int n, const float* p, int sy, int sz,
                                                  const FacesXY& W, const Faces<float>& Fx, const Faces<float>& Fy,
-                                                 const Faces<float>& Fz, float (&dq)[NQ]) {
+                                                 const Faces<float>& Fz, float th, float (&dq)[NQ]) {
   const float a0 = p[0];
   const float a2x = p[-2], a1x = p[-1], b1x = p[1], b2x = p[2];
   const float a2y = p[-2 * sy], a1y = p[-sy], b1y = p[sy], b2y = p[2 * sy];
@@ -389,24 +367,50 @@ __device__ __forceinline__ void component_rhs_xy(const Params& P, int n, const f
   up2(D1, d1x, d1y);
   up2(D2, d2x, d2y);
   up2(D3, d3x, d3y);
-  // three_slopes for both directions, the lower bounds as pairs
-  const float h1x = fmaxf(d1x, 0.f), h1y = fmaxf(d1y, 0.f), h2x = fmaxf(d2x, 0.f), h2y = fmaxf(d2y, 0.f);
-  float l1x, l1y, l2x, l2y;
-  up2(sub2(D1, pk2(h1x, h1y)), l1x, l1y);
-  up2(sub2(D2, pk2(h2x, h2y)), l2x, l2y);
-  smx = fminf(fmaxf(d0x, l1x), h1x);
-  smy = fminf(fmaxf(d0y, l1y), h1y);
-  s0x = fminf(fmaxf(d1x, l2x), h2x);
-  s0y = fminf(fmaxf(d1y, l2y), h2y);
-  spx = fminf(fmaxf(d3x, l2x), h2x);
-  spy = fminf(fmaxf(d3y, l2y), h2y);
+  // three_slopes for both directions
+  if constexpr (TH1) {
+    const float h1x = fmaxf(d1x, 0.f), h1y = fmaxf(d1y, 0.f), h2x = fmaxf(d2x, 0.f), h2y = fmaxf(d2y, 0.f);
+    float l1x, l1y, l2x, l2y;
+    up2(sub2(D1, pk2(h1x, h1y)), l1x, l1y);
+    up2(sub2(D2, pk2(h2x, h2y)), l2x, l2y);
+    smx = fminf(fmaxf(d0x, l1x), h1x);
+    smy = fminf(fmaxf(d0y, l1y), h1y);
+    s0x = fminf(fmaxf(d1x, l2x), h2x);
+    s0y = fminf(fmaxf(d1y, l2y), h2y);
+    spx = fminf(fmaxf(d3x, l2x), h2x);
+    spy = fminf(fmaxf(d3y, l2y), h2y);
+  } else {
+    const unsigned long long T = pk2(th, th), H = pk2(0.5f, 0.5f);
+    float h0x, h0y, l0x, l0y, h1x, h1y, l1x, l1y, h2x, h2y, l2x, l2y, h3x, h3y, l3x, l3y, cx, cy;
+    const auto bounds = [&](unsigned long long D, float& hx, float& hy, float& lx, float& ly) {
+      const unsigned long long t = mul2(T, D);
+      float tx, ty;
+      up2(t, tx, ty);
+      hx = fmaxf(tx, 0.f);
+      hy = fmaxf(ty, 0.f);
+      up2(sub2(t, pk2(hx, hy)), lx, ly);
+    };
+    bounds(D0, h0x, h0y, l0x, l0y);
+    bounds(D1, h1x, h1y, l1x, l1y);
+    bounds(D2, h2x, h2y, l2x, l2y);
+    bounds(D3, h3x, h3y, l3x, l3y);
+    up2(mul2(H, add2(D0, D1)), cx, cy);
+    smx = clamp_slope(cx, h0x, l0x, h1x, l1x);
+    smy = clamp_slope(cy, h0y, l0y, h1y, l1y);
+    up2(mul2(H, add2(D1, D2)), cx, cy);
+    s0x = clamp_slope(cx, h1x, l1x, h2x, l2x);
+    s0y = clamp_slope(cy, h1y, l1y, h2y, l2y);
+    up2(mul2(H, add2(D2, D3)), cx, cy);
+    spx = clamp_slope(cx, h2x, l2x, h3x, l3x);
+    spy = clamp_slope(cy, h2y, l2y, h3y, l3y);
+  }
   unsigned long long acc = mul2(W.wLm, fma2(pk2(0.5f, 0.5f), pk2(smx, smy), A1));
   acc = fma2(W.wRp, fma2(pk2(-0.5f, -0.5f), pk2(spx, spy), B1), acc);
   acc = fma2(W.hdW, pk2(s0x, s0y), acc);
   float accx, accy, a1z, b1z;
   up2(acc, accx, accy);
   const float accz =
-      component_flux<float, true, true>(p, sz, a0, 1.f, Fz, a1z, b1z, fmaf(Fx.c0 + Fy.c0 + Fz.c0, a0, accx + accy));
+      component_flux<TH1>(p, sz, a0, th, Fz, a1z, b1z, fmaf(Fx.c0 + Fy.c0 + Fz.c0, a0, accx + accy));
   add_row(dq, n, accz);
   if (n >= 4 && n <= 13) {  // pi components
     const int r0 = cross_row<0>(n, true);
