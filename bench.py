@@ -534,7 +534,8 @@ def run_ours(args, world, rank, local):
                 "learned_training": train_info,
                 "roofline": roofline, "kernels": kernels, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
                 "gpu_launches": (LAUNCHES_PER_STEP["fp64" if (args.mode == "fp64" or fused) else "mixed"]
-                                 + (1 if MODES[args.mode][1] == 1 else 0)) * main["steps"]}
+                                 + (1 if MODES[args.mode][1] == 1 else 0)
+                                 + (2 if args.iface == "invert" and args.mode != "fp64" else 0)) * main["steps"]}
         print(json.dumps(line), flush=True)
 
 

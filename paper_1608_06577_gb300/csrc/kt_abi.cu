@@ -614,9 +614,17 @@ StageIO<R> make_io(Ctx* c, int stage) {
   if constexpr (sizeof(R) == 4) {
     io.qr_in = (stage == 1) ? c->qf : c->qsf;
     io.qr_out = (stage == 1) ? c->qsf : c->qf;
+    // Six components that nothing else holds while a stage's faces are in use: k_2 in the first stage, the
+    // FP32 copy of q^n in the second (its update writes q^{n+1} there, ghosts included); with FP32 pi
+    // storage, which reads that copy there, the FP64 pi and Pi that it does not use.
+    io.fv = !c->P.iface_invert ? nullptr
+            : c->pi32          ? (const R*)(c->q + 4 * c->gs)
+            : (stage == 1)     ? (const R*)((float*)c->qs + 15 * c->gs)
+                               : (const R*)c->qf;
   } else {
     io.qr_in = (const R*)io.q_in;
     io.qr_out = nullptr;
+    io.fv = nullptr;
   }
   io.tau = c->d_tau + c->cur;
   io.tau_next = (stage == 2) ? c->d_tau + c->spare : nullptr;  // the next step's u^n buffer and tau slot
@@ -705,6 +713,17 @@ void with_flags(F&& f, bool b, B... rest) {
 template <int STAGE>
 void launch_rhs(Ctx* c, const StageIO<float>& io) {
   const Shape& s = kShapes[c->shape];
+  if (c->P.iface_invert) {
+    unsigned faces = 1;  // of the event and direction with the most
+    for (const Lattice& L : c->lat)
+      for (int d = 0; d < 3; ++d)
+        faces = std::max(faces, (unsigned)(L.nx + (d == 0)) * (unsigned)(L.ny + (d == 1)) * (unsigned)(L.nz + (d == 2)));
+    const dim3 grid((faces + kt::kFaceThreads - 1) / kt::kFaceThreads, 3, (unsigned)std::min(c->nev, 65535));
+    with_flags([&](auto t1) {
+      kt::face_velocity_kernel<t1.value><<<grid, kt::kFaceThreads, 0, c->stream>>>(
+          c->P, io.qr_in, io.e_in, io.tau, STAGE, c->d_lat, c->nev, (float*)io.fv);
+    }, c->P.theta == 1.0);
+  }
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
   with_flags([&](auto single, auto t1, auto inv, auto fixed) {
     constexpr int f = fixed.value ? 2 : 0;

@@ -39,6 +39,7 @@ struct StageIO {
   unsigned long long* counters;  // [0] Newton iterations, [1] regulated cells, [2] fallbacks
   const uint32_t* mlp_packed;  // learned start: packed weights (see kt_mlp.cuh), or null
   float* reg_out;        // stage 2: the regulation factor applied to pi^{n+1} at each cell, or null
+  const R* fv;           // FP32, KT_IFACE_INVERT: v^m, v^p of the faces i+1/2 of x, y, eta (face_velocity_kernel)
 };
 
 // ------------------------------------------------------------------ a) the stencil
@@ -65,9 +66,9 @@ struct Faces {
 // returns A at the root (v^d = M^d / A), or false if the state has none (E <= 0, M^2 >= E^2, no
 // convergence in 100 steps).  FP64: the cell root-find (stop at |de| <= 2^-50 E, below).  FP32: stop at
 // |de| <= 2^-21 E; the residual in product form g = (e - E) A + M^2 = f A, so that a step takes two fast
-// divisions, and the interval's record in two vector loads.  Twelve of these per cell and stage bound the
-// kernel; with IEEE divisions and eos_interval's dependent loads six steps of a 72 x 64 x 40 box took
-// 2.24 ms, so 1.66 ms.
+// divisions, and the interval's record in two vector loads.  Six of these per cell and stage bound such a
+// step (face_velocity_kernel); with IEEE divisions and eos_interval's dependent loads six steps of a 72 x
+// 64 x 40 box took 2.24 ms, so 1.66 ms, when each cell inverted the four states of both its faces.
 __device__ __forceinline__ FaceSeg face_seg(const Params& P, float e) {
   const int n1 = P.eos_n - 2;
   const float g = (__logf(e) - P.lne0) * P.inv_h;
@@ -127,7 +128,8 @@ __device__ __forceinline__ bool face_root(const Params& P, R E, R M2, R Pi, R gu
 // KT_IFACE_INVERT (literal reading of Sec. 3.1): the four extrapolated states along D -- left face
 // m (from cell i-1) and p (from cell i), right face m (from cell i) and p (from cell i+1) -- of the
 // components the root-find reads (T^{tau mu}, pi^{tau mu}, Pi), each inverted from the e of the cell
-// it was extrapolated from; v^d = M^d / (E + P0 + Pi) at the root, 0 for a state without one.
+// it was extrapolated from; v^d = M^d / (E + P0 + Pi) at the root, 0 for a state without one.  FP64; in
+// FP32 face_velocity_kernel has inverted every face once.
 template <typename R, int D, bool TH1>
 __device__ __forceinline__ void face_velocities_inverted(const Params& P, const Lattice& L, const StageIO<R>& io,
                                                          Idx<R> c, int s, R th, R gnn, R& vLm, R& vLp, R& vRm,
@@ -163,6 +165,40 @@ __device__ __forceinline__ void face_velocities_inverted(const Params& P, const 
     v[j] = face_root<R>(P, E4[j], M2, Pi4[j], g[j], A) ? sdiv(M4[D][j], A) : R(0);
   }
   vLm = v[0]; vLp = v[1]; vRm = v[2]; vRp = v[3];
+}
+
+// The same in FP32 for one face, i+1/2 of cell c: v^m from the state of cell i, v^p from that of i+1.
+template <int D, bool TH1>
+__device__ __forceinline__ void face_velocities_right(const Params& P, const float* q, const float* e, long long fs,
+                                                      unsigned c, int s, float th, float gnn, float& vm, float& vp) {
+  float E[2] = {0.f, 0.f}, M[3][2] = {}, Pi[2];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const int n = (k < 8) ? k : 14;
+    const float* p = q + n * fs;
+    const float a1 = ld<float>(p, c - s), a0 = ld<float>(p, c), b1 = ld<float>(p, c + s), b2 = ld<float>(p, c + 2 * s);
+    const float d1 = a0 - a1, d2 = b1 - a0, d3 = b2 - b1;
+    float sm, s0, sp;
+    three_slopes<float, TH1>(d1, d1, d2, d3, th, sm, s0, sp);
+    const float x[2] = {fmaf(0.5f, s0, a0), fmaf(-0.5f, sp, b1)};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (n == 0) E[j] += x[j];
+      else if (n == 4) E[j] -= x[j];
+      else if (n < 4) M[n - 1][j] += x[j];
+      else if (n < 8) M[n - 5][j] -= x[j];
+      else Pi[j] = x[j];
+    }
+  }
+  float v[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float M2 = fmaf(M[0][j], M[0][j], fmaf(M[1][j], M[1][j], rmul(rmul(gnn, M[2][j]), M[2][j])));
+    float A;
+    v[j] = face_root<float>(P, E[j], M2, Pi[j], ld<float>(e, j ? c + s : c), A) ? sdiv(M[D][j], A) : 0.f;
+  }
+  vm = v[0];
+  vp = v[1];
 }
 
 // How the stencil reads u^mu around cell c: from the field arrays, through the read-only cache.
@@ -202,7 +238,12 @@ __device__ __forceinline__ void face_setup(const Params& P, const Lattice& L, co
     up1[m] = ua(m, us);
   }
   R vLm, vLp, vRm, vRp;
-  if constexpr (IFACE) {
+  if constexpr (IFACE && sizeof(R) == 4) {
+    const R* vm = io.fv + 2 * D * fs;
+    const R* vp = vm + fs;
+    vLm = ld<R>(vm, c - s); vLp = ld<R>(vp, c - s);
+    vRm = ld<R>(vm, c); vRp = ld<R>(vp, c);
+  } else if constexpr (IFACE) {
     face_velocities_inverted<R, D, TH1>(P, L, io, c, s, th, sfac * sfac, vLm, vLp, vRm, vRp);
   } else {
     const R u0t = uc[0], u0d = uc[D + 1];
