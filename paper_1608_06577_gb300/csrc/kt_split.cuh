@@ -7,6 +7,7 @@
 //                   the stores (c-f).
 // fused_kernel<S>:  both in one launch, k in shared memory.
 // mlp_start_kernel: the network's output z for every cell at the start of the step (tensor cores).
+// face_velocity_kernel: with KT_IFACE_INVERT, the velocities of every face, before each right-hand side.
 //
 // Heun (Eqs. step1-finalStep) in increment form:
 //     q*      = q^n + k_1,            k_1 = dtau C[q^n]

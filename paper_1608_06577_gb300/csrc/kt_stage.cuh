@@ -1,4 +1,5 @@
-// kt_stage.cuh -- the fused KT + Heun stage kernel (one launch per Runge-Kutta stage).
+// kt_stage.cuh -- the fused KT + Heun stage kernels of the FP64 path (one launch per Runge-Kutta stage;
+// stage_kernel, and stage_team_kernel for small grids) and what they share with the mixed path.
 //
 // One thread owns one physical cell and performs, in order (Sec. 4.3 steps 1-4 / 5-8):
 //   a) for x, y, eta: generalised-minmod slopes of the 15 conserved components and of u^tau,
