@@ -664,7 +664,8 @@ UpdIO make_uio(Ctx* c, int stage) {
 
 // Two blocks of stage_team_kernel are resident per SM: beyond 304 strips a second wave doubles its time.
 // 12 viscous steps (us), one warp / four warps per strip: 64 strips 1672 / 1081, 480 strips 1692 / 2292;
-// the Gubser grid (256 strips, 20 steps) 3390 / 2255, the shock tube (7 strips, 80 steps) 3503 / 2955.
+// the Gubser grid (256 strips, 20 steps) 3390 / 2255 (2046 with the sources in a warp of their own), the
+// shock tube (7 strips, 80 steps) 3503 / 2955 (2912).
 constexpr int kTeamStrips = 2 * 152;
 
 template <int STAGE>
