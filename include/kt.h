@@ -244,7 +244,9 @@ void kt_free(kt_ctx* ctx);
  * persistent launch per Runge-Kutta stage walks a table of (event, tile) work items.  All
  * events share the physics parameters, dtau and tau.  kt_init is kt_init_batch with one event;
  * kt_set_state / kt_get_state address event 0.  kt_step advances every event; each event must
- * have been given a state first.  The results of an event do not depend on the batch it is in. */
+ * have been given a state first.  The results of an event do not depend on the batch it is in.
+ * KT_MIXED: one event's padded lattice must have less than 2^29 cells (KT_ERR_ARG; the state of a larger
+ * one would not fit on the device); a batch may hold any number. */
 int kt_state_bytes_batch(int n_events, const kt_grid* grids, const kt_eos* eos, const kt_options* opt,
                          size_t* bytes);
 int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, double deta, double dtau,

@@ -42,6 +42,14 @@ constexpr int kNumBase = 2 * kNumShapes;
 constexpr int kNumCandidates = 3 * kNumBase;
 constexpr int kFusedFirst = 2 * kNumBase;
 
+// A run of events [ev0, ev1) that the mixed-precision kernels take in one launch: their lattices lie within
+// kSpanElements of `base`, where the launch's field pointers start.  tile0, ntiles: their tiles.
+struct Span {
+  int ev0, ev1;
+  long long base;
+  int tile0, ntiles;
+};
+
 struct Ctx {
   kt_options opt;
   Params P;
@@ -52,6 +60,7 @@ struct Ctx {
   // events
   int nev = 0;
   std::vector<Lattice> lat;
+  std::vector<Span> spans;  // mixed precision: the events of each launch
   long long gs = 0;      // component stride of every field array
   size_t max_cells = 0;  // physical cells of the largest event
   std::vector<char> ev_set;
@@ -75,7 +84,7 @@ struct Ctx {
   unsigned* d_stat = nullptr;
   float* d_mlp = nullptr;
   uint32_t* d_mlp_packed = nullptr;
-  Lattice* d_lat = nullptr;
+  Lattice* d_lat = nullptr;        // mixed precision: bases relative to the event's span
   Tile* d_tiles = nullptr;
   CUtensorMap map0[2] = {};        // mixed precision: the first event's maps of qf and qsf (kernel parameters)
   CUtensorMap* d_tmaps = nullptr;  // mixed precision: per event, the 4-d maps of qf (first nev) and qsf
@@ -157,10 +166,30 @@ void layout(int nev, const kt_grid* grids, std::vector<Lattice>& lat, long long&
   for (auto& L : lat) L.fstride = gs;
 }
 
+// first element after event e's lattice
+long long end_of(const std::vector<Lattice>& lat, long long gs, size_t e) {
+  return (e + 1 < lat.size()) ? lat[e + 1].base : gs;
+}
+
+// the events in as few runs of less than kSpanElements as their order allows (almost always one); false if
+// an event alone is larger
+bool make_spans(const std::vector<Lattice>& lat, long long gs, std::vector<Span>& spans) {
+  spans.clear();
+  for (size_t e = 0; e < lat.size(); ++e) {
+    if (end_of(lat, gs, e) - lat[e].base >= kSpanElements) return false;
+    if (spans.empty() || end_of(lat, gs, e) - spans.back().base >= kSpanElements)
+      spans.push_back(Span{(int)e, (int)e, lat[e].base, 0, 0});
+    spans.back().ev1 = (int)e + 1;
+  }
+  return true;
+}
+
+long long tiles_of(const Lattice& L, const Shape& s) {
+  return (long long)((L.nx + s.x - 1) / s.x) * ((L.ny + s.y - 1) / s.y) * ((L.nz + s.z - 1) / s.z);
+}
 int tiles_for(const std::vector<Lattice>& lat, const Shape& s) {
   long long n = 0;
-  for (const auto& L : lat)
-    n += (long long)((L.nx + s.x - 1) / s.x) * ((L.ny + s.y - 1) / s.y) * ((L.nz + s.z - 1) / s.z);
+  for (const auto& L : lat) n += tiles_of(L, s);
   return (int)n;
 }
 
@@ -636,6 +665,23 @@ StageIO<R> make_io(Ctx* c, int stage) {
   return io;
 }
 
+// the same fields from element `off` of every component on
+template <typename R>
+StageIO<R> from(StageIO<R> io, long long off) {
+  auto move = [&](auto& p) { if (p) p += off; };
+  move(io.q_in); move(io.q_base); move(io.q_out); move(io.qr_in); move(io.qr_out);
+  move(io.u_in); move(io.u_prev); move(io.u_out);
+  move(io.e_in); move(io.p_in); move(io.e_out); move(io.p_out);
+  move(io.reg_out); move(io.fv);
+  return io;
+}
+UpdIO from(UpdIO u, long long off) {
+  auto move = [&](auto& p) { if (p) p += off; };
+  move(u.q); move(u.qf_n); move(u.qsf); move(u.k1); move(u.k2); move(u.qr_out);
+  move(u.u_out); move(u.e_out); move(u.p_out); move(u.e_guess); move(u.reg_out); move(u.z_net);
+  return u;
+}
+
 // Mixed precision: the Runge-Kutta increments k_1, k_2 (FP32, 15 components each) live in the
 // memory of the FP64 q* array, which that path never stores.
 float* k_buf(Ctx* c, int stage) { return (float*)c->qs + (stage == 1 ? 0 : 15 * c->gs); }
@@ -689,15 +735,16 @@ void launch_stage(Ctx* c, const StageIO<double>& io) {
   else go(stage_kernel<double, STAGE, false, true>);
 }
 
-Work make_work(Ctx* c) {
+Work make_work(Ctx* c, const Span& sp) {
   const Shape& s = kShapes[c->shape];
   Work w;
-  w.L0 = c->lat[0];
+  w.L0 = c->lat[sp.ev0];
+  w.L0.base = 0;
   w.tk = (unsigned)((w.L0.nz + s.z - 1) / s.z);
   w.ti = (unsigned)((w.L0.nx + s.x - 1) / s.x);
-  w.ntiles = c->ntiles;
+  w.ntiles = sp.ntiles;
   w.lats = c->d_lat;
-  w.tiles = c->d_tiles;
+  w.tiles = c->d_tiles + sp.tile0;
   return w;
 }
 
@@ -719,19 +766,23 @@ void launch_rhs(Ctx* c, const StageIO<float>& io) {
     for (const Lattice& L : c->lat)
       for (int d = 0; d < 3; ++d)
         faces = std::max(faces, (unsigned)(L.nx + (d == 0)) * (unsigned)(L.ny + (d == 1)) * (unsigned)(L.nz + (d == 2)));
-    const dim3 grid((faces + kt::kFaceThreads - 1) / kt::kFaceThreads, 3, (unsigned)std::min(c->nev, 65535));
-    with_flags([&](auto t1) {
-      kt::face_velocity_kernel<t1.value><<<grid, kt::kFaceThreads, 0, c->stream>>>(
-          c->P, io.qr_in, io.e_in, io.tau, STAGE, c->d_lat, c->nev, (float*)io.fv);
-    }, c->P.theta == 1.0);
+    for (const Span& sp : c->spans) {
+      const int n = sp.ev1 - sp.ev0;
+      const dim3 grid((faces + kt::kFaceThreads - 1) / kt::kFaceThreads, 3, (unsigned)std::min(n, 65535));
+      with_flags([&](auto t1) {
+        kt::face_velocity_kernel<t1.value><<<grid, kt::kFaceThreads, 0, c->stream>>>(
+            c->P, io.qr_in + sp.base, io.e_in + sp.base, io.tau, STAGE, c->d_lat + sp.ev0, n, (float*)io.fv + sp.base);
+      }, c->P.theta == 1.0);
+    }
   }
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  with_flags([&](auto single, auto t1, auto inv, auto fixed) {
-    constexpr int f = fixed.value ? 2 : 0;
-    rhs_kernel<single.value, t1.value, inv.value, f, f>
-        <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
-            c->P, io, STAGE, k_buf(c, STAGE), make_work(c), c->map0[STAGE - 1], maps);
-  }, c->nev == 1, c->P.theta == 1.0, c->P.iface_invert != 0, s.y == 2 && s.z == 2);
+  for (const Span& sp : c->spans)
+    with_flags([&](auto single, auto t1, auto inv, auto fixed) {
+      constexpr int f = fixed.value ? 2 : 0;
+      rhs_kernel<single.value, t1.value, inv.value, f, f>
+          <<<std::min(c->grid_rhs, sp.ntiles), dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
+              c->P, from(io, sp.base), STAGE, k_buf(c, STAGE) + sp.base, make_work(c, sp), c->map0[STAGE - 1], maps);
+    }, c->nev == 1, c->P.theta == 1.0, c->P.iface_invert != 0, s.y == 2 && s.z == 2);
 }
 
 // every rhs kernel may take the dynamic shared memory of the largest tile shape
@@ -768,17 +819,18 @@ void launch_update(Ctx* c, const UpdIO& uio) {
   const dim3 blk(s.x, s.y, s.z);
   if (c->staged && !c->pi32) {
     const size_t sm = upd_smem_bytes(s.x, s.y, s.z, c->upd_nbuf);
-    if (c->learned)
-      update_staged_kernel<STAGE, true><<<c->grid_upd, blk, sm, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles,
-                                                                             c->ntiles, c->d_umaps, c->upd_nbuf);
-    else
-      update_staged_kernel<STAGE, false><<<c->grid_upd, blk, sm, c->stream>>>(c->P, uio, c->d_lat, c->d_tiles,
-                                                                              c->ntiles, c->d_umaps, c->upd_nbuf);
+    for (const Span& sp : c->spans)
+      with_flags([&](auto learned) {
+        update_staged_kernel<STAGE, learned.value><<<std::min(c->grid_upd, sp.ntiles), blk, sm, c->stream>>>(
+            c->P, from(uio, sp.base), c->d_lat, c->d_tiles + sp.tile0, sp.ntiles, c->d_umaps, c->upd_nbuf);
+      }, c->learned != 0);
     return;
   }
-  with_flags([&](auto single, auto learned, auto pi32) {
-    update_kernel<single.value, STAGE, learned.value, pi32.value><<<c->grid_upd, blk, 0, c->stream>>>(c->P, uio, make_work(c));
-  }, c->nev == 1, c->learned != 0, c->pi32 != 0);
+  for (const Span& sp : c->spans)
+    with_flags([&](auto single, auto learned, auto pi32) {
+      update_kernel<single.value, STAGE, learned.value, pi32.value>
+          <<<std::min(c->grid_upd, sp.ntiles), blk, 0, c->stream>>>(c->P, from(uio, sp.base), make_work(c, sp));
+    }, c->nev == 1, c->learned != 0, c->pi32 != 0);
 }
 
 // the fused stage kernel (right-hand side and update in one launch)
@@ -786,12 +838,13 @@ template <int STAGE>
 void launch_fused(Ctx* c, const StageIO<float>& io, const UpdIO& uio) {
   const Shape& s = kShapes[c->shape];
   const CUtensorMap* maps = c->d_tmaps + (STAGE == 1 ? 0 : c->nev);
-  with_flags([&](auto single, auto t1, auto learned, auto fixed) {
-    constexpr int f = fixed.value ? 2 : 0;
-    fused_kernel<single.value, STAGE, t1.value, learned.value, f, f>
-        <<<c->grid_rhs, dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
-            c->P, io, uio, make_work(c), c->map0[STAGE - 1], maps);
-  }, c->nev == 1, c->P.theta == 1.0, c->learned != 0, s.y == 2 && s.z == 2);
+  for (const Span& sp : c->spans)
+    with_flags([&](auto single, auto t1, auto learned, auto fixed) {
+      constexpr int f = fixed.value ? 2 : 0;
+      fused_kernel<single.value, STAGE, t1.value, learned.value, f, f>
+          <<<std::min(c->grid_rhs, sp.ntiles), dim3(s.x, s.y, s.z), rhs_smem_bytes(s.x, s.y, s.z), c->stream>>>(
+              c->P, from(io, sp.base), from(uio, sp.base), make_work(c, sp), c->map0[STAGE - 1], maps);
+    }, c->nev == 1, c->P.theta == 1.0, c->learned != 0, s.y == 2 && s.z == 2);
 }
 
 template <int STAGE>
@@ -969,6 +1022,14 @@ int select_shape(Ctx* c, int cand) {
   CK(cudaStreamSynchronize(c->stream));
   c->shape = shape;
   c->ntiles = (int)tiles.size();
+  int at = 0;
+  for (Span& sp : c->spans) {
+    long long n = 0;
+    for (int e = sp.ev0; e < sp.ev1; ++e) n += tiles_of(c->lat[e], kShapes[shape]);
+    sp.tile0 = at;
+    sp.ntiles = (int)n;
+    at += sp.ntiles;
+  }
   int rc = encode_tensor_maps(c);
   if (rc != KT_OK) return rc;
   const Shape& sh = kShapes[shape];
@@ -1135,6 +1196,10 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->pi32 = (o.pi_storage == KT_STORE_PI_FP32);
   c->nev = n_events;
   layout(n_events, grids, c->lat, c->gs, c->max_cells);
+  if (c->mixed && !make_spans(c->lat, c->gs, c->spans)) {
+    fprintf(stderr, "kt_init: an event of 2^29 or more padded cells in mixed precision\n");
+    return bail(KT_ERR_ARG);
+  }
   c->ev_set.assign(n_events, 0);
 
   Params& P = c->P;
@@ -1299,7 +1364,10 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
     kt::mlp_pack_kernel<<<1, 256, 0, c->stream>>>(c->d_mlp, c->d_mlp_packed);
     CK(cudaGetLastError());
   }
-  CK(cudaMemcpyAsync(c->d_lat, c->lat.data(), c->lat.size() * sizeof(Lattice), cudaMemcpyHostToDevice, c->stream));
+  std::vector<Lattice> dl = c->lat;  // mixed precision: from the start of each event's span
+  for (const Span& sp : c->spans)
+    for (int e = sp.ev0; e < sp.ev1; ++e) dl[e].base -= sp.base;
+  CK(cudaMemcpyAsync(c->d_lat, dl.data(), dl.size() * sizeof(Lattice), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   int rc = c->mixed ? allow_rhs_smem(c) : KT_OK;
@@ -1639,13 +1707,14 @@ int kt_get_diagnostics(kt_ctx* c, int event, double* out, int on_device) {
   const Lattice& L = c->lat[event];
   const size_t ncp = (size_t)L.nx * L.ny * L.nz;
   const int nb = (int)((ncp + 255) / 256);
-  if (c->mixed) {
-    StageIO<float> io = make_io<float>(c, 1);
-    diag_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L, io, c->tau, c->reg, c->stage);
-  } else {
-    StageIO<double> io = make_io<double>(c, 1);
-    diag_kernel<double><<<nb, 256, 0, c->stream>>>(c->P, L, io, c->tau, c->reg, c->stage);
-  }
+  Lattice L0 = L;  // the event's own fields
+  L0.base = 0;
+  if (c->mixed)
+    diag_kernel<float><<<nb, 256, 0, c->stream>>>(c->P, L0, from(make_io<float>(c, 1), L.base), c->tau, c->reg + L.base,
+                                                  c->stage);
+  else
+    diag_kernel<double><<<nb, 256, 0, c->stream>>>(c->P, L0, from(make_io<double>(c, 1), L.base), c->tau, c->reg + L.base,
+                                                   c->stage);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(out, c->stage, 7 * ncp * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                      c->stream));

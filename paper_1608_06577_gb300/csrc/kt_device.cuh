@@ -41,9 +41,12 @@ struct Lattice {
   }
 };
 
-// The index of a cell within a component: 32 bits on the mixed-precision path, whose byte offsets c * 8 fit
-// (a component of 2^29 elements would need more memory than the device has), so that an access is a
-// uniform component base plus one 32-bit offset shared by all components; 64 bits on the FP64 path.
+// The index of a cell within a component: 32 bits on the mixed-precision path, so that an access is a
+// uniform component base plus one 32-bit offset shared by all components; 64 bits on the FP64 path.  The
+// byte offset of an FP64 element, 8 c, fits below kSpanElements: an event's padded lattice is smaller
+// (kt_init refuses others), and a launch covers a run of events whose lattices together are, its field
+// pointers moved to the first of them.
+constexpr long long kSpanElements = 1LL << 29;
 template <typename R> struct IdxOf { using type = long long; };
 template <> struct IdxOf<float> { using type = unsigned; };
 template <typename R> using Idx = typename IdxOf<R>::type;
