@@ -750,8 +750,12 @@ __device__ __forceinline__ R regulator_factor(const Params& P, R gnn, R sqrt_gnn
   const R Xe = gnn * X[3][3];
   const R PP = fma(Xe, Xe, fma(R(2) * gnn, Xn, fma(R(2), Xo, Xd)));
   if (!pos(PP)) return R(1);
+  const R ee = fma(R(3) * P0, P0, e * e);
+  // a norm beyond the range is an infinite rho, which suppresses pi altogether (its product with 1/sqrt(PP)
+  // = 0 below would be a NaN, which the maxima drop); with e^2 beyond it too nothing is known, and pi stays
+  if (!finite(PP)) return finite(ee) ? R(0) : R(1);
   const R rn = rsqrt_pos(PP);  // 1/sqrt(PP)
-  R rho = PP * rn * rsqrt_pos(fma(R(3) * P0, P0, e * e)) * pr<R>(P).inv_rho_max;
+  R rho = PP * rn * rsqrt_pos(ee) * pr<R>(P).inv_rho_max;
   const R den = rn * pr<R>(P).inv_xi0_rho_max;
   const R tr = fma(-gnn, pi[3][3], pi[0][0] - pi[1][1] - pi[2][2]);
   rho = nmax(rho, fabs(tr) * den);
