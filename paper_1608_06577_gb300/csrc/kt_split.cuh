@@ -233,12 +233,9 @@ __device__ __forceinline__ unsigned thr_hi(float t) {
   const unsigned b = __float_as_uint(t);
   return (b >= 0x00800000u && b < 0x7f800000u) ? (b >> 3) + (896u << 20) : 0u;
 }
-// The update kernels are bound by the FP64 pipe (stage 2: 57 instructions per cell at 19 cycles per warp
-// and SM), and the second Newton step needs almost none of it: with |de| < 2^-19 E the new residual
-//   g(e + de) = g + de A + (e + de - E) dP,  dP = c_s^2 de,
-// in single precision is good to a few 2^-24 |de| A, i.e. 3e-13 E A, and dP's next term to 2e-13 E, both
-// inside the threshold's margin; e and P0 take one FP64 addition each.  128^3: updates 206 / 277 ->
-// 192 / 263 us (with tau's squares formed once per step), step 0.906 -> 0.868 ms.
+// (The residual after a small second step, g + de A + (e + de - E) c_s^2 de in single precision, would save
+// its FP64 evaluation, but the term it leaves out grows with (de/e)^2: where e is far below E, and on tables
+// with a steep c_s^2, it accepted roots beyond the threshold.)
 __device__ __forceinline__ unsigned rootfind_learned(const Params& P, const InvIn& v, double EPi, double e_start,
                                                      double& e, double& P0, unsigned& iters, unsigned& fallbacks) {
   const double lo = P.root_lo;
@@ -254,19 +251,8 @@ __device__ __forceinline__ unsigned rootfind_learned(const Params& P, const InvI
       return 0u;
     }
     if (kk == 2) break;
-    const float gf = d2f_trunc(r.g), de = rmul(-gf, __frcp_rn(r.gp));
-    ++iters;
-    if (kk == 1 && fabsf(de) < 0x1p-19f * v.Ef && tolf > 0.f) {
-      const float dP = r.c2 * de;
-      const double en = e + f2d_bits(de);
-      if (obits(en) >= obits(lo) && obits(en) <= obits(v.E) &&
-          fabsf(fmaf(r.emf + de, dP, fmaf(de, r.Af, gf))) < tolf * r.Af) {
-        e = en;
-        P0 = r.p0 + f2d_bits(dP);
-        return 0u;
-      }
-    }
     e = clamp_pos(newton_step(e, r), lo, v.E);
+    ++iters;
   }
   ++fallbacks;
   return rootfind_plain(P, v.E, EPi, v.M2, v.M2f, e, e, P0, iters);

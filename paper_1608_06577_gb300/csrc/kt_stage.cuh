@@ -626,7 +626,7 @@ __device__ __forceinline__ double seg_P(const RootSegM& s, double d, float df) {
 // the learned start's Newton steps use it.
 struct Resid {
   double g, A, p0;
-  float gp, Af, c2, emf;  // A f', A, c_s^2, e - E
+  float gp, Af;
 };
 template <bool MIXED>
 __device__ __forceinline__ Resid residual(const Params& P, double e, double E, double EPi, double M2, float M2f) {
@@ -638,10 +638,9 @@ __device__ __forceinline__ Resid residual(const Params& P, double e, double E, d
   r.A = EPi + r.p0;
   const double em = e - E;
   r.g = fma(em, r.A, M2);
-  r.c2 = fmaf(df, fmaf(df, s.b3, s.b2), s.b1);
-  r.emf = d2f_trunc(em);
+  const float c2 = fmaf(df, fmaf(df, s.b3, s.b2), s.b1);
   r.Af = d2f_trunc(r.A);
-  r.gp = r.Af - __fdividef(M2f * r.c2, r.Af);
+  r.gp = r.Af - __fdividef(M2f * c2, r.Af);
   return r;
 }
 
