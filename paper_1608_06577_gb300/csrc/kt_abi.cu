@@ -55,6 +55,7 @@ struct Ctx {
   Params P;
   int mixed = 0;         // 1: float u, e, p and float stencil
   size_t esz = 8;        // bytes per u/e/p element
+  int device = 0;        // the device its memory and kernels are on
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   // events
@@ -136,6 +137,19 @@ struct Range {
     cudaError_t e_ = (call);                                                                     \
     if (e_ != cudaSuccess) return fail(c, KT_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
+
+// Whether this context's kernels may read and write the caller's device array in place: memory of their own
+// device, aligned for doubles.  Anything else that a copy can reach (another device's memory without peer
+// access, an array at an odd offset) is copied.
+bool in_place(const Ctx* c, const void* p) {
+  if ((uintptr_t)p % alignof(double)) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();  // not an error of this call
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -367,7 +381,7 @@ __device__ __forceinline__ void cell_coords(const Lattice& L, unsigned o, int& i
 // bit patterns, conversions on the integer pipe, no division.  It reads the caller's device arrays
 // themselves (host arrays come through the staging area).  With the gather below, set and get of a 128^3
 // event on the device: six learned steps between them 7.13 -> 6.79 ms, six steps of a 16-event batch
-// 26.5 -> 22.7 ms; a 64 x 64 x 48 output to the host (31 fields, diagnostics) 1.1 -> 0.72 ms.
+// 26.5 -> 22.7 ms.  (An output into new host arrays is bound by the host's copies: no gain there.)
 constexpr int kSetThreads = 128;
 template <typename R>
 __global__ void __launch_bounds__(kSetThreads, 4)
@@ -465,7 +479,7 @@ __device__ __forceinline__ double f2d_exact(float f) {
 
 // Rows of one event (double or float fields) gathered into packed physical arrays: one launch for up to
 // kRows rows, kRowsPerThread of them per thread (blockIdx.y picks the group), their loads in flight
-// together; the destination is the caller's device array itself or the staging area of a host copy.
+// together; the destination is the caller's device array itself or the staging area of a copy.
 constexpr int kRows = 18, kRowsPerThread = 6;
 struct GatherRows {
   const void* src[kRows];
@@ -1311,9 +1325,9 @@ int kt_init_batch(kt_ctx** out, int n_events, const kt_grid* grids, double dx, d
   c->z_net = (float*)carve(fs * 4);
   CK(cudaMemsetAsync(c->z_net, 0, fs * 4, c->stream));  // z = 0: the conformal start (no network)
   {
-    int nb = 0, dev = 0, sms = 0;
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int nb = 0, sms = 0;
+    CK(cudaGetDevice(&c->device));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kt::mlp_start_kernel, 256, 0));
     c->grid_mlp = (int)std::max(1LL, std::min((long long)std::max(1, nb) * sms, (long long)((fs + 255) / 256)));
   }
@@ -1391,20 +1405,20 @@ int kt_set_state_event(kt_ctx* c, int event, double tau, const double* e, const 
   const Lattice& L = c->lat[event];
   size_t ncp = (size_t)L.nx * L.ny * L.nz;
   Primaries in = {e, u, pi, Pi, u_prev};
-  if (!on_device) {  // through the staging area: rows 0, 1-3, 4-13, 14, 15-17
-    double* s = c->stage;
-    auto up = [&](const double*& p, int row, int rows) {
-      if (!p) return cudaSuccess;
-      const cudaError_t r = cudaMemcpyAsync(s + row * ncp, p, rows * ncp * 8, cudaMemcpyHostToDevice, c->stream);
-      p = s + row * ncp;
-      return r;
-    };
-    CK(up(in.e, 0, 1));
-    CK(up(in.u, 1, 3));
-    CK(up(in.pi, 4, 10));
-    CK(up(in.Pi, 14, 1));
-    CK(up(in.u_prev, 15, 3));
-  }
+  // what the kernel cannot read in place goes through the staging area: rows 0, 1-3, 4-13, 14, 15-17
+  auto up = [&](const double*& p, int row, int rows) {
+    if (!p || (on_device && in_place(c, p))) return cudaSuccess;
+    double* s = c->stage + row * ncp;
+    const cudaError_t r = cudaMemcpyAsync(s, p, rows * ncp * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                                          c->stream);
+    p = s;
+    return r;
+  };
+  CK(up(in.e, 0, 1));
+  CK(up(in.u, 1, 3));
+  CK(up(in.pi, 4, 10));
+  CK(up(in.Pi, 14, 1));
+  CK(up(in.u_prev, 15, 3));
   CK(cudaMemsetAsync(c->d_stat, 0, 256, c->stream));
   const unsigned nb = (unsigned)((ncp + kSetThreads - 1) / kSetThreads);
   const double g = c->P.milne ? tau * tau : 1.0, gp = c->P.milne ? (tau - c->P.dtau) * (tau - c->P.dtau) : 1.0;
@@ -1448,27 +1462,38 @@ struct Row {
   double* dst;
   int array;
 };
-// Rows to the caller's arrays: on the device in one launch per kRows rows, to the host through the staging
-// area with one copy per caller's array (its rows adjoin).  Two arrays that happen to adjoin are copied
-// apart all the same: each may be a pinned allocation of its own, and a copy across both is refused.
+// Rows to the caller's arrays, one launch per kRows rows: straight to arrays that kernels can write in place,
+// else (host arrays among them) through the staging area with one copy per caller's array (its rows adjoin).
+// Two arrays that happen to adjoin are copied apart all the same: each may be a pinned allocation of its own,
+// and a copy across both is refused.
 int gather_rows(Ctx* c, const Lattice& L, const std::vector<Row>& rows, int on_device) {
   const size_t ncp = (size_t)L.nx * L.ny * L.nz;
+  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  int array = -1;  // the caller's array that `direct` is about
+  bool direct = false;
   for (size_t b = 0; b < rows.size(); b += kRows) {
     GatherRows g = {};
+    unsigned staged = 0;  // bit r: row r goes through the staging area
     g.n = (int)std::min<size_t>(kRows, rows.size() - b);
     for (int r = 0; r < g.n; ++r) {
-      g.src[r] = rows[b + r].f;
-      g.dst[r] = on_device ? rows[b + r].dst : c->stage + r * ncp;
-      if (rows[b + r].f32) g.f32 |= 1u << r;
+      const Row& row = rows[b + r];
+      if (row.array != array) {
+        array = row.array;
+        direct = on_device && in_place(c, row.dst);
+      }
+      if (!direct) staged |= 1u << r;
+      g.src[r] = row.f;
+      g.dst[r] = direct ? row.dst : c->stage + r * ncp;
+      if (row.f32) g.f32 |= 1u << r;
     }
     const dim3 grid((unsigned)((ncp + 255) / 256), (unsigned)((g.n + kRowsPerThread - 1) / kRowsPerThread));
     gather_kernel<<<grid, 256, 0, c->stream>>>(L, g);
     CK(cudaGetLastError());
-    if (on_device) continue;
     for (int r = 0; r < g.n;) {
       int m = 1;
       while (r + m < g.n && rows[b + r + m].array == rows[b + r].array) ++m;
-      CK(cudaMemcpyAsync(rows[b + r].dst, c->stage + r * ncp, m * ncp * 8, cudaMemcpyDeviceToHost, c->stream));
+      if ((staged >> r) & 1u)
+        CK(cudaMemcpyAsync(rows[b + r].dst, c->stage + r * ncp, m * ncp * 8, kind, c->stream));
       r += m;
     }
   }
