@@ -681,9 +681,36 @@ __device__ __forceinline__ unsigned rootfind_plain(const Params& P, double E, do
   return (it >= 100) ? ST_INVERSION : 0u;
 }
 
-// (KT_IFACE_INVERT, FP64) A = E + P0 + Pi at the root of a face state
+// (KT_IFACE_INVERT, FP64) A = E + P0 + Pi at the root of a face state.  The product form of rootfind_plain
+// takes A > 0 for granted, which E + Pi > 0 guarantees.  A face state with a bulk pressure below -E (P0 > 0
+// keeps the A of the cells around it positive) may start where A < 0: there f = e - E + M^2/A itself decides.
+__device__ __noinline__ bool face_root_signed(const Params& P, double E, double M2, double Pi, double guess, double& A) {
+  double lo = P.root_lo, hi = E;
+  double e = (guess >= lo && guess <= hi) ? guess : hi;
+  const double stop = E * 0x1p-50;
+#pragma unroll 1
+  for (int it = 0; it < 100; ++it) {
+    const RootSeg s = root_seg(P, P.seg_r, e);
+    const double d = e - s.e0;
+    const double c2 = fma(d, fma(d, 3.0 * s.a3, 2.0 * s.a2), s.a1);
+    A = E + seg_P(s, d, 0.f) + Pi;
+    const double f = e - E + M2 / A;
+    if (f == 0.0) return true;
+    if (f < 0.0) lo = e; else hi = e;
+    double en = e - f / (1.0 - M2 * c2 / (A * A));
+    if (!(en >= lo && en <= hi)) en = 0.5 * (lo + hi);
+    const double de = fabs(en - e);
+    e = en;
+    if (de <= stop) {
+      A = E + eos_P_pos(P, (e < P.e_min) ? P.e_min : e) + Pi;
+      return true;
+    }
+  }
+  return false;
+}
 __device__ __forceinline__ bool face_root_table(const Params& P, double E, double M2, double Pi, double guess,
                                                 double& A) {
+  if (!pos(E + Pi)) return face_root_signed(P, E, M2, Pi, guess, A);
   double e, P0;
   unsigned its = 0;
   if (rootfind_plain(P, E, E + Pi, M2, d2f_trunc(M2), guess, e, P0, its)) return false;
