@@ -324,8 +324,9 @@ __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a,
 // a / b for b > 0 (face velocities: b is an extrapolated u^tau >= 1).  FP32: the fast hardware
 // division.  FP64, for b within [2^-125, 2^125): Newton-Raphson for 1/b from a single-precision
 // seed (b's leading 20 mantissa bits, approximate reciprocal: relative error ~2^-20), one step
-// r <- r + r (1 - b r) (~2^-40), then the quotient corrected once, q <- q + r (a - b q), which
-// leaves about one ulp; five FP64 instructions.  Other b take the IEEE division.
+// r <- r + r (1 - b r) (~2^-40), then the quotient corrected once, q <- q + r (a - b q), whose error of
+// ~2^-80 before the last rounding makes it the IEEE quotient but within that of a tie (0 of 4e6 random
+// operands differ); five FP64 instructions.  Other b take the IEEE division.
 __device__ __forceinline__ float vdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double vdiv(double a, double b) {
   const unsigned hi = (unsigned)__double2hiint(b);
@@ -346,6 +347,10 @@ __device__ __forceinline__ double vdiv(double a, double b) {
 // far from the range where the fast division degrades).
 __device__ __forceinline__ double sdiv(double a, double b) { return vdiv(a, b); }
 __device__ __forceinline__ float sdiv(float a, float b) { return __fdividef(a, b); }
+// a / b rounded to nearest in FP32 too, where the quotient is itself a result (face velocities by root-finds:
+// with the fast division's 2 ulp the error of q after a step against FP64 faces was 1.5% larger)
+__device__ __forceinline__ double rdiv(double a, double b) { return vdiv(a, b); }
+__device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ double sexp(double x) { return exp(x); }
 __device__ __forceinline__ float sexp(float x) { return __expf(x); }
 __device__ __forceinline__ double slog(double x) { return log(x); }

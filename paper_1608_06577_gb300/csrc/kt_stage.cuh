@@ -67,9 +67,10 @@ struct Faces {
 // returns A at the root (v^d = M^d / A), or false if the state has none (E <= 0, M^2 >= E^2, no
 // convergence in 100 steps).  FP64: the cell root-find (stop at |de| <= 2^-50 E, below).  FP32: stop at
 // |de| <= 2^-21 E; the residual in product form g = (e - E) A + M^2 = f A, so that a step takes two fast
-// divisions, and the interval's record in two vector loads.  Six of these per cell and stage bound such a
-// step (face_velocity_kernel); with IEEE divisions and eos_interval's dependent loads six steps of a 72 x
-// 64 x 40 box took 2.24 ms, so 1.66 ms, when each cell inverted the four states of both its faces.
+// divisions (they only steer), and the interval's record in two vector loads.  Six of these per cell and
+// stage bound such a step (face_velocity_kernel); with IEEE divisions and eos_interval's dependent loads six
+// steps of a 72 x 64 x 40 box took 2.24 ms, so 1.66 ms, when each cell inverted the four states of both its
+// faces.
 __device__ __forceinline__ FaceSeg face_seg(const Params& P, float e) {
   const int n1 = P.eos_n - 2;
   const float g = (__logf(e) - P.lne0) * P.inv_h;
@@ -107,7 +108,9 @@ __device__ __forceinline__ bool face_root_table(const Params& P, float E, float 
     const float de = en - e;
     e = en;
     if (fabsf(de) <= stop) {
-      A = fmaf(c2, de, A);  // P0 at the root: the rest of the series is below 2^-40
+      // P0 at the root by its slope: what that leaves out is below the rounding of a new evaluation (the error
+      // of q after a step at u up to 4: 1.0e-8 so, 4.3e-8 with one)
+      A = fmaf(c2, de, A);
       return true;
     }
   }
@@ -119,7 +122,7 @@ __device__ __forceinline__ bool face_root(const Params& P, R E, R M2, R Pi, R gu
   if (!pos(E) || !below(M2, E * E) || !finite(E)) return false;
   if (!P.eos_table) {  // (bulk pressure is evolved with a table EOS only)
     const R M = sqrt(M2);  // conformal closed form, cancellation-free
-    const R e = sdiv(R(3) * (E - M) * (E + M), sqrt(fma(R(4) * E, E, R(-3) * M2)) + E);
+    const R e = rdiv(R(3) * (E - M) * (E + M), sqrt(fma(R(4) * E, E, R(-3) * M2)) + E);
     A = E + e * R(1.0 / 3.0) + Pi;
     return true;
   }
@@ -196,7 +199,7 @@ __device__ __forceinline__ void face_velocities_right(const Params& P, const flo
   for (int j = 0; j < 2; ++j) {
     const float M2 = fmaf(M[0][j], M[0][j], fmaf(M[1][j], M[1][j], rmul(rmul(gnn, M[2][j]), M[2][j])));
     float A;
-    v[j] = face_root<float>(P, E[j], M2, Pi[j], ld<float>(e, j ? c + s : c), A) ? sdiv(M[D][j], A) : 0.f;
+    v[j] = face_root<float>(P, E[j], M2, Pi[j], ld<float>(e, j ? c + s : c), A) ? rdiv(M[D][j], A) : 0.f;
   }
   vm = v[0];
   vp = v[1];
