@@ -367,6 +367,18 @@ struct Primaries {
   const double *e, *u, *pi, *Pi, *u_prev;
 };
 
+// double -> float to nearest for every double: on the integer pipe, the conversion instruction (FP64 pipe) for
+// what d2f_bits does not keep (results below the smallest normal float, NaN)
+__device__ __forceinline__ float d2f_exact(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  if ((hi & 0x7fffffffu) - (897u << 20) < (254u << 20)) return d2f_bits(d);  // 2^-126 <= |d| < 2^128
+  if (((hi << 1) | lo) == 0u) return __uint_as_float(hi);
+  return (float)d;
+}
+template <typename R> __device__ __forceinline__ R stored(double x);
+template <> __device__ __forceinline__ double stored<double>(double x) { return x; }
+template <> __device__ __forceinline__ float stored<float>(double x) { return d2f_exact(x); }
+
 // padded coordinates of physical cell o (x fastest)
 __device__ __forceinline__ void cell_coords(const Lattice& L, unsigned o, int& i, int& j, int& k) {
   const unsigned row = o / (unsigned)L.nx;
@@ -443,15 +455,15 @@ __global__ void __launch_bounds__(kSetThreads, 4)
   float qs[NQ];
   if (qf) {
 #pragma unroll
-    for (int n = 0; n < NQ; ++n) qs[n] = d2f_bits(qn[n]);
+    for (int n = 0; n < NQ; ++n) qs[n] = d2f_exact(qn[n]);
   }
   R ur[4], upr[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    ur[m] = from_f64<R>(u4[m]);
-    upr[m] = from_f64<R>(up4[m]);
+    ur[m] = stored<R>(u4[m]);
+    upr[m] = stored<R>(up4[m]);
   }
-  const R er = from_f64<R>(e), pr0 = from_f64<R>(P0);
+  const R er = stored<R>(e), pr0 = stored<R>(P0);
   for_cell_and_ghosts(P, L, L.idx(i, j, k), i, j, k, [&](long long c) {
 #pragma unroll
     for (int n = 0; n < NQ; ++n) q[n * fs + c] = qn[n];
