@@ -438,14 +438,20 @@ __global__ void __launch_bounds__(kSetThreads, 4)
   if (bad) atomicOr(status, ST_NONFINITE);
   // the inversion of Eq. (eInferred) needs E = T^{tau tau} - pi^{tau tau} > 0 and M^2 < E^2 with
   // M^i = T^{tau i} - pi^{tau i}, M^2 = M_x^2 + M_y^2 + g_{eta eta} M_eta^2 (Sec. 2.4)
-  // Decided in single precision where that is certain: E and M within 2^60 of one, M^2 < 0.99 E^2 and a
+  // Decided in single precision where that is certain: every operand below 2^60 and g above 2^-60 (in the
+  // doubles' exponents: the truncated values say nothing beyond 2^128), E above 2^-60, M^2 < 0.99 E^2 and a
   // pi^{tau mu} no larger than E, so that the difference's rounding stays far inside the margin.
+  const auto ex = [](double x) { return (unsigned)__double2hiint(x) & 0x7ff00000u; };
+  unsigned top = ex(g);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) top = max(top, ex(qn[m]));
+  const bool in_range = top < ((1023u + 60u) << 20) && ex(g) >= ((1023u - 60u) << 20);
   const float Ef = d2f_trunc(qn[0]) - d2f_trunc(qn[4]), gf = d2f_trunc(g);
   const float mx = d2f_trunc(qn[1]) - d2f_trunc(qn[5]), my = d2f_trunc(qn[2]) - d2f_trunc(qn[6]),
               mn = d2f_trunc(qn[3]) - d2f_trunc(qn[7]);
-  const bool sure = Ef > 0x1p-60f && Ef < 0x1p60f && fmaf(gf * mn, mn, fmaf(my, my, mx * mx)) < 0.99f * Ef * Ef &&
+  const bool sure = in_range && Ef > 0x1p-60f && fmaf(gf * mn, mn, fmaf(my, my, mx * mx)) < 0.99f * Ef * Ef &&
                     fabsf(d2f_trunc(qn[4])) < Ef && fabsf(d2f_trunc(qn[5])) < Ef && fabsf(d2f_trunc(qn[6])) < Ef &&
-                    gf * d2f_trunc(qn[7]) * d2f_trunc(qn[7]) < Ef * Ef && fabsf(d2f_trunc(qn[0])) < 0x1p60f;
+                    gf * d2f_trunc(qn[7]) * d2f_trunc(qn[7]) < Ef * Ef;
   if (!bad && !sure) {
     const double Ei = qn[0] - qn[4], Mx = qn[1] - qn[5], My = qn[2] - qn[6], Mn = qn[3] - qn[7];
     if (!(pos(Ei) && obits(Mx * Mx + My * My + g * Mn * Mn) < obits(Ei * Ei))) atomicOr(status, ST_INVERSION);

@@ -1,5 +1,5 @@
 """kt_set_state at the ends of the number range: values that round to FP32 numbers below the smallest normal
-one are stored as those."""
+one are stored as those, and the inversion's admissibility does not depend on the range of FP32."""
 import numpy as np
 import pytest
 
@@ -44,3 +44,25 @@ def test_subnormal_values_round_to_nearest(mode):
     s = k.get_state()
     assert np.array_equal(s["u"][1], tiny.astype(np.float32).astype(np.float64))
     assert np.array_equal(s["u"][2], -tiny.astype(np.float32).astype(np.float64))
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("tau", [1e-25, 1e-21, 1e-8, 1.0, 1e8, 1e15, 2e19, 3e20, 1e60, 1e120])
+def test_inadmissible_states_at_any_time(precision, tau):
+    """e = 100, e + P0 + Pi = -1: T^{tau tau} = 101 - u_tau^2 and |T^{tau i}| = u_tau |u|; tau u^eta = 3 is
+    admissible (91 against 9.5), tau u^eta = 9 is not (19 against 81)."""
+    from paper_1608_06577_gb300 import KT
+    from paper_1608_06577_gb300.binding import KTError
+    p = _cells(33)
+    p.e[:] = 100.0
+    p.Pi[:] = -101.0 - 100.0 / 3.0
+    k = KT(p, precision=precision)
+    for tu, ok in ((3.0, True), (9.0, False)):
+        p.u[2] = 0.0
+        p.u[2, -1] = tu / tau
+        if ok:
+            k.set_state(tau, p.e, p.u, None, p.Pi)
+        else:
+            with pytest.raises(KTError) as err:
+                k.set_state(tau, p.e, p.u, None, p.Pi)
+            assert err.value.code == -5  # KT_ERR_STATE
