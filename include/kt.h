@@ -267,8 +267,9 @@ int kt_get_state_event(kt_ctx* ctx, int event, double* tau, double* e, double* u
  * The autotuner times the candidates with v = 0 and, where v = 2 applies, v = 2 (v = 1 measured
  * slower over a whole step); kt_set_tuning selects any.  v = 1 applies to KT_MIXED with FP64 pi
  * storage, v = 2 also needs KT_IFACE_RECON; elsewhere (FP32 pi storage) the v = 0 layout runs
- * whatever v is asked for.  KT_FP64 runs one layout, one warp per block on 32 consecutive cells of an
- * event, whatever candidate is asked for, and its autotuner times nothing. */
+ * whatever v is asked for.  KT_FP64 runs one layout, blocks of 32 consecutive cells of an event (one
+ * warp, or four warps where all blocks are resident at once and the faces are reconstructed), whatever
+ * candidate is asked for, and its autotuner times nothing. */
 int kt_get_tuning(kt_ctx* ctx, int* block_xyz, int* grid_blocks, float* candidate_ms, int* n_candidates);
 /* Use candidate `candidate` (numbered as above) from now on, without autotuning; KT_ERR_ARG if it
  * is out of range.  The results do not depend on the candidate: every candidate runs the same

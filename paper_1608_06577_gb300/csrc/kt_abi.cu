@@ -101,6 +101,7 @@ struct Ctx {
   int shape = 0;
   int ntiles = 0;
   int grid_blocks = 0;    // the stage kernel's blocks (FP64), or grid_rhs
+  int team = 0;           // FP64: four warps per strip (stage_team_kernel)
   int grid_rhs = 0;       // mixed precision: right-hand-side kernel
   int grid_upd = 0;       // mixed precision: update kernel
   bool tuned = false;
@@ -740,20 +741,13 @@ UpdIO make_uio(Ctx* c, int stage) {
   return u;
 }
 
-// Two blocks of stage_team_kernel are resident per SM: beyond 304 strips a second wave doubles its time.
-// 12 viscous steps (us), one warp / four warps per strip: 64 strips 1672 / 1081, 480 strips 1692 / 2292;
-// the Gubser grid (256 strips, 20 steps) 3390 / 2255 (2046 with the sources in a warp of their own), the
-// shock tube (7 strips, 80 steps) 3503 / 2955 (2912).
-constexpr int kTeamStrips = 2 * 152;
-
 template <int STAGE>
 void launch_stage(Ctx* c, const StageIO<double>& io) {
   const bool t1 = (c->P.theta == 1.0), inv = c->P.iface_invert;
   auto go = [&](auto kernel) {
     kernel<<<c->grid_blocks, 32, 0, c->stream>>>(c->P, io, c->lat[0], c->d_lat, c->d_tiles, c->nev);
   };
-  // up to kTeamStrips strips the four-warp kernel is the faster one: see there
-  if (!inv && c->grid_blocks <= kTeamStrips) {
+  if (c->team) {
     auto team = [&](auto kernel) {
       kernel<<<c->grid_blocks, 128, 0, c->stream>>>(c->P, io, c->lat[0], c->d_lat, c->d_tiles, c->nev);
     };
@@ -1025,9 +1019,13 @@ int encode_tensor_maps(Ctx* c) {
 }
 
 // The FP64 mode has one layout (see stage_kernel): blocks of 32 consecutive cells, whatever candidate
-// is asked for.
+// is asked for.  Four warps share a strip while all blocks of stage_team_kernel are resident at once: three
+// per SM (164 registers, 22 KB), 456 strips on 152 SMs.  One strip more is a second wave.  12 viscous steps
+// (us), one warp / four warps per strip: 64 strips 1598 / 793, 304 strips 1600 / 1010, 456 strips 1623 / 1277,
+// 464 strips 1637 / 2167, 608 strips 1692 / 2437.
 int select_strips(Ctx* c, int cand) {
   c->grid_blocks = (int)strips_for(c->lat);
+  c->team = !c->P.iface_invert && c->grid_blocks <= occupancy_blocks(stage_team_kernel<double, 2, false>, Shape{32, 4, 1});
   if (c->nev > 1 && c->ntiles == 0) {
     std::vector<Tile> strips;
     for (int e = 0; e < c->nev; ++e)
@@ -1784,7 +1782,7 @@ int kt_mlp_features(kt_ctx* c, long long n, const long long* cells, float* x, fl
 int kt_get_tuning(kt_ctx* c, int* block_xyz, int* grid_blocks, float* candidate_ms, int* n_candidates) {
   if (!c) return KT_ERR_ARG;
   if (block_xyz) {
-    const Shape s = c->mixed ? kShapes[c->shape] : Shape{32, 1, 1};
+    const Shape s = c->mixed ? kShapes[c->shape] : (c->team ? Shape{32, 4, 1} : Shape{32, 1, 1});
     block_xyz[0] = s.x;
     block_xyz[1] = s.y;
     block_xyz[2] = s.z;

@@ -783,6 +783,8 @@ __device__ __forceinline__ R regulator_factor(const Params& P, R gnn, R sqrt_gnn
   // a norm beyond the range is an infinite rho, which suppresses pi altogether (its product with 1/sqrt(PP)
   // = 0 below would be a NaN, which the maxima drop); with e^2 beyond it too nothing is known, and pi stays
   if (!finite(PP)) return finite(ee) ? R(0) : R(1);
+  // (In FP32 with two hardware reciprocal roots: f is off the FP64 mode's by the same 2.3e-7 to 1.1e-6 rms as
+  // with rounded roots and quotients, PP's own rounding, which cost 1% of a step.)
   const R rn = rsqrt_pos(PP);  // 1/sqrt(PP)
   R rho = PP * rn * rsqrt_pos(ee) * pr<R>(P).inv_rho_max;
   const R den = rn * pr<R>(P).inv_xi0_rho_max;
@@ -1378,8 +1380,8 @@ __global__ void __launch_bounds__(32, 8)
 // warp 3 meanwhile computes the transport coefficients and then the sources (as long a chain as five
 // components); warp 0 adds up and runs the update.  Values pass through shared memory and are added in
 // the order of the one-warp kernel, so both give the same bits.  Gubser grid 32 x 32 x 8 (256 strips), 20
-// steps: 2.24 ms with the sources in warp 0 after the fluxes, 2.05 ms beside them (start of both: 3.39
-// ms with one warp per strip); shock tube of 7 strips, 80 steps, 3.50 ms with one warp, 2.94 ms here.
+// steps: 2.24 ms with the sources in warp 0 after the fluxes, 2.05 ms beside them (3.39 ms with one warp per
+// strip); shock tube of 7 strips, 80 steps, 3.50 ms with one warp, 2.94 ms here.
 enum : int { TM_FACE = 0, TM_DU = 18, TM_DV = 30, TM_PR = 33, TM_ACC = 39, TM_MIX = 54, TM_DIFF = 58, TM_SRC = 70,
              TM_IU0 = 85, TM_VALUES = 86 };
 
