@@ -74,15 +74,15 @@ LAUNCHES_PER_STEP = {"fp64": 2, "mixed": 4}  # (+ 1 for the network, learned sta
 # kernel ncu captures of the 96^3 learned workload, per cell times the 128^3 cells (average over
 # the two stages of each kernel; the update and fused kernels captured on 32x2x2 tiles, one block
 # per tile).  Only that mode (workload EOS) has a capture.
-MEASURED_TRAFFIC = {("learned", 128): {"rhs_kernel": 312.8e6, "update_kernel": 745.2e6, "fused_kernel": 821.8e6,
+MEASURED_TRAFFIC = {("learned", 128): {"rhs_kernel": 313.5e6, "update_kernel": 743.8e6, "fused_kernel": 822.1e6,
                                         "mlp_start_kernel": 85.4e6}}
 # Warp instructions per 32 cells of each launch slot (ncu smsp__inst_executed.sum over the warps of
 # one-kernel captures of the 96^3 learned workload, current kernels), for each kernel's fraction of
 # the SMs' issue rate: one warp instruction per scheduler and clock, 4 schedulers per SM.  The
 # kernels are bound by instruction issue and latency rather than by HBM.
-INST_PER_WARP = {"learned": {"learned_start": 291, "stage1_rhs": 2556, "stage2_rhs": 2556, "stage1_update": 1706,
-                             "stage2_update": 2005}}
-INST_PER_WARP_FUSED = {"learned": {"learned_start": 291, "stage1_rhs": 4025, "stage2_rhs": 4372}}  # fused launches
+INST_PER_WARP = {"learned": {"learned_start": 291, "stage1_rhs": 2555, "stage2_rhs": 2555, "stage1_update": 1699,
+                             "stage2_update": 1988}}
+INST_PER_WARP_FUSED = {"learned": {"learned_start": 291, "stage1_rhs": 4016, "stage2_rhs": 4362}}  # fused launches
 ISSUE_PER_SM_CLK = 4
 REPEATS = 3  # timed runs of K steps per mode; the median is reported
 

@@ -165,8 +165,8 @@ int kt_init(kt_ctx** out, const kt_grid* grid, double dx, double deta, double dt
 int kt_set_state(kt_ctx* ctx, double tau, const double* e, const double* u, const double* pi,
                  const double* Pi, const double* u_prev, int on_device);
 
-/* Advance n_steps full Heun steps (Eqs. step1-finalStep; Sec. 4.3 steps 1-9), each two fused
- * stage launches.  Asynchronous on the context's stream; it synchronises once at the end to
+/* Advance n_steps full Heun steps (Eqs. step1-finalStep; Sec. 4.3 steps 1-9), each one or two launches
+ * per stage (see kt_get_tuning).  Asynchronous on the context's stream; it synchronises once at the end to
  * read the status word.  Returns KT_ERR_INVERSION / KT_ERR_NONFINITE if any cell failed. */
 int kt_step(kt_ctx* ctx, int n_steps);
 

@@ -234,8 +234,8 @@ __device__ __forceinline__ unsigned thr_hi(float t) {
   return (b >= 0x00800000u && b < 0x7f800000u) ? (b >> 3) + (896u << 20) : 0u;
 }
 // (The residual after a small second step, g + de A + (e + de - E) c_s^2 de in single precision, would save
-// its FP64 evaluation, but the term it leaves out grows with (de/e)^2: where e is far below E, and on tables
-// with a steep c_s^2, it accepted roots beyond the threshold.)
+// its FP64 evaluation, 2.6% of a 128^3 step, but the term it leaves out grows with (de/e)^2: where e is far
+// below E, and on tables with a steep c_s^2, it accepted roots beyond the threshold.)
 __device__ __forceinline__ unsigned rootfind_learned(const Params& P, const InvIn& v, double EPi, double e_start,
                                                      double& e, double& P0, unsigned& iters, unsigned& fallbacks) {
   const double lo = P.root_lo;
